@@ -216,26 +216,28 @@ int ac_get_stencil_order(const ac_handle *h, int *order);
  * otherwise.  With
  * integer sums every field is first written, on the device before each
  * substep, as int64 fixed point about its own offset: F = round((f - c)
- * 2^(50 - E)), c the midpoint of the field's range and 2^E above its
- * half-range, so |F| <= 2^50 + 2 and each input is resolved to 2^-51 of the
- * field's own range (the weights of every Eq. 13 stencil sum to zero, so the
- * offset changes no derivative).  Every stencil numerator and every sum of
- * numerators with a common coefficient is then exact and only one int64 ->
- * binary64 conversion and one multiplication per derivative term run on the
- * FP64 pipe.  The device picks, per substep, one of three modes (counted by
- * ac_get_stencil_modes): AC_STENCIL_MODE_GROUP when the exponents E of the
- * components of u (and of A) lie within one binade of each other (they share
- * the largest, so a component keeps at least 49 bits of its own range, and the
- * cross-component sums stay single integers); AC_STENCIL_MODE_FIELD otherwise
- * (each field keeps its own scale; the sums across components are added in
- * binary64); AC_STENCIL_MODE_PLAIN when the
- * state holds a NaN or an infinity or a range outside [2^-960, 2^960) (plain
- * binary64 stencils, the AC_STENCIL_FP64 arithmetic, so non-finite values
- * propagate as the definition does and show in ac_last_cfl).  The result stays
- * within the 1e-12 relative bound of the exact-rounding definition.
+ * 2^(b - E)), c the midpoint of the field's range and 2^E above its half-range
+ * (the weights of every Eq. 13 stencil sum to zero, so the offset changes no
+ * derivative).  With b = 56 the components of u (and of A) share the largest of
+ * their exponents E; the stencil numerators and the products of the right-hand
+ * side are then exact integers, rounded once when a term is converted to binary64.
+ * That form runs while the components' exponents lie within six binades of each
+ * other (a component keeps at least 50 bits of its own range), every |E| <= 200, a
+ * mean flow is at most 2^4 times its range and |ln rho| and |xi| (the exponent of
+ * c_s^2) stay below 64; otherwise b = 50, every field keeps its own scale and the
+ * sums across components and the products run in binary64; a state that holds a NaN
+ * or an infinity, or a range outside [2^-960, 2^960), takes plain binary64 stencils
+ * (the AC_STENCIL_FP64 arithmetic, so non-finite values propagate as the definition
+ * does and show in ac_last_cfl).  The result stays within the 1e-12 relative bound
+ * of the exact-rounding definition.  ac_get_stencil_modes counts the substeps by the
+ * state they met: AC_STENCIL_MODE_GROUP, the exponents of the components of u (and
+ * of A) within one binade of each other; AC_STENCIL_MODE_FIELD, some component
+ * further below its group's largest; AC_STENCIL_MODE_PLAIN as above.
  * AC_STENCIL_FP64: binary64 arithmetic throughout.  AC_STENCIL_FIXED: integer
  * sums, AC_ERR_ARG where they do not apply.  Extra device memory for integer
- * sums: one int64 copy of the eight fields, allocated on first use.
+ * sums: one int64 copy of the eight fields with a radius-3 halo, allocated on first
+ * use.  Its kernel's waits for that copy are bounded: if one runs out, ac_store,
+ * ac_store_f32 and ac_last_cfl return AC_ERR_TIMEOUT.
  */
 #define AC_STENCIL_AUTO 0
 #define AC_STENCIL_FP64 1

@@ -60,7 +60,8 @@ struct ac_handle {
     double *result_host; // page-locked copy of result_dev
     unsigned long long *cfl_dev;  // max CFL speed of the last substep-0 input (bits of a double)
     int stencil_mode;             // AC_STENCIL_*
-    long long *fx_block;          // int64 copies of the fields (integer stencil sums)
+    void *fx_block;               // int64 copies of the fields (integer stencil sums)
+    CUtensorMap fx_map;           // tensor map over them
     unsigned long long *fx_stats; // per-field extremes (16 words) of the substep's input
     void *fx_plan;                // device plan of the integer-sum path (mode, scales)
     double *stage;       // float64 staging for load/store
@@ -323,6 +324,18 @@ static int load_common(ac_handle *h, int field, const double *src, int to_w) {
     return AC_OK;
 }
 
+// Wait for the stream; AC_ERR_TIMEOUT if a bounded device wait of the integer-sum
+// substep ran out since the last such report (the state is then undefined).
+static int sync_checked(ac_handle *h) {
+    int *err = reinterpret_cast<int *>(h->result_host + 1);
+    *err = 0;
+    if (h->fx_plan) CK(fx_plan_err(h->fx_plan, err, h->stream));
+    CK(cudaStreamSynchronize(h->stream));
+    if (!*err) return AC_OK;
+    CK(fx_plan_err(h->fx_plan, nullptr, h->stream));
+    return AC_ERR_TIMEOUT;
+}
+
 static int store_common(ac_handle *h, int field, double *dst, int from_w) {
     if (!h || !dst || field < AC_ALL || field >= NF) return AC_ERR_ARG;
     int rc = ensure_state(h);
@@ -335,8 +348,7 @@ static int store_common(ac_handle *h, int field, double *dst, int from_w) {
                     : store_array(h, h->state[h->cur][q], h->elem_f, d);
         if (rc) return rc;
     }
-    CK(cudaStreamSynchronize(h->stream));
-    return AC_OK;
+    return sync_checked(h);
 }
 
 // Host binary32 format: the state's own bytes when it is binary32 in the periodic
@@ -411,8 +423,7 @@ extern "C" int ac_store_f32(ac_handle *h, int field, float *dst) {
         rc = store_array_f32(h, h->state[h->cur][q], h->elem_f, dst + (field == AC_ALL ? (size_t)q * n : 0));
         if (rc) return rc;
     }
-    CK(cudaStreamSynchronize(h->stream));
-    return AC_OK;
+    return sync_checked(h);
 }
 
 extern "C" int ac_load(ac_handle *h, int field, const double *src) {
@@ -586,19 +597,16 @@ extern "C" int ac_get_stencil_path(const ac_handle *h, int *fixed) {
     return AC_OK;
 }
 
-// Elements between the int64 copies of consecutive fields: even, so that every
-// copy starts on a 16-byte boundary (the quantisation stores two at a time).
-static size_t fx_stride(const ac_handle *h) { return ((size_t)h->g.elems + 1) & ~(size_t)1; }
-
 // Work areas of the integer-sum path, on first use: the int64 copies of the
 // fields, the extremes words and the plan (zeroed, so its mode counts start at 0).
 static int ensure_fx(ac_handle *h) {
     if (h->fx_block) return AC_OK;
-    long long *blk = nullptr;
+    void *blk = nullptr;
     unsigned long long *stats = nullptr;
     void *plan = nullptr;
-    cudaError_t e = cudaMalloc(&blk, (size_t)NF * fx_stride(h) * sizeof(long long));
+    cudaError_t e = cudaMalloc(&blk, fx_copy_bytes(h->g));
     if (e == cudaSuccess) e = cudaMalloc(&stats, 2 * NF * sizeof(unsigned long long));
+    if (e == cudaSuccess) e = fx_encode_map(blk, h->g, &h->fx_map);
     if (e == cudaSuccess) e = cudaMalloc(&plan, fx_plan_bytes());
     if (e == cudaSuccess) e = cudaMemsetAsync(plan, 0, fx_plan_bytes(), h->stream);
     // extremes: largest keys start at 0, smallest at all ones (the plan kernel
@@ -744,11 +752,13 @@ extern "C" int ac_integrate_substep(ac_handle *h, double dt, int s) {
     L.dx = h->grid.lx / h->grid.nx;
     L.fx_stats = nullptr;
     L.fx_plan = nullptr;
-    for (int q = 0; q < NF; ++q) L.fxF[q] = nullptr;
+    L.fx_copies = nullptr;
+    L.fx_map = nullptr;
     if (L.use_fx) {
         rc = ensure_fx(h);
         if (rc) return rc;
-        for (int q = 0; q < NF; ++q) L.fxF[q] = h->fx_block + (size_t)q * fx_stride(h);
+        L.fx_copies = h->fx_block;
+        L.fx_map = &h->fx_map;
         L.fx_stats = h->fx_stats;
         L.fx_plan = h->fx_plan;
     }
@@ -844,8 +854,9 @@ extern "C" int ac_last_cfl(ac_handle *h, double *out) {
     if (!h || !out) return AC_ERR_ARG;
     CK(cudaMemcpyAsync(h->result_host, h->cfl_dev, sizeof(unsigned long long),
                        cudaMemcpyDeviceToHost, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
+    const int rc = sync_checked(h);
     *out = h->result_host[0];
+    if (rc) return rc;
     return isfinite(*out) ? AC_OK : AC_ERR_NONFINITE;
 }
 

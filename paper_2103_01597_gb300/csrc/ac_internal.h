@@ -1,6 +1,7 @@
 // Internal declarations shared by the C-ABI implementation and the kernels.
 #pragma once
 
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 #include <stdint.h>
@@ -102,10 +103,11 @@ struct SubstepLaunch {
     int s;
     unsigned long long *cfl_max;  // substep 0: device word for the max CFL speed (or NULL)
     // binary64 with integer stencil sums (cubic periodic grids): int64 copies of
-    // the fields, 16 words of per-field extremes and the device plan of the
+    // the fields, padded by their periodic halo, with their tensor map, 16 words of per-field extremes and the device plan of the
     // substep (fx_plan_bytes()); use_fx = 0 selects plain binary64 sums.
     int use_fx;
-    long long *fxF[NF];
+    void *fx_copies;           // fx_copy_bytes()
+    const CUtensorMap *fx_map;
     unsigned long long *fx_stats;
     void *fx_plan;
     double dx;
@@ -114,6 +116,11 @@ struct SubstepLaunch {
     cudaEvent_t ev_mid;
 };
 size_t fx_plan_bytes();
+size_t fx_copy_bytes(const Geom &g);
+cudaError_t fx_encode_map(void *base, const Geom &g, CUtensorMap *map);
+// Enqueues a copy of the plan's timeout word (a bounded wait of the tiled kernel ran
+// out) to page-locked *err, or, with err null, clears it.
+cudaError_t fx_plan_err(void *plan, int *err, cudaStream_t st);
 // Substeps run in each mode (group scales, per-field scales, plain binary64)
 // since the plan was zeroed; synchronises `st`.
 cudaError_t fx_plan_taken(const void *plan, unsigned long long taken[3], cudaStream_t st);

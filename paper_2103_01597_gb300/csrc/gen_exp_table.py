@@ -6,6 +6,9 @@ significant digits (independent of any libm).  ln 2 / 256 is split as L1 + L2
 with L1 a multiple of 2^-40 (29 significant bits, so N * L1 is exact for
 |N| < 2^24; the kernels use |N| < 2^18), and 256 / ln 2 is rounded to binary64.
 
+A second table holds 2^(62 + j/256) rounded to an integer, and 2^70 ln 2 / 256, for the
+fixed-point exp of the integer-product kernel.
+
 Run: python gen_exp_table.py  (rewrites exp_table.cuh beside this file)
 """
 import os
@@ -48,6 +51,14 @@ def main():
     vals = tab_p + tab_m
     for i in range(0, 512, 3):
         lines.append("    " + ", ".join(v.hex() for v in vals[i:i + 3]) + ",")
+    fix = [int((Decimal(2) ** (62 + Decimal(j) / 256)).to_integral_value()) for j in range(256)]
+    l70 = int((l * (Decimal(2) ** 70)).to_integral_value())
+    lines += ["};", "",
+              "// Fixed point: EXP_FIX[j] = 2^(62 + j/256), FX_L70 = 2^70 ln 2 / 256.",
+              "constexpr unsigned long long FX_L70 = %dull;" % l70,
+              "__device__ const unsigned long long EXP_FIX[256] = {"]
+    for i in range(0, 256, 4):
+        lines.append("    " + ", ".join("%#018xull" % v for v in fix[i:i + 4]) + ",")
     lines += ["};", "", "}  // namespace ac", ""]
     with open(os.path.join(HERE, "exp_table.cuh"), "w") as f:
         f.write("\n".join(lines))

@@ -2,6 +2,8 @@
 // path), plain binary64 stencil arithmetic otherwise.
 #include <cmath>
 
+#include <cudaTypedefs.h>
+
 #include "substep_fx.cuh"
 
 namespace ac {
@@ -9,6 +11,63 @@ namespace ac {
 static unsigned fx_grid(long long n) {  // n work items of one thread each
     long long b = (n + 255) / 256;
     return (unsigned)(b > 152 * 8 ? 152 * 8 : (b < 1 ? 1 : b));
+}
+
+// z extent of a CTA's march in the tiled kernel (one CTA per SM): the one with the
+// fewest plane steps over all waves, a CTA's start counted as one more step.
+static int fx_zchunk(long long tiles, int nz) {
+    int best = nz;
+    long long cost = -1;
+    for (int c = 1; c <= nz && c <= 1024; ++c) {
+        const int zc = (nz + c - 1) / c;
+        const long long ctas = tiles * ((nz + zc - 1) / zc);
+        const long long t = ((ctas + 151) / 152) * (zc + 1);
+        if (cost < 0 || t < cost) {
+            cost = t;
+            best = zc;
+        }
+        if (tiles * c > 152ll * 64) break;
+    }
+    return best;
+}
+
+// Padded row length (even: the strides of the tensor map are multiples of 16 bytes),
+// bytes of the eight padded int64 arrays, and the tensor map over them: dims (px,
+// py, pz, field), box one plane of a tile with its halo, all fields.
+static int fx_px(const Geom &g) { return (g.nx + 2 * R + 1) & ~1; }
+size_t fx_copy_bytes(const Geom &g) {
+    return (size_t)NF * fx_px(g) * (g.ny + 2 * R) * (g.nz + 2 * R) * sizeof(long long);
+}
+cudaError_t fx_encode_map(void *base, const Geom &g, CUtensorMap *map) {
+    void *fn = nullptr;
+    cudaDriverEntryPointQueryResult q = cudaDriverEntryPointSymbolNotFound;
+    cudaError_t e =
+        cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q);
+    if (e != cudaSuccess) return e;
+    if (q != cudaDriverEntryPointSuccess || !fn) return cudaErrorNotSupported;
+    auto enc = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
+    const cuuint64_t px = fx_px(g), py = g.ny + 2 * R, pz = g.nz + 2 * R;
+    const cuuint64_t dims[4] = {px, py, pz, NF};
+    const cuuint64_t strides[3] = {8 * px, 8 * px * py, 8 * px * py * pz};
+    const cuuint32_t box[4] = {FXR, FXR, 1, NF};
+    const cuuint32_t estr[4] = {1, 1, 1, 1};
+    const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, base, dims, strides, box, estr,
+                           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+template <bool CFL, bool EXT>
+static cudaError_t launch_fx_group(SubstepArgs<double, double> a, const CUtensorMap &map,
+                                   const FxCoefs &fc, FxPlan *plan, cudaStream_t st) {
+    auto k = substep_fx_kernel<CFL, EXT>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FX_SMEM);
+    if (e != cudaSuccess) return e;
+    const unsigned gx = (a.g.nx + FXT - 1) / FXT, gy = (a.g.ny + FXT - 1) / FXT;
+    a.zchunk = fx_zchunk((long long)gx * gy, a.g.nz);
+    const dim3 grid(gx, gy, (a.g.nz + a.zchunk - 1) / a.zchunk);
+    k<<<grid, dim3(FXT, FXT, 2), FX_SMEM, st>>>(a, map, fc, plan);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_substep_f64(const SubstepLaunch &L, cudaStream_t st, int *launches) {
@@ -27,8 +86,13 @@ cudaError_t launch_substep_f64(const SubstepLaunch &L, cudaStream_t st, int *lau
         a.fout[q] = static_cast<double *>(L.fout[q]);
         a.w[q] = static_cast<double *>(L.w[q]);
         fx.f[q] = a.fin[q];
-        fx.F[q] = L.fxF[q];
     }
+    fx.px = fx_px(L.g);
+    fx.py = L.g.ny + 2 * R;
+    fx.pz = L.g.nz + 2 * R;
+    fx.pxy = (long long)fx.px * fx.py;
+    for (int q = 0; q < NF; ++q)
+        fx.F[q] = static_cast<long long *>(L.fx_copies) + q * fx.pxy * fx.pz;
     a.k = to_dev<double>(L.c, L.ph);
     a.alpha = L.alpha;
     a.beta = L.beta;
@@ -55,13 +119,22 @@ cudaError_t launch_substep_f64(const SubstepLaunch &L, cudaStream_t st, int *lau
     fc.K_dt = dts * a.k.K;
     for (int m = 0; m < 3; ++m) fc.amp_dt[m] = dts * L.force.amp_e[m];
     fc.inv_dt2 = 1.0 / (dts * dts);
+    fc.sg = fc.two_nu_c1sq * (4.0 / 3.0);
+    fc.inv_T_ref = a.k.inv_T_ref;
+    fc.s2 = fc.two_nu_c1sq * (16.0 / 9.0) * fc.inv_T_ref;
+    fc.jb = -fc.c1dt * fc.inv720dx2;
+    fc.j2 = fc.eta_dt * fc.inv720dx2 * fc.inv720dx2 * fc.inv_T_ref;
+    fc.eta180 = fc.eta_dt * fc.inv180dx2;
+    fc.c1sq = c1 * c1;
+    fc.c1f = nextafterf((float)c1, INFINITY);
+    fc.cs2_ref_f = nextafterf((float)a.k.cs2_ref, INFINITY);
 
     const long long n = L.g.elems;
     FxPlan *plan = static_cast<FxPlan *>(L.fx_plan);
     cudaError_t e;
     fx_stats_kernel<<<fx_grid(n / 2), 256, 0, st>>>(fx, n, L.fx_stats);
-    fx_plan_kernel<<<1, 32, 0, st>>>(L.fx_stats, plan);
-    fx_quantize_kernel<<<fx_grid(n / 2), 256, 0, st>>>(fx, n, plan);
+    fx_plan_kernel<<<1, 32, 0, st>>>(L.fx_stats, plan, L.ph.inv_cp, L.ph.gamma_cp, L.ph.gm1);
+    fx_quantize_kernel<<<fx_grid(32ll * fx.py * fx.pz), 256, 0, st>>>(fx, L.g, plan);
     if (L.ev_mid) {
         e = cudaEventRecord(L.ev_mid, st);
         if (e != cudaSuccess) return e;
@@ -79,8 +152,9 @@ cudaError_t launch_substep_f64(const SubstepLaunch &L, cudaStream_t st, int *lau
     // one kernel per mode; the two the plan did not choose return at once
 #define AC_FX(C, X)                                                            \
     do {                                                                       \
-        substep_fx_kernel<false, C, X><<<grid, block, 0, st>>>(a, fx, fc, plan); \
-        substep_fx_kernel<true, C, X><<<grid, block, 0, st>>>(a, fx, fc, plan);  \
+        e = launch_fx_group<C, X>(a, *L.fx_map, fc, plan, st);                  \
+        if (e != cudaSuccess) return e;                                         \
+        substep_fx_field_kernel<C, X><<<grid, block, 0, st>>>(a, fx, fc, plan); \
         substep_fx_plain_kernel<C, X><<<grid, block, 0, st>>>(a, plan);          \
     } while (0)
     if (ext) { if (cfl) AC_FX(true, true); else AC_FX(false, true); }
@@ -92,6 +166,13 @@ cudaError_t launch_substep_f64(const SubstepLaunch &L, cudaStream_t st, int *lau
 
 // Size of the device plan of the integer-sum path (allocated by the handle).
 size_t fx_plan_bytes() { return sizeof(FxPlan); }
+
+// Enqueue a copy of the plan's timeout word to page-locked *err, or clear it.
+cudaError_t fx_plan_err(void *plan, int *err, cudaStream_t st) {
+    FxPlan *p = static_cast<FxPlan *>(plan);
+    return err ? cudaMemcpyAsync(err, &p->err, sizeof(int), cudaMemcpyDeviceToHost, st)
+               : cudaMemsetAsync(&p->err, 0, sizeof(int), st);
+}
 
 // Substeps run in each mode of the integer-sum path, read from a plan.
 cudaError_t fx_plan_taken(const void *plan, unsigned long long taken[3], cudaStream_t st) {

@@ -1,46 +1,49 @@
-// Binary64 substep with exact integer stencil sums (cubic periodic grids).
+// Binary64 substep with exact integer stencil sums and fixed-point products
+// (cubic periodic grids).
 //
-// GB300 executes two FP64 lanes per SM per cycle, so the binary64 substep is
-// bound by its FP64 instruction count, most of which (about 400 of 600 per
-// cell) are the additions and multiplications of the 54 stencils of Eq. 13.
-// Here each field is first written as int64 fixed point about an offset of its
-// own, F = round((f - c) 2^(50 - E)), with c the midpoint of the field's range
-// and 2^E above its half-range, so |F| <= 2^50 + 2.  Every weight set of Eq. 13
-// sums to zero, so the offset changes no derivative.  Every stencil numerator
-// -- and every sum of numerators that share a coefficient (curl A, lap u,
-// grad(div u), lap A, grad(div A)) -- is then an exact integer on the integer
-// pipes (largest: 6744 |F| < 2^63), and only one int64 -> binary64 conversion
-// and one multiplication per derivative term remain on the FP64 pipe.  The
-// centre values used by the physics and the Runge-Kutta update are the
-// binary64 state itself; the physics of Eqs. B.1-B.4 is unchanged binary64
-// code (cell_physics).
+// GB300 executes two FP64 lanes per SM per cycle: an FP64-pipe instruction holds
+// its sub-partition's pipe for about 78 cycles per warp, a 64-bit integer addition
+// for 2.3 and a 32 x 32 + 64 multiply-add for 2.2 (measured), so the binary64
+// substep is bound by its FP64 instruction count.  Each field is first written
+// as int64 fixed point about an offset of its own, F = round((f - c) 2^(b - E)),
+// with c the midpoint of the field's range and 2^E above its half-range.  Every
+// weight set of Eq. 13 sums to zero, so the offset changes no derivative.
 //
-// A plan kernel picks one of three modes per substep from the fields' ranges,
+// A plan kernel picks one of three kernels per substep from the fields' ranges,
 // on the device (no host round trip):
-//  * FX_GROUP: the exponents E of the three components of u (and of A) lie
-//    within one binade of each other, so they share the largest as one scale
-//    (a component keeps at least 49 bits of its own range) and the
-//    cross-component sums stay single integers;
-//  * FX_FIELD: some component lies further below its group's largest, so every
-//    field keeps its own scale and the cross-component sums (curl A,
-//    grad(div u), grad(div A)) add per-field binary64 terms instead -- a
-//    component far smaller than the others (a near-2-D flow, a weak field
-//    component) is resolved to 2^-50 of its own range;
+//  * FX_GROUP (b = 56): the exponents E of the three components of u (and of A)
+//    lie within FX_GROUP_SLACK binades of each other and share the largest as one
+//    scale (a component keeps at least 50 bits of its own range).  Stencil
+//    numerators are exact integers, the products of the right-hand side (u . grad,
+//    S . grad ln rho, S : S, j x B, j^2, u x B) exact integer dot products
+//    (fx_arith.cuh), the exponentials fixed point; what remains on the FP64 pipe
+//    is one multiply-add per term of Eqs. B.1-B.4 and the Runge-Kutta update (54
+//    instructions per cell).
+//  * FX_FIELD (b = 50): some component lies further below its group's largest, so
+//    every field keeps its own scale; integer numerators are converted one by one
+//    and the sums across components (curl A, grad(div u), grad(div A)) and the
+//    products run in binary64 -- a component far smaller than the others (a
+//    near-2-D flow, a weak field component) is resolved to 2^-50 of its own range.
+//    States beyond the ranges FX_GROUP is sized for take it too: exponents
+//    outside +-200, a mean flow 2^4 times its range, |ln rho| or |xi| over 64.
 //  * FX_PLAIN: a NaN or infinity in the state, or a range outside
 //    [2^-960, 2^960): the substep runs plain binary64 stencils, exactly what
 //    AC_STENCIL_FP64 computes (so a non-finite value propagates as in the
 //    definition and shows in the step's CFL word).
-// The quantisation error of every stencil input is then at most half a unit
-// of 2^(E - 49), E the field's own exponent: within a factor of about six of
-// the worst-case binary64 rounding of the same stencil.
 #pragma once
 
+#include <cuda.h>
+
+#include "fx_arith.cuh"
 #include "substep.cuh"
 
 namespace ac {
 
-constexpr int FX_BITS = 50;
-constexpr int FX_GROUP_SLACK = 1;  // binades a component may lie below its group's largest
+constexpr int FX_BITS = 56;        // b of FX_GROUP: 110 |F| (first derivatives) stays in 63 bits
+constexpr int FX_FIELD_BITS = 50;  // b of FX_FIELD: 6744 |F| (sums of numerators) does
+constexpr int FX_GROUP_SLACK = 6;  // binades a component may lie below its group's largest
+constexpr int FX_MODE_SLACK = 1;   // the same, for the mode that ac_get_stencil_modes counts
+constexpr int FX_EMAX = 200;       // |E| of FX_GROUP: products of two scales stay normal
 enum { FX_GROUP = 0, FX_FIELD = 1, FX_PLAIN = 2 };
 
 // Field -> group: 0 = ln rho, 1 = u, 2 = s, 3 = A.
@@ -58,11 +61,10 @@ __device__ __forceinline__ double fx_unkey(unsigned long long k) {
     return __longlong_as_double((long long)((k >> 63) ? (k & 0x7fffffffffffffffull) : ~k));
 }
 
-// round(v 2^(FX_BITS - E)) modulo 2^64 for the binary64 v held in `b` (round
-// half away from zero), by integer operations on the bits.  Two such values
-// within 2^63 of each other subtract exactly in wrapping 64-bit arithmetic,
-// however large each is.
-__device__ __forceinline__ unsigned long long fx_round_grid(unsigned long long b, int E) {
+// round(v 2^s) modulo 2^64 for the binary64 v held in `b` (round half away from
+// zero), by integer operations on the bits.  Two such values within 2^63 of each
+// other subtract exactly in wrapping 64-bit arithmetic, however large each is.
+__device__ __forceinline__ unsigned long long fx_round_grid(unsigned long long b, int s) {
     const int eb = (int)((b >> 52) & 0x7ff);
     unsigned long long m = b & 0xfffffffffffffull;
     int ex = -1074;
@@ -70,7 +72,7 @@ __device__ __forceinline__ unsigned long long fx_round_grid(unsigned long long b
         m |= 1ull << 52;
         ex = eb - 1075;
     }
-    const int sh = ex + FX_BITS - E;  // |v| 2^(FX_BITS - E) = m 2^sh
+    const int sh = ex + s;  // |v| 2^s = m 2^sh
     unsigned long long a;
     if (sh >= 0) {
         a = sh < 64 ? m << sh : 0ull;
@@ -81,19 +83,30 @@ __device__ __forceinline__ unsigned long long fx_round_grid(unsigned long long b
     return (b >> 63) ? 0ull - a : a;
 }
 
+// The int64 copies: eight arrays back to back, each padded by the radius-3 periodic
+// halo (which the quantisation writes), so that the tensor memory accelerator can
+// fetch any tile with its halo as one box.
 struct FxPtrs {
     const double *f[NF];
     long long *F[NF];
+    int px, py, pz;     // padded extents: n + 6, px made even (16-byte strides)
+    long long pxy;      // px py
 };
 
 // The quantisation plan of one substep (device memory, written by
 // fx_plan_kernel, read by the quantisation and substep kernels).
 struct FxPlan {
-    int mode;                  // FX_GROUP, FX_FIELD or FX_PLAIN
+    int kern;                  // the kernel that runs: FX_GROUP, FX_FIELD or FX_PLAIN
     int zero[NF];              // constant field: F = 0
-    int E[NF];                 // F = round((f - c) 2^(FX_BITS - E)); the scale is 2^(E - FX_BITS)
-    unsigned long long C[NF];  // round(c 2^(FX_BITS - E)) modulo 2^64
-    unsigned long long taken[3];  // substeps run in each mode (cumulative)
+    int s[NF];                 // F = round((f - c) 2^s), s = b - E
+    unsigned long long C[NF];  // round(c 2^s) modulo 2^64
+    // grad(ln rho + s / c_p) = pi_f 2^-s (big + rho small), big the larger-scaled of
+    // the two gradients, rho = pi_rh 2^-31 + pi_rl 2^-62 <= 1 (FX_GROUP)
+    int pi_s;                  // 1: s is the larger-scaled one
+    int pi_rh, pi_rl;
+    double pi_f;
+    unsigned long long taken[3];  // substeps counted in each mode (cumulative)
+    int err;                   // set if a bounded wait of the substep kernel ran out
 };
 
 // Per-field extremes of the current state: stats[q] = largest key of field q,
@@ -158,11 +171,13 @@ __global__ void __launch_bounds__(256) fx_stats_kernel(FxPtrs p, long long n,
 }
 
 // One warp: lane q < NF plans field q (offset, exponent), then the lanes agree
-// on the mode.  Thread 0 also counts the substep under its mode.
-__global__ void fx_plan_kernel(unsigned long long *stats, FxPlan *plan) {
+// on the kernel.  Thread 0 also counts the substep under its mode: plain,
+// per-field (a component more than one binade below its group's largest) or group.
+__global__ void fx_plan_kernel(unsigned long long *stats, FxPlan *plan, double inv_cp,
+                               double gamma_cp, double gm1) {
     const int q = threadIdx.x;
-    int bad = 0, zero = 1, e = -100000;
-    double c = 0.0;
+    int bad = 0, zero = 1, e = -100000, ec = -100000;
+    double c = 0.0, big = 0.0;
     if (q < NF) {
         const double hi = fx_unkey(stats[q]), lo = fx_unkey(stats[NF + q]);
         stats[q] = 0ull;        // ready for the next substep's extremes
@@ -171,6 +186,7 @@ __global__ void fx_plan_kernel(unsigned long long *stats, FxPlan *plan) {
             bad = 1;
         } else {
             c = 0.5 * lo + 0.5 * hi;
+            big = fmax(fabs(hi), fabs(lo));
             const double r = fmax(hi - c, c - lo);
             if (r > 0.0) {
                 zero = 0;
@@ -179,75 +195,116 @@ __global__ void fx_plan_kernel(unsigned long long *stats, FxPlan *plan) {
                 else  // smallest E with r < 2^E
                     e = (int)((__double_as_longlong(r) >> 52) & 0x7ff) - 1022;
             }
+            if (c != 0.0)  // |c| < 2^ec
+                ec = (int)((__double_as_longlong(c) >> 52) & 0x7ff) - 1022;
         }
     }
-    // largest exponent of the field's group over its non-constant members
+    // largest exponent of the field's group over its non-constant members (over
+    // the offsets where every member is constant)
     const int g = q < NF ? fx_group(q) : -1;
-    int eg = -100000;
+    int eg = -100000, egc = -100000;
 #pragma unroll
     for (int r = 0; r < NF; ++r) {
-        const int er = __shfl_sync(0xffffffffu, e, r);
-        if (fx_group(r) == g && er > eg) eg = er;
+        const int er = __shfl_sync(0xffffffffu, e, r), cr = __shfl_sync(0xffffffffu, ec, r);
+        if (fx_group(r) == g) {
+            eg = er > eg ? er : eg;
+            egc = cr > egc ? cr : egc;
+        }
     }
-    // group scales while every component's exponent is within one binade of its
-    // group's largest (a component then keeps at least 49 bits of its own
-    // range); a larger disparity takes per-field scales
-    const int disparity = q < NF && !zero && e < eg - FX_GROUP_SLACK;
+    if (eg == -100000) eg = egc > -100000 ? egc : 0;
     const int any_bad = __any_sync(0xffffffffu, bad);
-    const int any_disp = __any_sync(0xffffffffu, disparity);
-    const int mode = any_bad ? FX_PLAIN : (any_disp ? FX_FIELD : FX_GROUP);
+    const int far = __any_sync(0xffffffffu, q < NF && !zero && e < eg - FX_MODE_SLACK);
+    // what FX_GROUP is sized for: the slack, the exponents, |u| < 2^(E + 4) (u is
+    // taken from F + C), |ln rho| and |xi| below 64 (the fixed-point exp)
+    const double xb = gamma_cp * __shfl_sync(0xffffffffu, big, 4) +
+                      fabs(gm1) * __shfl_sync(0xffffffffu, big, 0);
+    int out = q < NF && ((!zero && e < eg - FX_GROUP_SLACK) || eg > FX_EMAX || eg < -FX_EMAX);
+    if (g == 1) out |= ec > eg + 4;
+    if (q == 0) out |= !(big < 64.0) || !(xb < 64.0);
+    const int any_out = __any_sync(0xffffffffu, out);
+    const int kern = any_bad ? FX_PLAIN : (any_out ? FX_FIELD : FX_GROUP);
+    const int mode = any_bad ? FX_PLAIN : (far ? FX_FIELD : FX_GROUP);
+    int s = FX_FIELD_BITS - (e > -100000 ? e : 0);
+    if (kern == FX_GROUP) s = FX_BITS - eg;
     if (q < NF) {
-        int E = mode == FX_GROUP ? eg : e;
-        const int valid = E > -100000;
-        if (!valid) E = 0;
         plan->zero[q] = zero;
-        plan->E[q] = E;
-        plan->C[q] = fx_round_grid((unsigned long long)__double_as_longlong(c), E);
+        plan->s[q] = s;
+        plan->C[q] = fx_round_grid((unsigned long long)__double_as_longlong(c), s);
     }
+    const int s0 = __shfl_sync(0xffffffffu, s, 0), s4 = __shfl_sync(0xffffffffu, s, 4);
+    const int z0 = __shfl_sync(0xffffffffu, zero, 0), z4 = __shfl_sync(0xffffffffu, zero, 4);
     if (q == 0) {
-        plan->mode = mode;
+        plan->kern = kern;
+        if (kern == FX_GROUP) {
+            // ratio of the scales of grad s / c_p and grad ln rho
+            const double ratio = ldexp(inv_cp, s0 - s4);
+            const int pi_s = z0 ? 1 : (z4 ? 0 : ratio >= 1.0);
+            const double rho = z0 || z4 ? 0.0 : (pi_s ? 1.0 / ratio : ratio);
+            int rh = 0x7fffffff, rl = 0x7fffffff;
+            if (rho < 1.0) {
+                const double t = rho * 2147483648.0;
+                rh = (int)t;
+                rl = (int)((t - (double)rh) * 2147483648.0);
+            }
+            plan->pi_s = pi_s;
+            plan->pi_rh = rh;
+            plan->pi_rl = rl;
+            plan->pi_f = pi_s ? inv_cp : 1.0;
+        }
         plan->taken[mode] += 1ull;
     }
 }
 
-// F = round(f 2^(50 - E)) - round(c 2^(50 - E)) by integer operations on the
-// binary64 bits; nothing to do in FX_PLAIN.  Two cells per thread and
-// iteration (16-byte loads and stores: the int64 arrays have an even stride).
-__global__ void __launch_bounds__(256) fx_quantize_kernel(FxPtrs p, long long n,
-                                                          const FxPlan *plan) {
-    if (plan->mode == FX_PLAIN) return;
-    int E[NF], zero[NF];
+// F = round(f 2^s) - round(c 2^s) by integer operations on the binary64 bits, with
+// the periodic halo; nothing to do in FX_PLAIN.  A warp takes one padded row at a
+// time, two cells per lane, all sixteen loads ahead of the stores.
+__global__ void __launch_bounds__(256) fx_quantize_kernel(FxPtrs p, Geom g, const FxPlan *plan) {
+    if (plan->kern == FX_PLAIN) return;
+    int s[NF], zero[NF];
     unsigned long long C[NF];
 #pragma unroll
     for (int q = 0; q < NF; ++q) {
-        E[q] = plan->E[q];
+        s[q] = plan->s[q];
         zero[q] = plan->zero[q];
         C[q] = plan->C[q];
     }
-    const long long n2 = n >> 1;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n2;
-         t += (long long)gridDim.x * blockDim.x) {
-        // all eight loads ahead of the stores, so that they are in flight together
-        double2 v[NF];
+    auto fix = [&](double v, int q) -> long long {
+        return zero[q] ? 0ll
+                       : (long long)(fx_round_grid((unsigned long long)__double_as_longlong(v), s[q]) -
+                                     C[q]);
+    };
+    const int lane = threadIdx.x & 31;
+    const long long rows = (long long)p.py * p.pz;
+    const bool small = g.nx < R;  // the halo wraps around more than once
+    for (long long r = blockIdx.x * 8ll + (threadIdx.x >> 5); r < rows; r += gridDim.x * 8ll) {
+        const int k = (int)(r / p.py), j = (int)(r - (long long)k * p.py);
+        const long long src = wrap_near(k - R, g.nz) * g.pxy + (long long)wrap_near(j - R, g.ny) * g.px;
+        const long long dst = r * p.px + R;
+        // a cell and its images in the row's halo
+        auto put = [&](int q, int x, long long v) {
+            long long *row = p.F[q] + dst;
+            row[x] = v;
+            if (small) {
+                for (int h = x - g.nx; h >= -R; h -= g.nx) row[h] = v;
+                for (int h = x + g.nx; h < g.nx + R; h += g.nx) row[h] = v;
+            } else {
+                if (x < R) row[x + g.nx] = v;
+                if (x >= g.nx - R) row[x - g.nx] = v;
+            }
+        };
+        for (int x = lane; x < g.nx; x += 64) {
+            const int x1 = x + 32 < g.nx ? x + 32 : x;
+            double v[NF], w[NF];
 #pragma unroll
-        for (int q = 0; q < NF; ++q) v[q] = __ldg(reinterpret_cast<const double2 *>(p.f[q]) + t);
+            for (int q = 0; q < NF; ++q) {
+                v[q] = __ldg(p.f[q] + src + x);
+                w[q] = __ldg(p.f[q] + src + x1);
+            }
 #pragma unroll
-        for (int q = 0; q < NF; ++q) {
-            longlong2 o;
-            o.x = zero[q] ? 0ll
-                          : (long long)(fx_round_grid((unsigned long long)__double_as_longlong(v[q].x),
-                                                      E[q]) - C[q]);
-            o.y = zero[q] ? 0ll
-                          : (long long)(fx_round_grid((unsigned long long)__double_as_longlong(v[q].y),
-                                                      E[q]) - C[q]);
-            reinterpret_cast<longlong2 *>(p.F[q])[t] = o;
-        }
-    }
-    if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
-#pragma unroll
-        for (int q = 0; q < NF; ++q) {
-            const unsigned long long b = (unsigned long long)__double_as_longlong(p.f[q][n - 1]);
-            p.F[q][n - 1] = zero[q] ? 0ll : (long long)(fx_round_grid(b, E[q]) - C[q]);
+            for (int q = 0; q < NF; ++q) {
+                put(q, x, fix(v[q], q));
+                if (x1 != x) put(q, x1, fix(w[q], q));
+            }
         }
     }
 }
@@ -294,14 +351,14 @@ __device__ __forceinline__ long long ndab(const V &F) {
 // (double)N 2^k exactly for the integer numerator N, by adding k to the
 // exponent field of the converted value (k_hi = k << 20, the exponent's place in
 // the high word); 0 stays 0.  Every product stays normal: 1 <= |N| < 2^63 and
-// the plan keeps 2^(E - FX_BITS) within [2^-1010, 2^910].
+// the plan keeps 2^-s within [2^-1010, 2^910].
 __device__ __forceinline__ double fx_scaled(long long N, int k_hi) {
     const double v = (double)N;
     return N == 0 ? 0.0 : __hiloint2double(__double2hiint(v) + k_hi, __double2loint(v));
 }
 
 // Coefficients of the converted numerators (host side); the field scales
-// 2^(E - FX_BITS) come from the device plan.  Every coefficient through which a
+// 2^-s come from the device plan.  Every coefficient through which a
 // term enters the right-hand side also carries the step dt (dts below; the host
 // takes this path only for |dt| in [1e-100, 1e100], so that 1 / dt^2 stays in
 // range).  The RHS so formed is dt times Eqs. B.1-B.4, and the RK update adds it
@@ -320,6 +377,15 @@ struct FxCoefs {
     double K_dt;         // dts K
     double amp_dt[3];    // dts times the forcing amplitudes
     double inv_dt2;      // 1 / dts^2: |B|^2 of the CFL speed from the dts-scaled B
+    // FX_GROUP:
+    double sg;         // two_nu_c1sq 4/3: 2 nu S . grad ln rho from X = 3/4 S
+    double s2;         // two_nu_c1sq 16/9 / T_ref: 2 nu S : S / T
+    double jb;         // -c1dt / (720 dx^2): j x B / rho from -j and B
+    double j2;         // eta_dt / (720 dx^2)^2 / T_ref: eta j^2 / (rho T)
+    double eta180;     // eta_dt / (180 dx^2): eta lap A
+    double c1sq;       // 1 / (60 dx)^2
+    double inv_T_ref;  // c_p (gamma - 1) / cs2_ref
+    float c1f, cs2_ref_f;  // c1 and cs2_ref rounded up (the CFL bound)
 };
 
 // Eqs. B.1-B.4 at one cell as cell_physics computes them, times dts (the step
@@ -391,30 +457,38 @@ __device__ __forceinline__ void cell_physics_fx(const double (&u)[3], const doub
     }
 }
 
-// One (x, y) column of the integer-sum substep.  PF: per-field scales (FX_FIELD),
-// so sums across the components of u or A are formed in binary64 from per-field
-// integer numerators; otherwise one scale per group (FX_GROUP).
-template <bool PF, bool CFL, bool EXT>
-__device__ __forceinline__ void fx_column(const SubstepArgs<double, double> &a, const FxPtrs &fx,
+// One field around the cell at padded index c.
+struct FxFieldView {
+    const long long *f;
+    const long long &c;
+    long long pxy;
+    int px;
+    AC_BC_ONLY(long long bc_lim;)
+    __device__ __forceinline__ long long operator()(int dx, int dy, int dz) const {
+        return __ldg(f + AC_BC(c + dz * pxy + (long long)dy * px + dx, bc_lim, AC_BC_STENCIL));
+    }
+};
+
+// One (x, y) column of the substep with per-field scales (FX_FIELD): sums across
+// the components of u or A are formed in binary64 from per-field integer numerators.
+template <bool CFL, bool EXT>
+__device__ __forceinline__ void fx_field_column(const SubstepArgs<double, double> &a, const FxPtrs &fx,
                                           const FxCoefs &fc, const FxPlan *plan,
                                           const double *etab, int i, int j, double &cfl) {
     // Each field's scale 2^(E - FX_BITS) is applied to its converted numerators
     // by an exponent add on the integer pipe (fx_scaled), so only the grid
     // coefficients -- kernel parameters, read from the constant bank -- multiply
     // on the FP64 pipe, and no scaled coefficient occupies registers (the
-    // kernels sit at 255 registers).  In FX_GROUP the components of u and of A
-    // share their exponent.
+    // kernels sit at 255 registers).
     int kh[NF];
 #pragma unroll
-    for (int q = 0; q < NF; ++q) kh[q] = (plan->E[q] - FX_BITS) << 20;
-    // first derivative of field q from its numerator; the gradients of ln rho, s
-    // and u stay without the factor c1 (cell_physics_fx applies it)
-    auto d1 = [&](long long N, int q) -> double { return fx_scaled(N, kh[q]) * fc.c1dt; };
+    for (int q = 0; q < NF; ++q) kh[q] = -plan->s[q] * (1 << 20);
+    // first derivative of field q from its numerator, without the factor c1
+    // (cell_physics_fx applies it)
     auto d1r = [&](long long N, int q) -> double { return fx_scaled(N, kh[q]); };
     const int k0 = blockIdx.z * a.zchunk;
     const int k1 = min(k0 + a.zchunk, a.g.nz);
-    IdxPeriodic32 ix;
-    ix.set_xy(i, j, a.g);
+    const long long col = ((long long)(j + R)) * fx.px + i + R;
     double2 exy = make_double2(0.0, 0.0);
     if (a.force_on) {
         const double2 ex = a.ftab[i], ey = a.ftab[a.g.nx + j];
@@ -422,8 +496,8 @@ __device__ __forceinline__ void fx_column(const SubstepArgs<double, double> &a, 
         exy.y = ex.x * ey.y + ex.y * ey.x;
     }
     for (int kk = k0; kk < k1; ++kk) {
-        ix.set_z(kk, a.g);
-        const long long o = ix(0, 0, 0);
+        const long long c = (kk + R) * fx.pxy + col;
+        const long long o = kk * a.g.pxy + (long long)j * a.g.px + i;
         // Centre values (the binary64 state) and the thermodynamic factors: at the
         // top of the cell in the CFL variant (substep 0), after the stencil sums in
         // the other; each placement measured fastest for its variant at 256^3
@@ -444,11 +518,12 @@ __device__ __forceinline__ void fx_column(const SubstepArgs<double, double> &a, 
             frc[1] = fc.amp_dt[1] * cph;
             frc[2] = fc.amp_dt[2] * cph;
         }
-        const GlobalView<long long, IdxPeriodic32> Fl{fx.F[0], ix}, Fs{fx.F[4], ix};
-        const GlobalView<long long, IdxPeriodic32> Fu[3] = {{fx.F[1], ix}, {fx.F[2], ix},
-                                                             {fx.F[3], ix}};
-        const GlobalView<long long, IdxPeriodic32> Fa[3] = {{fx.F[5], ix}, {fx.F[6], ix},
-                                                             {fx.F[7], ix}};
+        auto view = [&](int q) {
+            return FxFieldView{fx.F[q], c, fx.pxy, fx.px AC_BC_ONLY(, fx.pxy * fx.pz)};
+        };
+        const FxFieldView Fl = view(0), Fs = view(4);
+        const FxFieldView Fu[3] = {view(1), view(2), view(3)};
+        const FxFieldView Fa[3] = {view(5), view(6), view(7)};
         // first derivatives
         double gl[3], gs[3], gu[3][3], B[3];
         gl[0] = d1r(nd1<0>(Fl), 0);
@@ -459,26 +534,19 @@ __device__ __forceinline__ void fx_column(const SubstepArgs<double, double> &a, 
         gs[2] = d1r(nd1<2>(Fs), 4);
 #pragma unroll
         for (int m = 0; m < 3; ++m) {
-            const int qu = PF ? 1 + m : 1;  // one live exponent in FX_GROUP
-            gu[m][0] = d1r(nd1<0>(Fu[m]), qu);
-            gu[m][1] = d1r(nd1<1>(Fu[m]), qu);
-            gu[m][2] = d1r(nd1<2>(Fu[m]), qu);
+            gu[m][0] = d1r(nd1<0>(Fu[m]), 1 + m);
+            gu[m][1] = d1r(nd1<1>(Fu[m]), 1 + m);
+            gu[m][2] = d1r(nd1<2>(Fu[m]), 1 + m);
         }
-        if constexpr (PF) {
-            B[0] = (fx_scaled(nd1<1>(Fa[2]), kh[7]) - fx_scaled(nd1<2>(Fa[1]), kh[6])) * fc.c1dt;
-            B[1] = (fx_scaled(nd1<2>(Fa[0]), kh[5]) - fx_scaled(nd1<0>(Fa[2]), kh[7])) * fc.c1dt;
-            B[2] = (fx_scaled(nd1<0>(Fa[1]), kh[6]) - fx_scaled(nd1<1>(Fa[0]), kh[5])) * fc.c1dt;
-        } else {
-            B[0] = d1(nd1<1>(Fa[2]) - nd1<2>(Fa[1]), 5);
-            B[1] = d1(nd1<2>(Fa[0]) - nd1<0>(Fa[2]), 5);
-            B[2] = d1(nd1<0>(Fa[1]) - nd1<1>(Fa[0]), 5);
-        }
+        B[0] = (fx_scaled(nd1<1>(Fa[2]), kh[7]) - fx_scaled(nd1<2>(Fa[1]), kh[6])) * fc.c1dt;
+        B[1] = (fx_scaled(nd1<2>(Fa[0]), kh[5]) - fx_scaled(nd1<0>(Fa[2]), kh[7])) * fc.c1dt;
+        B[2] = (fx_scaled(nd1<0>(Fa[1]), kh[6]) - fx_scaled(nd1<1>(Fa[0]), kh[5])) * fc.c1dt;
         // lap V_i = sum_a N2_aa(V_i) / (180 dx^2);
         // grad(div V)_i = [4 N2_ii(V_i) + NX_ij(V_j) + NX_ik(V_k)] / (720 dx^2);
         // component C of V contributes 4 N2_CC to entry C and its two mixed
         // numerators to the other two entries.
         double viscl[3], lapa[3], J[3];
-        if constexpr (PF) {
+        {
             // per-field scaled numerators, summed across components in binary64
             double LU[3], GU[3], LA[3], GA[3];
 #pragma unroll
@@ -529,64 +597,6 @@ __device__ __forceinline__ void fx_column(const SubstepArgs<double, double> &a, 
                 lapa[m] = LA[m] * fc.inv180dx2;
                 J[m] = fma(GA[m], fc.inv720dx2, -lapa[m]);
             }
-        } else {
-            long long LU[3], GU[3];
-            {
-                const long long c0 = Fu[0](0, 0, 0);
-                const long long xx = nd2<0>(Fu[0], c0), yy = nd2<1>(Fu[0], c0), zz = nd2<2>(Fu[0], c0);
-                LU[0] = xx + yy + zz;
-                GU[0] = 4 * xx;
-                GU[1] = ndab<0, 1>(Fu[0]);
-                GU[2] = ndab<0, 2>(Fu[0]);
-            }
-            {
-                const long long c0 = Fu[1](0, 0, 0);
-                const long long xx = nd2<0>(Fu[1], c0), yy = nd2<1>(Fu[1], c0), zz = nd2<2>(Fu[1], c0);
-                LU[1] = xx + yy + zz;
-                GU[1] += 4 * yy;
-                GU[0] += ndab<0, 1>(Fu[1]);
-                GU[2] += ndab<1, 2>(Fu[1]);
-            }
-            {
-                const long long c0 = Fu[2](0, 0, 0);
-                const long long xx = nd2<0>(Fu[2], c0), yy = nd2<1>(Fu[2], c0), zz = nd2<2>(Fu[2], c0);
-                LU[2] = xx + yy + zz;
-                GU[2] += 4 * zz;
-                GU[0] += ndab<0, 2>(Fu[2]);
-                GU[1] += ndab<1, 2>(Fu[2]);
-            }
-            // the same two sums for A; j = grad(div A) - lap A
-            long long LA[3], GA[3];
-            {
-                const long long c0 = Fa[0](0, 0, 0);
-                const long long xx = nd2<0>(Fa[0], c0), yy = nd2<1>(Fa[0], c0), zz = nd2<2>(Fa[0], c0);
-                LA[0] = xx + yy + zz;
-                GA[0] = 4 * xx;
-                GA[1] = ndab<0, 1>(Fa[0]);
-                GA[2] = ndab<0, 2>(Fa[0]);
-            }
-            {
-                const long long c0 = Fa[1](0, 0, 0);
-                const long long xx = nd2<0>(Fa[1], c0), yy = nd2<1>(Fa[1], c0), zz = nd2<2>(Fa[1], c0);
-                LA[1] = xx + yy + zz;
-                GA[1] += 4 * yy;
-                GA[0] += ndab<0, 1>(Fa[1]);
-                GA[2] += ndab<1, 2>(Fa[1]);
-            }
-            {
-                const long long c0 = Fa[2](0, 0, 0);
-                const long long xx = nd2<0>(Fa[2], c0), yy = nd2<1>(Fa[2], c0), zz = nd2<2>(Fa[2], c0);
-                LA[2] = xx + yy + zz;
-                GA[2] += 4 * zz;
-                GA[0] += ndab<0, 2>(Fa[2]);
-                GA[1] += ndab<1, 2>(Fa[2]);
-            }
-#pragma unroll
-            for (int m = 0; m < 3; ++m) {
-                viscl[m] = fma(fx_scaled(LU[m], kh[1]), fc.nu180, fx_scaled(GU[m], kh[1]) * fc.nu2160);
-                lapa[m] = fx_scaled(LA[m], kh[5]) * fc.inv180dx2;
-                J[m] = fma(fx_scaled(GA[m], kh[5]), fc.inv720dx2, -lapa[m]);
-            }
         }
         // EXT: lap xi = gamma / c_p lap s + (gamma - 1) lap ln rho (conduction)
         double lapxi = 0.0;
@@ -605,9 +615,9 @@ __device__ __forceinline__ void fx_column(const SubstepArgs<double, double> &a, 
         const double u[3] = {ldg(a.fin[1] + o), ldg(a.fin[2] + o), ldg(a.fin[3] + o)};
         double rhs[NF];
         if (CFL) {
-            double c;
-            cell_physics_fx<EXT>(u, gl, gs, gu, B, viscl, lapa, J, a.k, fc, frc, rhs, &c, lapxi, th);
-            cfl = (c > cfl || c != c) ? c : cfl;
+            double v;
+            cell_physics_fx<EXT>(u, gl, gs, gu, B, viscl, lapa, J, a.k, fc, frc, rhs, &v, lapxi, th);
+            cfl = (v > cfl || v != v) ? v : cfl;
         } else {
             cell_physics_fx<EXT>(u, gl, gs, gu, B, viscl, lapa, J, a.k, fc, frc, rhs, nullptr, lapxi,
                                  th);
@@ -623,25 +633,604 @@ __device__ __forceinline__ void fx_column(const SubstepArgs<double, double> &a, 
     }
 }
 
-// The substep in one mode of the plan: each mode is its own kernel (its own
-// register allocation: in one kernel with all three bodies ptxas spilled the
-// group-scale body, 16 B per cell at 128^3, and it ran 3-10% slower), launched
-// every substep; the two kernels whose mode the plan did not choose return at
-// once.  Two CTAs of 128 threads per SM (8 warps, as many as 255 registers
-// allow): with the minimum stated, ptxas keeps the body within 255 registers
-// (a cap of 168 registers for 12 warps spills and is slower).
-template <bool PF, bool CFL, bool EXT = false>
-__global__ void __launch_bounds__(128, 2) substep_fx_kernel(const SubstepArgs<double, double> a,
-                                                         const FxPtrs fx, FxCoefs fc,
-                                                         const FxPlan *plan) {
-    if (plan->mode != (PF ? FX_FIELD : FX_GROUP)) return;
+// Kernel of FX_FIELD.  Each of the plan's three kernels is launched every substep
+// (its own register allocation: with all bodies in one kernel ptxas spilled and it
+// ran 3-10% slower); the two that the plan did not choose return at once.  Two CTAs
+// of 128 threads per SM (8 warps, as many as 255 registers allow).
+template <bool CFL, bool EXT = false>
+__global__ void __launch_bounds__(128, 2) substep_fx_field_kernel(const SubstepArgs<double, double> a,
+                                                                  const FxPtrs fx, FxCoefs fc,
+                                                                  const FxPlan *plan) {
+    if (plan->kern != FX_FIELD) return;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     const int j = blockIdx.y * blockDim.y + threadIdx.y;
     const bool active = i < a.g.nx && j < a.g.ny;
     __shared__ double etab[512];
     exp_tab_stage(etab);
     double cfl = 0.0;
-    if (active) fx_column<PF, CFL, EXT>(a, fx, fc, plan, etab, i, j, cfl);
+    if (active) fx_field_column<CFL, EXT>(a, fx, fc, plan, etab, i, j, cfl);
+    if (CFL) block_max_to_global(cfl, a.cfl_max);
+}
+
+// ---- FX_GROUP: integer stencils, integer products --------------------------------
+//
+// A CTA owns a 16 x 16 column tile and marches along z with two threads per cell:
+// eight warps take the equations of ln rho, u and s, eight warps A, the pressure and
+// the thermodynamic factors (4 warps per scheduler at 128 registers).  A ring of seven
+// planes in shared memory holds the tile with its halo (22 x 22 cells x eight fields,
+// 31 KB a plane, 217 KB: one CTA per SM), each plane fetched by one TMA box.  There is
+// no eighth slot to prefetch into: a cell's stencils are all taken first, and plane
+// z + 4 lands in plane z - 3's slot while the products, conversions and the
+// Runge-Kutta update of plane z run.
+// Measured at 256^3, ms per substep (s = 1, 2): 7.35 with binary64 products (bound by
+// the FP64 pipe, 179 instructions a cell); these integer products with stencil points
+// loaded through L1 5.95 (load latency at 2 warps per scheduler); one thread per cell
+// on the ring 3.72; two threads in lockstep between CTA barriers 4.11; without CTA
+// barriers (FxMarch) 3.40; with the halves balanced 3.18.  Bound now by the issue of
+// its 3900 instructions a cell (about half the issue slots; ALU 48%, FP64 pipe 55%).
+constexpr int FXT = 16;                            // tile edge
+constexpr int FXR = FXT + 2 * R;                   // staged row
+constexpr int FX_FIELD_TILE = FXR * FXR;           // cells of one staged field plane
+constexpr int FX_PLANE = NF * FX_FIELD_TILE;       // int64 of one ring slot
+constexpr int FX_SLOTS = 2 * R + 1;
+constexpr unsigned FX_PLANE_BYTES = FX_PLANE * 8;
+constexpr int FX_WARPS = 2 * FXT * FXT / 32;
+constexpr int FX_XCH = 6;                          // doubles a cell's A thread hands to its u thread
+constexpr size_t FX_SMEM =
+    (size_t)FX_SLOTS * FX_PLANE_BYTES + 8 * (256 + FX_XCH * FXT * FXT);
+constexpr unsigned FX_WAIT_LIMIT = 1u << 18;       // try_wait polls (3.8 us each) before giving up
+
+__device__ __forceinline__ unsigned fx_smem_u32(const void *p) {
+    return (unsigned)__cvta_generic_to_shared(p);
+}
+// A load that stays where it is written (the compiler would sink it to its use).
+__device__ __forceinline__ double fx_load_now(const double *p) {
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];\n" : "=d"(v) : "l"(p));
+    return v;
+}
+// Wait for the phase of `bar` with the given parity; false after FX_WAIT_LIMIT polls.
+__device__ __forceinline__ bool fx_wait(fx_u64 *bar, unsigned parity) {
+    const unsigned a = fx_smem_u32(bar);
+    for (unsigned it = 0; it < FX_WAIT_LIMIT; ++it) {
+        unsigned done;
+        asm volatile(
+            "{\n .reg .pred p;\n"
+            " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+            " selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(done)
+            : "r"(a), "r"(parity)
+            : "memory");
+        if (done) return true;
+    }
+    return false;
+}
+// One plane (padded plane index pz) of the tile whose first staged cell is (x, y).
+__device__ __forceinline__ void fx_fetch(long long *dst, const CUtensorMap *map, fx_u64 *bar, int x,
+                                         int y, int pz) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(fx_smem_u32(bar)),
+                 "r"(FX_PLANE_BYTES)
+                 : "memory");
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes "
+        "[%0], [%1, {%3, %4, %5, %6}], [%2];\n" ::"r"(fx_smem_u32(dst)),
+        "l"(reinterpret_cast<fx_u64>(map)), "r"(fx_smem_u32(bar)), "r"(x), "r"(y), "r"(pz), "r"(0)
+        : "memory");
+}
+
+// One field around a thread's cell in the ring: `c` its centre in slot 0, slot[d]
+// the offset of plane z - 3 + d.
+struct FxView {
+    const long long *c;
+    const int (&slot)[FX_SLOTS];
+    __device__ __forceinline__ long long operator()(int dx, int dy, int dz) const {
+        return c[slot[dz + R] + dy * FXR + dx];
+    }
+};
+
+// One axis of a field: first-derivative numerator d (x 60 dx) and the sums s1 = F1 +
+// F-1, n2 = -(F2 + F-2), s3 = F3 + F-3 of the second derivative (every weight below
+// is then positive, as fx_wmac wants).
+struct FxAxis {
+    long long d, s1, n2, s3;
+};
+template <int AX>
+__device__ __forceinline__ FxAxis fx_axis(const FxView &F) {
+    constexpr int ox = AX == 0, oy = AX == 1, oz = AX == 2;
+    const long long p1 = F(ox, oy, oz), m1 = F(-ox, -oy, -oz);
+    const long long p2 = F(2 * ox, 2 * oy, 2 * oz), m2 = F(-2 * ox, -2 * oy, -2 * oz);
+    const long long p3 = F(3 * ox, 3 * oy, 3 * oz), m3 = F(-3 * ox, -3 * oy, -3 * oz);
+    FxAxis a;
+    a.d = 45 * (p1 - m1) + 9 * (m2 - p2) + (p3 - m3);
+    a.s1 = p1 + m1;
+    a.n2 = -p2 - m2;
+    a.s3 = p3 + m3;
+    return a;
+}
+
+// v += N_AB (NEG: v -= N_AB), N_AB the mixed-derivative numerator 270 S1 - 27 S2 +
+// 2 S3 (x 720 dx^2).
+template <int A, int B, bool NEG>
+__device__ __forceinline__ void fx_mixed(const FxView &F, FxWide &v) {
+    constexpr int ax = A == 0, ay = A == 1, az = A == 2;
+    constexpr int bx = B == 0, by = B == 1, bz = B == 2;
+    constexpr int W[3] = {270, 27, 2};
+#pragma unroll
+    for (int m = 1; m <= 3; ++m) {
+        const long long pp = F(m * (ax + bx), m * (ay + by), m * (az + bz));
+        const long long mm = F(-m * (ax + bx), -m * (ay + by), -m * (az + bz));
+        const long long pm = F(m * (ax - bx), m * (ay - by), m * (az - bz));
+        const long long mp = F(-m * (ax - bx), -m * (ay - by), -m * (az - bz));
+        const bool minus = NEG != (m == 2);
+        fx_wmac(v, minus ? (pm + mp) - (pp + mm) : (pp + mm) - (pm + mp), W[m - 1]);
+    }
+}
+
+// lap F (x 180 dx^2) from its three axes and the centre.
+__device__ __forceinline__ FxWide fx_lap(const FxAxis (&a)[3], long long f0) {
+    FxWide w = {0, 0};
+    fx_wmac(w, -f0, 1470);
+    fx_wmac(w, a[0].s1 + a[1].s1 + a[2].s1, 270);
+    fx_wmac(w, a[0].n2 + a[1].n2 + a[2].n2, 27);
+    fx_wmac(w, a[0].s3 + a[1].s3 + a[2].s3, 2);
+    return w;
+}
+
+// Component C of u: G[a] = d_a u_C (x 60 dx, over 4); its share of V, the viscous
+// numerators 12 lap u + grad(div u) (x 2160 dx^2; with EXT, for any zeta, grad(div u)
+// alone, x 720 dx^2, and LU = lap u_C).
+template <int C, bool EXT>
+__device__ __forceinline__ void fx_u_component(const FxView &F, long long f0, FxWide (&V)[3],
+                                               long long (&G)[3], FxWide &LU) {
+    constexpr int B1 = C == 0 ? 1 : 0, B2 = C == 2 ? 1 : 2;
+    const FxAxis u[3] = {fx_axis<0>(F), fx_axis<1>(F), fx_axis<2>(F)};
+#pragma unroll
+    for (int a = 0; a < 3; ++a) G[a] = u[a].d >> 2;
+    if (EXT) {
+        fx_wmac(V[C], -f0, 1960);
+        fx_wmac(V[C], u[C].s1, 1080);
+        fx_wmac(V[C], u[C].n2, 108);
+        fx_wmac(V[C], u[C].s3, 8);
+        LU = fx_lap(u, f0);
+    } else {
+        fx_wmac(V[C], -f0, 19600);
+        fx_wmac(V[C], u[C].s1, 4320);
+        fx_wmac(V[C], u[C].n2, 432);
+        fx_wmac(V[C], u[C].s3, 32);
+        fx_wmac(V[C], u[B1].s1 + u[B2].s1, 3240);
+        fx_wmac(V[C], u[B1].n2 + u[B2].n2, 324);
+        fx_wmac(V[C], u[B1].s3 + u[B2].s3, 24);
+    }
+    fx_mixed<(C < B1 ? C : B1), (C < B1 ? B1 : C), false>(F, V[B1]);
+    fx_mixed<(C < B2 ? C : B2), (C < B2 ? B2 : C), false>(F, V[B2]);
+}
+
+// Component C of A: its share of B = curl A (x 60 dx, over 8) and of Jn = 4 (lap A -
+// grad(div A)) (x 720 dx^2, minus the current); LA = lap A_C (x 180 dx^2).
+template <int C>
+__device__ __forceinline__ void fx_a_component(const FxView &F, long long f0, FxWide (&Jn)[3],
+                                               long long (&B)[3], FxWide &LA) {
+    constexpr int B1 = C == 0 ? 1 : 0, B2 = C == 2 ? 1 : 2;
+    const FxAxis v[3] = {fx_axis<0>(F), fx_axis<1>(F), fx_axis<2>(F)};
+    if (C == 0) {
+        B[2] -= v[1].d >> 3;
+        B[1] += v[2].d >> 3;
+    } else if (C == 1) {
+        B[2] += v[0].d >> 3;
+        B[0] -= v[2].d >> 3;
+    } else {
+        B[1] -= v[0].d >> 3;
+        B[0] += v[1].d >> 3;
+    }
+    LA = fx_lap(v, f0);
+    fx_wmac(Jn[C], -f0, 3920);
+    fx_wmac(Jn[C], v[B1].s1 + v[B2].s1, 1080);
+    fx_wmac(Jn[C], v[B1].n2 + v[B2].n2, 108);
+    fx_wmac(Jn[C], v[B1].s3 + v[B2].s3, 8);
+    fx_mixed<(C < B1 ? C : B1), (C < B1 ? B1 : C), true>(F, Jn[B1]);
+    fx_mixed<(C < B2 ? C : B2), (C < B2 ? B2 : C), true>(F, Jn[B2]);
+}
+
+// An upper bound of a positive double as binary32 (its exponent within binary32's).
+__device__ __forceinline__ float fx_float_up(double v) {
+    const long long b = __double_as_longlong(v);
+    return __int_as_float((int)((b - (896ll << 52)) >> 29) + 1);
+}
+
+// The Runge-Kutta update of rk_update, the RHS already multiplied by dt.
+__device__ __forceinline__ void fx_update(const SubstepArgs<double, double> &a, bool active, int q,
+                                          long long o, double f, double w, double rhs) {
+    double wn = rhs;
+    if (!a.s0) wn = a.alpha * w + wn;
+    if (active) {
+        a.w[q][o] = wn;
+        a.fout[q][o] = f + a.beta * wn;
+    }
+}
+
+__device__ __forceinline__ void fx_arrive(fx_u64 *bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(fx_smem_u32(bar)) : "memory");
+}
+
+// What a CTA's warps share in the march along z.  No barrier spans the CTA inside the
+// march: a warp waits for the plane it needs, and the last of the sixteen to finish
+// its stencils of plane z asks for plane z + 4, so that some warps' stencils (shared
+// memory, integer pipes) run beside others' products and updates (FP64 pipe).
+struct FxShared {
+    fx_u64 full[FX_SLOTS];           // a plane has landed
+    fx_u64 given[FX_WARPS / 2];      // the A warp's exchange values are written ...
+    fx_u64 taken[FX_WARPS / 2];      // ... and read by the u warp of the same cells
+    unsigned done;                   // warps that have finished their stencils (cumulative)
+    int cfl_low;                     // the CTA's cfl_low below (bits of a positive float)
+};
+struct FxMarch {
+    const CUtensorMap *map;
+    long long *sm;
+    FxShared *sh;
+    int x0, y0, z0, z1;
+    int slot[FX_SLOTS];  // ring offsets of planes z-3 .. z+3, rolled by one per plane
+    int last;            // the slot that plane z + 3 is in, and the parity of its fill
+    unsigned parity;
+    bool ok;             // false once a bounded wait has run out
+    // plane z + 3 has landed
+    __device__ __forceinline__ bool arrive() {
+        ok = __all_sync(0xffffffffu, fx_wait(&sh->full[last], parity));
+        return ok;
+    }
+    // this warp has taken its stencils of plane z; once all have, plane z - 3's slot
+    // is free for plane z + 4
+    __device__ __forceinline__ void refill(int z) {
+        __syncwarp();
+        if ((threadIdx.x & 15) == 0 && (threadIdx.y & 1) == 0) {
+            __threadfence_block();
+            const unsigned n = atomicAdd(&sh->done, 1u) + 1u;
+            if (n == FX_WARPS * (unsigned)(z - z0 + 1) && z + 1 < z1) {
+                __threadfence_block();
+                fx_fetch(sm + slot[0], map, &sh->full[last == FX_SLOTS - 1 ? 0 : last + 1], x0, y0,
+                         z + 7);
+            }
+        }
+    }
+    __device__ __forceinline__ void next() {
+        const int first = slot[0];
+#pragma unroll
+        for (int d = 0; d < FX_SLOTS - 1; ++d) slot[d] = slot[d + 1];
+        slot[FX_SLOTS - 1] = first;
+        parity ^= last == FX_SLOTS - 1;
+        last = last == FX_SLOTS - 1 ? 0 : last + 1;
+    }
+};
+
+// Units of both halves: with kl, ku, ks, ka the binary exponents -s of the scales of
+// ln rho, u, s and A, a stencil numerator N stands for N 2^k; GL, GS, GU carry
+// 2^(k+2), B 2^(ka+3), J 2^(ka+9), X = 3/4 S 2^(ku+2), each below 2^60.8 as fx_split
+// wants.
+
+// The A half: A and the gradients of ln rho and s; dA/dt, the CFL speed, and for the
+// cell's other thread (through xch) the pressure and Lorentz forces, the advection
+// and conduction of s, eta j^2 / rho and 1/T.  (Which half takes which term is a
+// matter of balance: with the pressure and the entropy's advection in the u half,
+// that half ran 17.6 and this one 13.3 thousand cycles a plane.)
+template <bool CFL, bool EXT>
+__device__ __forceinline__ void fx_march_a(const SubstepArgs<double, double> &a, const FxCoefs &fc,
+                                           const FxPlan *plan, const fx_u64 *etab, double *xch,
+                                           FxMarch &m, int i, int j, double &cfl) {
+    const bool active = i < a.g.nx && j < a.g.ny;
+    const int kl = -plan->s[0], ku = -plan->s[1], ks = -plan->s[4], ka = -plan->s[5];
+    const bool pi_s = plan->pi_s != 0;
+    const int pi_rh = plan->pi_rh, pi_rl = plan->pi_rl;
+    const long long Cu[3] = {(long long)plan->C[1], (long long)plan->C[2], (long long)plan->C[3]};
+    const double c1cs2_ref = fc.c1dt * a.k.cs2_ref * plan->pi_f;
+    // sh->cfl_low: the largest CFL speed known so far, rounded down (the CTA's own and,
+    // from the start, what other CTAs have reported); cells whose upper bound lies below
+    // it need no exact speed (two square roots: 1150 FP64-pipe cycles)
+    const long long *const ring = m.sm + (threadIdx.y + R) * FXR + threadIdx.x + R;
+    fx_u64 *const given = &m.sh->given[threadIdx.y >> 1], *const taken = &m.sh->taken[threadIdx.y >> 1];
+    const int z0 = m.z0;
+    for (int z = z0; z < m.z1; ++z) {
+        if (!m.arrive()) break;
+        const long long o =
+            AC_BC(z * a.g.pxy + (long long)j * a.g.px + i, active ? a.g.elems : 1ll << 62, AC_BC_TILE_OUT);
+        // the cell's own values: asked for ahead of the stencils, needed after them
+        double f0[3] = {}, w0[3] = {}, lnrho = 0.0, ss = 0.0;
+        if (active) {
+            lnrho = fx_load_now(a.fin[0] + o);
+            ss = fx_load_now(a.fin[4] + o);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                f0[q] = fx_load_now(a.fin[5 + q] + o);
+                if (!a.s0) w0[q] = fx_load_now(a.w[5 + q] + o);
+            }
+        }
+        FxWide Jn[3] = {}, LA[3];
+        long long Bn[3] = {0, 0, 0};
+        const FxView Fx{ring + 5 * FX_FIELD_TILE, m.slot}, Fy{ring + 6 * FX_FIELD_TILE, m.slot},
+            Fz{ring + 7 * FX_FIELD_TILE, m.slot};
+        fx_a_component<0>(Fx, Fx(0, 0, 0), Jn, Bn, LA[0]);
+        fx_a_component<1>(Fy, Fy(0, 0, 0), Jn, Bn, LA[1]);
+        fx_a_component<2>(Fz, Fz(0, 0, 0), Jn, Bn, LA[2]);
+        long long GL[3], GS[3];
+        FxWide LL, LS;
+        {
+            const FxView Fl{ring, m.slot}, Fs{ring + 4 * FX_FIELD_TILE, m.slot};
+            const FxAxis l[3] = {fx_axis<0>(Fl), fx_axis<1>(Fl), fx_axis<2>(Fl)};
+            const FxAxis e[3] = {fx_axis<0>(Fs), fx_axis<1>(Fs), fx_axis<2>(Fs)};
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                GL[q] = l[q].d >> 2;
+                GS[q] = e[q].d >> 2;
+            }
+            if (EXT) {
+                LL = fx_lap(l, Fl(0, 0, 0));
+                LS = fx_lap(e, Fs(0, 0, 0));
+            }
+        }
+        FxSplit U[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            U[q] = fx_split(ring[(1 + q) * FX_FIELD_TILE + m.slot[R]] + Cu[q]);
+        m.refill(z);
+        // (every thread of a ragged tile computes, the active ones load and store: the
+        // barriers below want whole warps)
+        FxSplit B[3], J[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            B[q] = fx_split(Bn[q]);
+            J[q] = fx_split(fx_shift96<9>(fx_wide96(Jn[q])));
+        }
+        // thermodynamic factors 1/rho, e^xi, e^-xi
+        const double xi = a.k.gamma_cp * ss + a.k.gm1 * lnrho;
+        const long long xx = fx_from_double55(xi);
+        const double rho_inv = fx_exp55(-fx_from_double55(lnrho), etab, FX_L70);
+        const double exi = fx_exp55(xx, etab, FX_L70), emxi = fx_exp55(-xx, etab, FX_L70);
+        const double cjb = rho_inv * fc.jb, cp = exi * c1cs2_ref;
+        // pressure, from grad(ln rho + s / c_p), and Lorentz force
+        const int ej = FX_EB + 44 + 2 * ka;
+        double pl[3] = {cjb * fx_to_double(fx_det2(J[1], B[2], J[2], B[1]), ej),
+                        cjb * fx_to_double(fx_det2(J[2], B[0], J[0], B[2]), ej),
+                        cjb * fx_to_double(fx_det2(J[0], B[1], J[1], B[0]), ej)};
+        FxSplit SS[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const long long big = pi_s ? GS[q] : GL[q], small = pi_s ? GL[q] : GS[q];
+            pl[q] = fma(-cp, fx_to_double(big + fx_mulfrac(small, pi_rh, pi_rl),
+                                          FX_EB64 + 2 + (pi_s ? ks : kl)), pl[q]);
+            SS[q] = fx_split(GS[q]);
+        }
+        // entropy: advection, conduction, eta j^2 / rho
+        double rs = -(fc.c1dt * fx_to_double(fx_dot3(U, SS), FX_EB + 34 + ku + ks));
+        double h = fx_to_double(fx_dot3(J, J), FX_EB + 50 + 2 * ka) * (rho_inv * fc.j2);
+        if (EXT) {
+            h = fma(fc.inv_T_ref * fc.hc_dt, rho_inv, h);
+            // lap xi and |grad xi|^2 / c1^2, xi = gamma s / c_p + (gamma - 1) ln rho
+            const FxSplit SL[3] = {fx_split(GL[0]), fx_split(GL[1]), fx_split(GL[2])};
+            const double lapxi = (a.k.gamma_cp * fx_to_double(fx_wide96(LS), FX_EB + ks) +
+                                  a.k.gm1 * fx_to_double(fx_wide96(LL), FX_EB + kl)) * fc.inv180dx2;
+            const double ss2 = fx_to_double(fx_dot3(SS, SS), FX_EB + 36 + 2 * ks);
+            const double sl2 = fx_to_double(fx_dot3(SS, SL), FX_EB + 36 + ks + kl);
+            const double ll2 = fx_to_double(fx_dot3(SL, SL), FX_EB + 36 + 2 * kl);
+            const double gxi2 = a.k.gamma_cp * (a.k.gamma_cp * ss2 + 2.0 * a.k.gm1 * sl2) +
+                                a.k.gm1 * a.k.gm1 * ll2;
+            rs += rho_inv * (fc.K_dt * lapxi + fc.K_c1sq * gxi2);
+        }
+        // the u warp has read the values of the plane before
+        if (z > z0) m.ok = __all_sync(0xffffffffu, fx_wait(taken, (z - z0 - 1) & 1)) && m.ok;
+#pragma unroll
+        for (int q = 0; q < 3; ++q) xch[q * FXT * FXT] = pl[q];
+        xch[3 * FXT * FXT] = h;
+        xch[4 * FXT * FXT] = rs;
+        xch[5 * FXT * FXT] = emxi;
+        __syncwarp();
+        if ((threadIdx.x & 15) == 0 && (threadIdx.y & 1) == 0) fx_arrive(given);
+        const int eu = FX_EB + 35 + ku + ka;
+        const double ub[3] = {fx_to_double(fx_det2(U[1], B[2], U[2], B[1]), eu),
+                              fx_to_double(fx_det2(U[2], B[0], U[0], B[2]), eu),
+                              fx_to_double(fx_det2(U[0], B[1], U[1], B[0]), eu)};
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const double la = fx_to_double(fx_wide96(LA[q]), FX_EB + ka);
+            fx_update(a, active, 5 + q, o, f0[q], w0[q], fma(fc.c1dt, ub[q], fc.eta180 * la));
+        }
+        if (CFL && active) {
+            // upper bound of |u| + sqrt(c_s^2 + |B|^2 / rho) from the high words in
+            // binary32; the exact speed only where that exceeds the largest known
+            float u2 = 0.f, b2 = 0.f;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const float uf = fabsf((float)U[q].hi) + 1.f, bf = fabsf((float)B[q].hi) + 1.f;
+                u2 = fmaf(uf, uf, u2);
+                b2 = fmaf(bf, bf, b2);
+            }
+            // (floors: a scale that binary32 cannot hold only makes the bound larger)
+            const float us = fmaxf(exp2f((float)(ku + 32)), 1e-37f),
+                        bs = fmaxf(exp2f((float)(ka + 35)) * fc.c1f, 1e-18f);
+            const float up =
+                1.0001f * (us * sqrtf(u2) + sqrtf(fc.cs2_ref_f * fx_float_up(exi) +
+                                                  bs * bs * b2 * fx_float_up(rho_inv)));
+            if (!(up <= __int_as_float(*(volatile int *)&m.sh->cfl_low))) {
+                const double x = ldg(a.fin[1] + o), y = ldg(a.fin[2] + o), zz = ldg(a.fin[3] + o);
+                const double bb = fx_to_double(fx_dot3(B, B), FX_EB + 38 + 2 * ka) * fc.c1sq;
+                const double c = sqrt(x * x + y * y + zz * zz) +
+                                 sqrt(a.k.cs2_ref * exi + bb * rho_inv);
+                if (c > cfl || c != c) {
+                    cfl = c;
+                    if (c < 1e30) atomicMax(&m.sh->cfl_low, __float_as_int(__double2float_rd(c)));
+                }
+            }
+        }
+        if (!m.ok) break;
+        m.next();
+    }
+}
+
+// The other half: the equations of ln rho, u and s.
+template <bool EXT>
+__device__ __forceinline__ void fx_march_u(const SubstepArgs<double, double> &a, const FxCoefs &fc,
+                                           const FxPlan *plan, const double *xch, FxMarch &m, int i, int j) {
+    const bool active = i < a.g.nx && j < a.g.ny;
+    const int kl = -plan->s[0], ku = -plan->s[1];
+    const long long Cu[3] = {(long long)plan->C[1], (long long)plan->C[2], (long long)plan->C[3]};
+    double2 exy = make_double2(0.0, 0.0);
+    if (a.force_on && active) {
+        const double2 ex = a.ftab[i], ey = a.ftab[a.g.nx + j];
+        exy.x = ex.x * ey.x - ex.y * ey.y;
+        exy.y = ex.x * ey.y + ex.y * ey.x;
+    }
+    const long long *const ring = m.sm + (threadIdx.y + R) * FXR + threadIdx.x + R;
+    fx_u64 *const given = &m.sh->given[threadIdx.y >> 1], *const taken = &m.sh->taken[threadIdx.y >> 1];
+    const int z0 = m.z0;
+    for (int z = z0; z < m.z1; ++z) {
+        if (!m.arrive()) break;
+        const long long o =
+            AC_BC(z * a.g.pxy + (long long)j * a.g.px + i, active ? a.g.elems : 1ll << 62, AC_BC_TILE_OUT);
+        double f0[5] = {}, w0[5] = {};
+        if (active) {
+#pragma unroll
+            for (int q = 0; q < 5; ++q) {
+                f0[q] = fx_load_now(a.fin[q] + o);
+                if (!a.s0) w0[q] = fx_load_now(a.w[q] + o);
+            }
+        }
+        long long GL[3], GU[3][3], u0[3];
+        FxWide V[3] = {}, LU[3];
+        {
+            const FxView Fl{ring, m.slot};
+            const FxAxis l[3] = {fx_axis<0>(Fl), fx_axis<1>(Fl), fx_axis<2>(Fl)};
+#pragma unroll
+            for (int q = 0; q < 3; ++q) GL[q] = l[q].d >> 2;
+        }
+        {
+            const FxView Fx{ring + FX_FIELD_TILE, m.slot}, Fy{ring + 2 * FX_FIELD_TILE, m.slot},
+                Fz{ring + 3 * FX_FIELD_TILE, m.slot};
+            u0[0] = Fx(0, 0, 0);
+            u0[1] = Fy(0, 0, 0);
+            u0[2] = Fz(0, 0, 0);
+            fx_u_component<0, EXT>(Fx, u0[0], V, GU[0], LU[0]);
+            fx_u_component<1, EXT>(Fy, u0[1], V, GU[1], LU[1]);
+            fx_u_component<2, EXT>(Fz, u0[2], V, GU[2], LU[2]);
+        }
+        m.refill(z);
+        FxSplit U[3], SL[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            U[q] = fx_split(u0[q] + Cu[q]);
+            SL[q] = fx_split(GL[q]);
+        }
+        const long long div = GU[0][0] + GU[1][1] + GU[2][2];
+        const double divu = fx_to_double(div, FX_EB64 + 2 + ku);
+        const double adv_l = fx_to_double(fx_dot3(U, SL), FX_EB + 34 + ku + kl);
+        fx_update(a, active, 0, o, f0[0], w0[0], -(fc.c1dt * adv_l) - fc.c1dt * divu);
+        // viscosity, advection, 2 nu S . grad ln rho and the forcing
+        double cph = 0.0;
+        if (a.force_on) {
+            const double2 ez = a.ftab[a.g.nx + a.g.ny + z];
+            cph = exy.x * ez.x - exy.y * ez.y;
+        }
+        double ru[3];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const FxSplit g[3] = {fx_split(GU[q][0]), fx_split(GU[q][1]), fx_split(GU[q][2])};
+            const double v = fc.nu2160 * fx_to_double(fx_wide96(V[q]), FX_EB + ku);
+            ru[q] = EXT ? fma(fc.nu180, fx_to_double(fx_wide96(LU[q]), FX_EB + ku), v) : v;
+            ru[q] = fma(-fc.c1dt, fx_to_double(fx_dot3(U, g), FX_EB + 34 + 2 * ku), ru[q]);
+            ru[q] = fma(fc.amp_dt[q], cph, ru[q]);
+        }
+        // the traceless rate of strain, X = 3/4 S
+        double h;
+        {
+            FxSplit D[3], O[3];  // diagonal; xy, xz, yz
+#pragma unroll
+            for (int q = 0; q < 3; ++q) D[q] = fx_split((3 * GU[q][q] - div) >> 2);
+            const long long xy = GU[0][1] + GU[1][0], xz = GU[0][2] + GU[2][0],
+                            yz = GU[1][2] + GU[2][1];
+            O[0] = fx_split((xy + (xy >> 1)) >> 2);
+            O[1] = fx_split((xz + (xz >> 1)) >> 2);
+            O[2] = fx_split((yz + (yz >> 1)) >> 2);
+            const FxSplit r0[3] = {D[0], O[0], O[1]}, r1[3] = {O[0], D[1], O[2]},
+                          r2[3] = {O[1], O[2], D[2]};
+            const int eb = FX_EB + 36 + ku + kl;
+            ru[0] = fma(fc.sg, fx_to_double(fx_dot3(r0, SL), eb), ru[0]);
+            ru[1] = fma(fc.sg, fx_to_double(fx_dot3(r1, SL), eb), ru[1]);
+            ru[2] = fma(fc.sg, fx_to_double(fx_dot3(r2, SL), eb), ru[2]);
+            const Fx96 dd = fx_dot3(D, D), oo = fx_dot3(O, O);
+            const fx_u64 low = (fx_u64)dd.low + 2ull * oo.low;
+            Fx96 t;
+            t.top = dd.top + 2 * oo.top + (long long)(low >> 32);
+            t.low = (unsigned)low;
+            h = fc.s2 * fx_to_double(t, FX_EB + 36 + 2 * ku);
+        }
+        if (EXT) h = fma(fc.inv_T_ref * fc.zeta_c1sq * divu, divu, h);
+        // the other thread's terms
+        m.ok = __all_sync(0xffffffffu, fx_wait(given, (z - z0) & 1)) && m.ok;
+        double x[FX_XCH];
+#pragma unroll
+        for (int q = 0; q < FX_XCH; ++q) x[q] = xch[q * FXT * FXT];
+        __syncwarp();
+        if ((threadIdx.x & 15) == 0 && (threadIdx.y & 1) == 0) fx_arrive(taken);
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            fx_update(a, active, 1 + q, o, f0[1 + q], w0[1 + q], ru[q] + x[q]);
+        fx_update(a, active, 4, o, f0[4], w0[4], fma(x[5], h + x[3], x[4]));
+        if (!m.ok) break;
+        m.next();
+    }
+}
+
+template <bool CFL, bool EXT = false>
+__global__ void __launch_bounds__(2 * FXT * FXT, 1)
+    substep_fx_kernel(const SubstepArgs<double, double> a, const __grid_constant__ CUtensorMap map,
+                      const FxCoefs fc, FxPlan *plan) {
+    if (plan->kern != FX_GROUP) return;
+    extern __shared__ __align__(128) unsigned char fx_smem[];
+    __shared__ FxShared sh;
+    fx_u64 *const etab = reinterpret_cast<fx_u64 *>(fx_smem + (size_t)FX_SLOTS * FX_PLANE_BYTES);
+    double *const xch = reinterpret_cast<double *>(etab + 256) + threadIdx.y * FXT + threadIdx.x;
+    const int tid = (threadIdx.z * FXT + threadIdx.y) * FXT + threadIdx.x;
+    FxMarch m;
+    m.map = &map;
+    m.sm = reinterpret_cast<long long *>(fx_smem);
+    m.sh = &sh;
+    m.x0 = blockIdx.x * FXT;
+    m.y0 = blockIdx.y * FXT;
+    m.z0 = blockIdx.z * a.zchunk;
+    m.z1 = min(m.z0 + a.zchunk, a.g.nz);
+    if (tid == 0) {
+        fx_u64 *const bars = sh.full;  // all of them, each for one arrival a phase
+        for (int b = 0; b < FX_SLOTS + FX_WARPS; ++b)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(fx_smem_u32(bars + b))
+                         : "memory");
+        sh.done = 0;
+        if (CFL) {
+            const double g = __longlong_as_double(
+                (long long)*reinterpret_cast<volatile unsigned long long *>(a.cfl_max));
+            sh.cfl_low = __float_as_int(g < 1e30 ? __double2float_rd(g) : 1e30f);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        // padded plane z + d holds plane z - 3 + d: the planes z0 - 3 .. z0 + 3
+        for (int d = 0; d < FX_SLOTS; ++d)
+            fx_fetch(m.sm + d * FX_PLANE, &map, &sh.full[d], m.x0, m.y0, m.z0 + d);
+    }
+    for (int t = tid; t < 256; t += 2 * FXT * FXT) etab[t] = EXP_FIX[t];
+    __syncthreads();
+#pragma unroll
+    for (int d = 0; d < FX_SLOTS; ++d) m.slot[d] = d * FX_PLANE;
+    m.ok = true;
+    for (int d = 0; d < FX_SLOTS - 1; ++d) m.ok = fx_wait(&sh.full[d], 0) && m.ok;
+    m.ok = __all_sync(0xffffffffu, m.ok);
+    m.last = FX_SLOTS - 1;
+    m.parity = 0;
+    double cfl = 0.0;
+    const int i = m.x0 + threadIdx.x, j = m.y0 + threadIdx.y;
+    if (m.ok) {
+        if (threadIdx.z)
+            fx_march_a<CFL, EXT>(a, fc, plan, etab, xch, m, i, j, cfl);
+        else
+            fx_march_u<EXT>(a, fc, plan, xch, m, i, j);
+    }
+    if (!m.ok) {  // report, and let no copy be in flight when the CTA ends
+        atomicExch(&plan->err, 1);
+        for (int d = 0; d < FX_SLOTS; ++d) fx_wait(&sh.full[d], d <= m.last ? m.parity : m.parity ^ 1);
+    }
     if (CFL) block_max_to_global(cfl, a.cfl_max);
 }
 
@@ -649,7 +1238,7 @@ __global__ void __launch_bounds__(128, 2) substep_fx_kernel(const SubstepArgs<do
 template <bool CFL, bool EXT = false>
 __global__ void __launch_bounds__(128) substep_fx_plain_kernel(const SubstepArgs<double, double> a,
                                                               const FxPlan *plan) {
-    if (plan->mode != FX_PLAIN) return;
+    if (plan->kern != FX_PLAIN) return;
     substep_body<double, double, IdxPeriodic32, CFL, 3, EXT>(a);
 }
 
