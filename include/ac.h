@@ -213,7 +213,10 @@ int ac_get_stencil_order(const ac_handle *h, int *order);
  * integer sums whenever they apply (binary64 fields, periodic layout, equal
  * spacing dx = dy = dz, stencil order 6, a step dt with |dt| in [1e-100, 1e100]:
  * those kernels fold dt into their coefficients), plain binary64 sums
- * otherwise.  With
+ * otherwise.  (Unequal spacings no more than a factor of 8 apart, from 16384 cells
+ * on, use them too, each axis's numerators scaled to the smallest spacing, while the
+ * state lies in the ranges of the form b = 56 below; ac_get_stencil_path and
+ * ac_get_stencil_modes do not count that form.)  With
  * integer sums every field is first written, on the device before each
  * substep, as int64 fixed point about its own offset: F = round((f - c)
  * 2^(b - E)), c the midpoint of the field's range and 2^E above its half-range

@@ -102,7 +102,8 @@ struct SubstepLaunch {
     double alpha, beta, dt;
     int s;
     unsigned long long *cfl_max;  // substep 0: device word for the max CFL speed (or NULL)
-    // binary64 with integer stencil sums (cubic periodic grids): int64 copies of
+    // binary64 with integer stencil sums (periodic grids): use_fx = 1 for equal spacing,
+    // 2 for unequal; int64 copies of
     // the fields, padded by their periodic halo, with their tensor map, 16 words of per-field extremes and the device plan of the
     // substep (fx_plan_bytes()); use_fx = 0 selects plain binary64 sums.
     int use_fx;
@@ -110,7 +111,7 @@ struct SubstepLaunch {
     const CUtensorMap *fx_map;
     unsigned long long *fx_stats;
     void *fx_plan;
-    double dx;
+    double dx[3];
     // optional: recorded after the preparation kernels (integer-sum path:
     // extremes, plan, quantisation), before the substep kernel itself
     cudaEvent_t ev_mid;

@@ -31,6 +31,16 @@ static int fx_zchunk(long long tiles, int nz) {
     return best;
 }
 
+// r in (0, 1] as hi 2^-31 + lo 2^-62 (1 as 1 - 2^-62).
+static void fx_fraction(double r, int *hi, int *lo) {
+    *hi = *lo = 0x7fffffff;
+    if (r < 1.0) {
+        const double t = r * 2147483648.0;
+        *hi = (int)t;
+        *lo = (int)((t - (double)*hi) * 2147483648.0);
+    }
+}
+
 // Padded row length (even: the strides of the tensor map are multiples of 16 bytes),
 // bytes of the eight padded int64 arrays, and the tensor map over them: dims (px,
 // py, pz, field), box one plane of a tile with its halo, all fields.
@@ -57,10 +67,10 @@ cudaError_t fx_encode_map(void *base, const Geom &g, CUtensorMap *map) {
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <bool CFL, bool EXT>
+template <bool CFL, bool EXT, bool ANISO>
 static cudaError_t launch_fx_group(SubstepArgs<double, double> a, const CUtensorMap &map,
                                    const FxCoefs &fc, FxPlan *plan, cudaStream_t st) {
-    auto k = substep_fx_kernel<CFL, EXT>;
+    auto k = substep_fx_kernel<CFL, EXT, ANISO>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FX_SMEM);
     if (e != cudaSuccess) return e;
     const unsigned gx = (a.g.nx + FXT - 1) / FXT, gy = (a.g.ny + FXT - 1) / FXT;
@@ -102,15 +112,27 @@ cudaError_t launch_substep_f64(const SubstepLaunch &L, cudaStream_t st, int *lau
     a.ftab = L.force.tab;
     for (int m = 0; m < 3; ++m) a.amp_e[m] = L.force.amp_e[m];
     a.cfl_max = L.cfl_max;
-    // the step folded into the RHS coefficients
-    FxCoefs fc;
+    // the step folded into the RHS coefficients; with unequal spacing they hold the
+    // smallest one and the numerators carry the ratios
+    const bool aniso = L.use_fx == 2;
+    const double h = fmin(L.dx[0], fmin(L.dx[1], L.dx[2]));
+    FxCoefs fc = {};
+    if (aniso) {
+        const int pa[3] = {0, 0, 1}, pb[3] = {1, 2, 2};
+        for (int m = 0; m < 3; ++m) {
+            const double r = h / L.dx[m];
+            fx_fraction(r, &fc.r1h[m], &fc.r1l[m]);
+            fx_fraction(r * r, &fc.r2h[m], &fc.r2l[m]);
+            fx_fraction((h / L.dx[pa[m]]) * (h / L.dx[pb[m]]), &fc.rmh[m], &fc.rml[m]);
+        }
+    }
     const double dts = L.dt;
-    const double c1 = 1.0 / (60.0 * L.dx);
+    const double c1 = 1.0 / (60.0 * h);
     fc.c1dt = dts * c1;
-    fc.nu180 = dts * (L.ph.nu / (180.0 * L.dx * L.dx));
-    fc.nu2160 = dts * ((L.ph.nu + 3.0 * L.ph.zeta) / (2160.0 * L.dx * L.dx));
-    fc.inv180dx2 = 1.0 / (180.0 * L.dx * L.dx);
-    fc.inv720dx2 = 1.0 / (720.0 * L.dx * L.dx);
+    fc.nu180 = dts * (L.ph.nu / (180.0 * h * h));
+    fc.nu2160 = dts * ((L.ph.nu + 3.0 * L.ph.zeta) / (2160.0 * h * h));
+    fc.inv180dx2 = 1.0 / (180.0 * h * h);
+    fc.inv720dx2 = 1.0 / (720.0 * h * h);
     fc.two_nu_c1sq = dts * (2.0 * L.ph.nu * c1 * c1);
     fc.K_c1sq = dts * (L.ph.K * c1 * c1);
     fc.zeta_c1sq = dts * (L.ph.zeta * c1 * c1);
@@ -133,7 +155,7 @@ cudaError_t launch_substep_f64(const SubstepLaunch &L, cudaStream_t st, int *lau
     FxPlan *plan = static_cast<FxPlan *>(L.fx_plan);
     cudaError_t e;
     fx_stats_kernel<<<fx_grid(n / 2), 256, 0, st>>>(fx, n, L.fx_stats);
-    fx_plan_kernel<<<1, 32, 0, st>>>(L.fx_stats, plan, L.ph.inv_cp, L.ph.gamma_cp, L.ph.gm1);
+    fx_plan_kernel<<<1, 32, 0, st>>>(L.fx_stats, plan, L.ph.inv_cp, L.ph.gamma_cp, L.ph.gm1, aniso);
     fx_quantize_kernel<<<fx_grid(32ll * fx.py * fx.pz), 256, 0, st>>>(fx, L.g, plan);
     if (L.ev_mid) {
         e = cudaEventRecord(L.ev_mid, st);
@@ -149,18 +171,19 @@ cudaError_t launch_substep_f64(const SubstepLaunch &L, cudaStream_t st, int *lau
     a.zchunk = zchunk;
     const dim3 grid(gx, gy, (L.g.nz + zchunk - 1) / zchunk);
     const bool ext = L.ph.ext(), cfl = a.cfl_max != nullptr;
-    // one kernel per mode; the two the plan did not choose return at once
-#define AC_FX(C, X)                                                            \
-    do {                                                                       \
-        e = launch_fx_group<C, X>(a, *L.fx_map, fc, plan, st);                  \
-        if (e != cudaSuccess) return e;                                         \
-        substep_fx_field_kernel<C, X><<<grid, block, 0, st>>>(a, fx, fc, plan); \
-        substep_fx_plain_kernel<C, X><<<grid, block, 0, st>>>(a, plan);          \
+    // one kernel per plan; those the plan did not choose return at once
+#define AC_FX(C, X)                                                                \
+    do {                                                                           \
+        e = aniso ? launch_fx_group<C, X, true>(a, *L.fx_map, fc, plan, st)        \
+                  : launch_fx_group<C, X, false>(a, *L.fx_map, fc, plan, st);      \
+        if (e != cudaSuccess) return e;                                            \
+        if (!aniso) substep_fx_field_kernel<C, X><<<grid, block, 0, st>>>(a, fx, fc, plan); \
+        substep_fx_plain_kernel<C, X><<<grid, block, 0, st>>>(a, plan);            \
     } while (0)
     if (ext) { if (cfl) AC_FX(true, true); else AC_FX(false, true); }
     else { if (cfl) AC_FX(true, false); else AC_FX(false, false); }
 #undef AC_FX
-    *launches += 6;
+    *launches += aniso ? 5 : 6;
     return cudaGetLastError();
 }
 

@@ -174,7 +174,7 @@ __global__ void __launch_bounds__(256) fx_stats_kernel(FxPtrs p, long long n,
 // on the kernel.  Thread 0 also counts the substep under its mode: plain,
 // per-field (a component more than one binade below its group's largest) or group.
 __global__ void fx_plan_kernel(unsigned long long *stats, FxPlan *plan, double inv_cp,
-                               double gamma_cp, double gm1) {
+                               double gamma_cp, double gm1, int aniso) {
     const int q = threadIdx.x;
     int bad = 0, zero = 1, e = -100000, ec = -100000;
     double c = 0.0, big = 0.0;
@@ -222,7 +222,8 @@ __global__ void fx_plan_kernel(unsigned long long *stats, FxPlan *plan, double i
     if (g == 1) out |= ec > eg + 4;
     if (q == 0) out |= !(big < 64.0) || !(xb < 64.0);
     const int any_out = __any_sync(0xffffffffu, out);
-    const int kern = any_bad ? FX_PLAIN : (any_out ? FX_FIELD : FX_GROUP);
+    // (FX_FIELD wants equal spacing: without it the plain stencils take its place)
+    const int kern = any_bad || (aniso && any_out) ? FX_PLAIN : (any_out ? FX_FIELD : FX_GROUP);
     const int mode = any_bad ? FX_PLAIN : (far ? FX_FIELD : FX_GROUP);
     int s = FX_FIELD_BITS - (e > -100000 ? e : 0);
     if (kern == FX_GROUP) s = FX_BITS - eg;
@@ -251,7 +252,7 @@ __global__ void fx_plan_kernel(unsigned long long *stats, FxPlan *plan, double i
             plan->pi_rl = rl;
             plan->pi_f = pi_s ? inv_cp : 1.0;
         }
-        plan->taken[mode] += 1ull;
+        if (!aniso) plan->taken[mode] += 1ull;
     }
 }
 
@@ -386,6 +387,10 @@ struct FxCoefs {
     double c1sq;       // 1 / (60 dx)^2
     double inv_T_ref;  // c_p (gamma - 1) / cs2_ref
     float c1f, cs2_ref_f;  // c1 and cs2_ref rounded up (the CFL bound)
+    // unequal spacing (dx above then stands for the smallest, h): the numerators of axis
+    // a times h / dx_a, (h / dx_a)^2 and, for the planes xy, xz, yz, h^2 / (dx_a dx_b),
+    // each hi 2^-31 + lo 2^-62
+    int r1h[3], r1l[3], r2h[3], r2l[3], rmh[3], rml[3];
 };
 
 // Eqs. B.1-B.4 at one cell as cell_physics computes them, times dts (the step
@@ -776,6 +781,70 @@ __device__ __forceinline__ FxWide fx_lap(const FxAxis (&a)[3], long long f0) {
     return w;
 }
 
+// Unequal spacing: each numerator is brought to the smallest spacing's factor by one
+// fixed-point product, then sums run in 64 bits: first derivatives in the units above,
+// second ones over 2^6 (a quantum of 64 beside the 180 that the rounding of F leaves
+// in a second-derivative numerator), mixed ones and grad(div) over 2^8.
+template <bool ANISO>
+__device__ __forceinline__ long long fx_first(long long d, const FxCoefs &fc, int a) {
+    return ANISO ? fx_mulfrac(d, fc.r1h[a], fc.r1l[a]) : d;
+}
+__device__ __forceinline__ long long fx_second(const FxAxis &a, long long f0, const FxCoefs &fc, int ax) {
+    FxWide w = {0, 0};
+    fx_wmac(w, -f0, 490);
+    fx_wmac(w, a.s1, 270);
+    fx_wmac(w, a.n2, 27);
+    fx_wmac(w, a.s3, 2);
+    return fx_mulfrac(fx_shift96<6>(fx_wide96(w)), fc.r2h[ax], fc.r2l[ax]);
+}
+template <int A, int B, bool NEG>
+__device__ __forceinline__ long long fx_mixed_scaled(const FxView &F, const FxCoefs &fc) {
+    FxWide w = {0, 0};
+    fx_mixed<A, B, NEG>(F, w);
+    constexpr int pl = Plane<A, B>::id;
+    return fx_mulfrac(fx_shift96<6>(fx_wide96(w)), fc.rmh[pl], fc.rml[pl]) >> 2;
+}
+template <int C>
+__device__ __forceinline__ void fx_u_component_scaled(const FxView &F, long long f0, const FxCoefs &fc,
+                                                      long long (&GD)[3], long long (&G)[3],
+                                                      long long &LU) {
+    constexpr int B1 = C == 0 ? 1 : 0, B2 = C == 2 ? 1 : 2;
+    const FxAxis u[3] = {fx_axis<0>(F), fx_axis<1>(F), fx_axis<2>(F)};
+    long long n[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        G[a] = fx_first<true>(u[a].d >> 2, fc, a);
+        n[a] = fx_second(u[a], f0, fc, a);
+    }
+    LU = n[0] + n[1] + n[2];
+    GD[C] += n[C];
+    GD[B1] += fx_mixed_scaled<(C < B1 ? C : B1), (C < B1 ? B1 : C), false>(F, fc);
+    GD[B2] += fx_mixed_scaled<(C < B2 ? C : B2), (C < B2 ? B2 : C), false>(F, fc);
+}
+template <int C>
+__device__ __forceinline__ void fx_a_component_scaled(const FxView &F, long long f0, const FxCoefs &fc,
+                                                      long long (&Jn)[3], long long (&B)[3],
+                                                      long long &LA) {
+    constexpr int B1 = C == 0 ? 1 : 0, B2 = C == 2 ? 1 : 2;
+    const FxAxis v[3] = {fx_axis<0>(F), fx_axis<1>(F), fx_axis<2>(F)};
+    if (C == 0) {
+        B[2] -= fx_first<true>(v[1].d >> 3, fc, 1);
+        B[1] += fx_first<true>(v[2].d >> 3, fc, 2);
+    } else if (C == 1) {
+        B[2] += fx_first<true>(v[0].d >> 3, fc, 0);
+        B[0] -= fx_first<true>(v[2].d >> 3, fc, 2);
+    } else {
+        B[1] -= fx_first<true>(v[0].d >> 3, fc, 0);
+        B[0] += fx_first<true>(v[1].d >> 3, fc, 1);
+    }
+    const long long n[3] = {fx_second(v[0], f0, fc, 0), fx_second(v[1], f0, fc, 1),
+                            fx_second(v[2], f0, fc, 2)};
+    LA = n[0] + n[1] + n[2];
+    Jn[C] += n[B1] + n[B2];
+    Jn[B1] += fx_mixed_scaled<(C < B1 ? C : B1), (C < B1 ? B1 : C), true>(F, fc);
+    Jn[B2] += fx_mixed_scaled<(C < B2 ? C : B2), (C < B2 ? B2 : C), true>(F, fc);
+}
+
 // Component C of u: G[a] = d_a u_C (x 60 dx, over 4); its share of V, the viscous
 // numerators 12 lap u + grad(div u) (x 2160 dx^2; with EXT, for any zeta, grad(div u)
 // alone, x 720 dx^2, and LU = lap u_C).
@@ -911,7 +980,7 @@ struct FxMarch {
 // and conduction of s, eta j^2 / rho and 1/T.  (Which half takes which term is a
 // matter of balance: with the pressure and the entropy's advection in the u half,
 // that half ran 17.6 and this one 13.3 thousand cycles a plane.)
-template <bool CFL, bool EXT>
+template <bool CFL, bool EXT, bool ANISO>
 __device__ __forceinline__ void fx_march_a(const SubstepArgs<double, double> &a, const FxCoefs &fc,
                                            const FxPlan *plan, const fx_u64 *etab, double *xch,
                                            FxMarch &m, int i, int j, double &cfl) {
@@ -946,23 +1015,36 @@ __device__ __forceinline__ void fx_march_a(const SubstepArgs<double, double> &a,
         long long Bn[3] = {0, 0, 0};
         const FxView Fx{ring + 5 * FX_FIELD_TILE, m.slot}, Fy{ring + 6 * FX_FIELD_TILE, m.slot},
             Fz{ring + 7 * FX_FIELD_TILE, m.slot};
-        fx_a_component<0>(Fx, Fx(0, 0, 0), Jn, Bn, LA[0]);
-        fx_a_component<1>(Fy, Fy(0, 0, 0), Jn, Bn, LA[1]);
-        fx_a_component<2>(Fz, Fz(0, 0, 0), Jn, Bn, LA[2]);
+        long long Js[3] = {0, 0, 0}, Ls[3];  // unequal spacing: -j over 2^8, lap A over 2^6
+        if constexpr (ANISO) {
+            fx_a_component_scaled<0>(Fx, Fx(0, 0, 0), fc, Js, Bn, Ls[0]);
+            fx_a_component_scaled<1>(Fy, Fy(0, 0, 0), fc, Js, Bn, Ls[1]);
+            fx_a_component_scaled<2>(Fz, Fz(0, 0, 0), fc, Js, Bn, Ls[2]);
+        } else {
+            fx_a_component<0>(Fx, Fx(0, 0, 0), Jn, Bn, LA[0]);
+            fx_a_component<1>(Fy, Fy(0, 0, 0), Jn, Bn, LA[1]);
+            fx_a_component<2>(Fz, Fz(0, 0, 0), Jn, Bn, LA[2]);
+        }
         long long GL[3], GS[3];
         FxWide LL, LS;
+        long long LLs = 0, LSs = 0;
         {
             const FxView Fl{ring, m.slot}, Fs{ring + 4 * FX_FIELD_TILE, m.slot};
             const FxAxis l[3] = {fx_axis<0>(Fl), fx_axis<1>(Fl), fx_axis<2>(Fl)};
             const FxAxis e[3] = {fx_axis<0>(Fs), fx_axis<1>(Fs), fx_axis<2>(Fs)};
 #pragma unroll
             for (int q = 0; q < 3; ++q) {
-                GL[q] = l[q].d >> 2;
-                GS[q] = e[q].d >> 2;
+                GL[q] = fx_first<ANISO>(l[q].d >> 2, fc, q);
+                GS[q] = fx_first<ANISO>(e[q].d >> 2, fc, q);
             }
-            if (EXT) {
+            if (EXT && !ANISO) {
                 LL = fx_lap(l, Fl(0, 0, 0));
                 LS = fx_lap(e, Fs(0, 0, 0));
+            }
+            if (EXT && ANISO) {
+                const long long l0 = Fl(0, 0, 0), e0 = Fs(0, 0, 0);
+                LLs = fx_second(l[0], l0, fc, 0) + fx_second(l[1], l0, fc, 1) + fx_second(l[2], l0, fc, 2);
+                LSs = fx_second(e[0], e0, fc, 0) + fx_second(e[1], e0, fc, 1) + fx_second(e[2], e0, fc, 2);
             }
         }
         FxSplit U[3];
@@ -976,7 +1058,7 @@ __device__ __forceinline__ void fx_march_a(const SubstepArgs<double, double> &a,
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
             B[q] = fx_split(Bn[q]);
-            J[q] = fx_split(fx_shift96<9>(fx_wide96(Jn[q])));
+            J[q] = fx_split(ANISO ? Js[q] >> 1 : fx_shift96<9>(fx_wide96(Jn[q])));
         }
         // thermodynamic factors 1/rho, e^xi, e^-xi
         const double xi = a.k.gamma_cp * ss + a.k.gm1 * lnrho;
@@ -1004,8 +1086,11 @@ __device__ __forceinline__ void fx_march_a(const SubstepArgs<double, double> &a,
             h = fma(fc.inv_T_ref * fc.hc_dt, rho_inv, h);
             // lap xi and |grad xi|^2 / c1^2, xi = gamma s / c_p + (gamma - 1) ln rho
             const FxSplit SL[3] = {fx_split(GL[0]), fx_split(GL[1]), fx_split(GL[2])};
-            const double lapxi = (a.k.gamma_cp * fx_to_double(fx_wide96(LS), FX_EB + ks) +
-                                  a.k.gm1 * fx_to_double(fx_wide96(LL), FX_EB + kl)) * fc.inv180dx2;
+            const double ls = ANISO ? fx_to_double(LSs, FX_EB64 + 6 + ks)
+                                    : fx_to_double(fx_wide96(LS), FX_EB + ks);
+            const double ll = ANISO ? fx_to_double(LLs, FX_EB64 + 6 + kl)
+                                    : fx_to_double(fx_wide96(LL), FX_EB + kl);
+            const double lapxi = (a.k.gamma_cp * ls + a.k.gm1 * ll) * fc.inv180dx2;
             const double ss2 = fx_to_double(fx_dot3(SS, SS), FX_EB + 36 + 2 * ks);
             const double sl2 = fx_to_double(fx_dot3(SS, SL), FX_EB + 36 + ks + kl);
             const double ll2 = fx_to_double(fx_dot3(SL, SL), FX_EB + 36 + 2 * kl);
@@ -1028,7 +1113,8 @@ __device__ __forceinline__ void fx_march_a(const SubstepArgs<double, double> &a,
                               fx_to_double(fx_det2(U[0], B[1], U[1], B[0]), eu)};
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            const double la = fx_to_double(fx_wide96(LA[q]), FX_EB + ka);
+            const double la = ANISO ? fx_to_double(Ls[q], FX_EB64 + 6 + ka)
+                                    : fx_to_double(fx_wide96(LA[q]), FX_EB + ka);
             fx_update(a, active, 5 + q, o, f0[q], w0[q], fma(fc.c1dt, ub[q], fc.eta180 * la));
         }
         if (CFL && active) {
@@ -1064,7 +1150,7 @@ __device__ __forceinline__ void fx_march_a(const SubstepArgs<double, double> &a,
 }
 
 // The other half: the equations of ln rho, u and s.
-template <bool EXT>
+template <bool EXT, bool ANISO>
 __device__ __forceinline__ void fx_march_u(const SubstepArgs<double, double> &a, const FxCoefs &fc,
                                            const FxPlan *plan, const double *xch, FxMarch &m, int i, int j) {
     const bool active = i < a.g.nx && j < a.g.ny;
@@ -1093,11 +1179,12 @@ __device__ __forceinline__ void fx_march_u(const SubstepArgs<double, double> &a,
         }
         long long GL[3], GU[3][3], u0[3];
         FxWide V[3] = {}, LU[3];
+        long long GDs[3] = {0, 0, 0}, LUs[3];  // unequal spacing: over 2^8 and 2^6
         {
             const FxView Fl{ring, m.slot};
             const FxAxis l[3] = {fx_axis<0>(Fl), fx_axis<1>(Fl), fx_axis<2>(Fl)};
 #pragma unroll
-            for (int q = 0; q < 3; ++q) GL[q] = l[q].d >> 2;
+            for (int q = 0; q < 3; ++q) GL[q] = fx_first<ANISO>(l[q].d >> 2, fc, q);
         }
         {
             const FxView Fx{ring + FX_FIELD_TILE, m.slot}, Fy{ring + 2 * FX_FIELD_TILE, m.slot},
@@ -1105,9 +1192,15 @@ __device__ __forceinline__ void fx_march_u(const SubstepArgs<double, double> &a,
             u0[0] = Fx(0, 0, 0);
             u0[1] = Fy(0, 0, 0);
             u0[2] = Fz(0, 0, 0);
-            fx_u_component<0, EXT>(Fx, u0[0], V, GU[0], LU[0]);
-            fx_u_component<1, EXT>(Fy, u0[1], V, GU[1], LU[1]);
-            fx_u_component<2, EXT>(Fz, u0[2], V, GU[2], LU[2]);
+            if constexpr (ANISO) {
+                fx_u_component_scaled<0>(Fx, u0[0], fc, GDs, GU[0], LUs[0]);
+                fx_u_component_scaled<1>(Fy, u0[1], fc, GDs, GU[1], LUs[1]);
+                fx_u_component_scaled<2>(Fz, u0[2], fc, GDs, GU[2], LUs[2]);
+            } else {
+                fx_u_component<0, EXT>(Fx, u0[0], V, GU[0], LU[0]);
+                fx_u_component<1, EXT>(Fy, u0[1], V, GU[1], LU[1]);
+                fx_u_component<2, EXT>(Fz, u0[2], V, GU[2], LU[2]);
+            }
         }
         m.refill(z);
         FxSplit U[3], SL[3];
@@ -1130,8 +1223,14 @@ __device__ __forceinline__ void fx_march_u(const SubstepArgs<double, double> &a,
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
             const FxSplit g[3] = {fx_split(GU[q][0]), fx_split(GU[q][1]), fx_split(GU[q][2])};
-            const double v = fc.nu2160 * fx_to_double(fx_wide96(V[q]), FX_EB + ku);
-            ru[q] = EXT ? fma(fc.nu180, fx_to_double(fx_wide96(LU[q]), FX_EB + ku), v) : v;
+            if (ANISO)
+                ru[q] = fma(fc.nu180, fx_to_double(LUs[q], FX_EB64 + 6 + ku),
+                            fc.nu2160 * fx_to_double(GDs[q], FX_EB64 + 8 + ku));
+            else if (EXT)
+                ru[q] = fma(fc.nu180, fx_to_double(fx_wide96(LU[q]), FX_EB + ku),
+                            fc.nu2160 * fx_to_double(fx_wide96(V[q]), FX_EB + ku));
+            else
+                ru[q] = fc.nu2160 * fx_to_double(fx_wide96(V[q]), FX_EB + ku);
             ru[q] = fma(-fc.c1dt, fx_to_double(fx_dot3(U, g), FX_EB + 34 + 2 * ku), ru[q]);
             ru[q] = fma(fc.amp_dt[q], cph, ru[q]);
         }
@@ -1176,7 +1275,7 @@ __device__ __forceinline__ void fx_march_u(const SubstepArgs<double, double> &a,
     }
 }
 
-template <bool CFL, bool EXT = false>
+template <bool CFL, bool EXT, bool ANISO>
 __global__ void __launch_bounds__(2 * FXT * FXT, 1)
     substep_fx_kernel(const SubstepArgs<double, double> a, const __grid_constant__ CUtensorMap map,
                       const FxCoefs fc, FxPlan *plan) {
@@ -1223,9 +1322,9 @@ __global__ void __launch_bounds__(2 * FXT * FXT, 1)
     const int i = m.x0 + threadIdx.x, j = m.y0 + threadIdx.y;
     if (m.ok) {
         if (threadIdx.z)
-            fx_march_a<CFL, EXT>(a, fc, plan, etab, xch, m, i, j, cfl);
+            fx_march_a<CFL, EXT, ANISO>(a, fc, plan, etab, xch, m, i, j, cfl);
         else
-            fx_march_u<EXT>(a, fc, plan, xch, m, i, j);
+            fx_march_u<EXT, ANISO>(a, fc, plan, xch, m, i, j);
     }
     if (!m.ok) {  // report, and let no copy be in flight when the CTA ends
         atomicExch(&plan->err, 1);

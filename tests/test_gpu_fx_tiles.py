@@ -1,4 +1,4 @@
-"""The tiled integer-product substep (binary64, equal spacing) where it can go wrong:
+"""The tiled integer-product substep (binary64) where it can go wrong:
 grids against the edges of its 16 x 16 tiles and of its z march, states against the
 edges of the ranges its fixed point is sized for.  Each substep runs from the GPU's
 own previous state and is compared with the FP64 oracle at 1e-12 relative per field
@@ -124,3 +124,70 @@ def test_thermodynamic_range(lnrho, ss):
     f[0] += lnrho
     f[4] += ss
     _parity(N, f, phys=dict(PHYS, cs0=math.exp(-0.5 * (1.4 * ss / 1.3 + 0.4 * lnrho))))
+
+
+# unequal spacings on grids large enough for the integer form (16384 cells), ragged
+# against the tiles; the ratios of the spacings up to 8, either way
+UNEQUAL = [((33, 32, 17), (1.0, 1.5, 0.7)), ((17, 31, 33), (8.0, 1.0, 1.0)),
+           ((16, 1, 1100), (1.0, 3.0, 2.0)), ((26, 26, 26), (1.0, 1.0, 8.0)),
+           ((48, 40, 9), (1.0, 1.0 + 2.0 ** -50, 1.0))]
+
+
+def _unequal(n, hs, f, mode, **terms):
+    L = tuple(0.25 * h * v for v, h in zip(n, hs))
+    sim = ac.Simulation(n, L=L, force_amp=0.05, seed=3, **PHYS, **terms)
+    ac.ac_set_stencil_mode(sim.h, mode)
+    sim.load(f)
+    out = []
+    for s in range(3):
+        sim.substep(1e-3, s)
+        out.append((sim.store(), sim.store_w()))
+    cfl = ac.ac_last_cfl(sim.h)
+    sim.close()
+    return L, out, cfl
+
+
+@pytest.mark.parametrize("n,hs", UNEQUAL)
+@pytest.mark.parametrize("entropy", [False, True])
+def test_unequal_spacing(n, hs, entropy):
+    """The default path scales each axis's integer numerators; every substep against the
+    oracle from the path's own previous state, and not the plain stencils' bits."""
+    terms = dict(K=1e-2, zeta=2e-2, heat=0.02, cool=0.01) if entropy else {}
+    f = _state(n, 51)
+    L, out, cfl = _unequal(n, hs, f, ac.AC_STENCIL_AUTO, **terms)
+    p = core.Params(n=n, L=L, forcing=core.forcing_draw(3, 0, 0.05), **PHYS, **terms)
+    c = core.reduce(f, p, "max", "cfl")
+    assert abs(cfl - c) <= 1e-12 * c
+    w = None
+    for s, (fg, wg) in enumerate(out):
+        fo, wo = core.substep(f, w, p, 1e-3, s)
+        assert np.all(rel_err(fg, fo) <= 1e-12), (s, rel_err(fg, fo))
+        assert np.all(rel_err(wg, wo) <= 1e-12), (s, rel_err(wg, wo))
+        f, w = fg, wg
+    _, plain, _ = _unequal(n, hs, _state(n, 51), ac.AC_STENCIL_FP64, **terms)
+    assert not np.array_equal(plain[-1][1], out[-1][1])
+
+
+@pytest.mark.parametrize("case", ["small", "ratio", "range", "nan"])
+def test_unequal_spacing_left_to_the_plain_stencils(case):
+    """Few cells, spacings more than 8 apart, a state outside the ranges the fixed point
+    is sized for, a NaN: bit for bit what AC_STENCIL_FP64 computes."""
+    n, hs = ((15, 16, 17), (1.0, 1.5, 1.0)) if case == "small" else ((26, 26, 26), (1.0, 1.5, 1.0))
+    if case == "ratio":
+        hs = (1.0, 9.0, 1.0)
+    f = _state(n, 61)
+    if case == "range":
+        f[3] *= 1e-4
+    if case == "nan":
+        f[2][3, 4, 5] = np.nan
+    L, out, plain = None, [], []
+    for mode, dst in ((ac.AC_STENCIL_AUTO, out), (ac.AC_STENCIL_FP64, plain)):
+        L = tuple(0.25 * h * v for v, h in zip(n, hs))
+        sim = ac.Simulation(n, L=L, force_amp=0.05, seed=3, **PHYS)
+        ac.ac_set_stencil_mode(sim.h, mode)
+        sim.load(f)
+        sim.step(1e-3)
+        dst += [sim.store(), sim.store_w()]
+        sim.close()
+    for a, b in zip(out, plain):
+        assert np.array_equal(a, b, equal_nan=True)
