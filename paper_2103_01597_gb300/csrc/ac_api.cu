@@ -161,7 +161,9 @@ extern "C" int ac_init(ac_handle **out, const ac_grid *grid, const ac_params *pa
     const int ntab = grid->nx + grid->ny + grid->nz;
     cudaError_t e = cudaMalloc(&h->ftab, (size_t)ntab * (sizeof(double2) + sizeof(float2)));
     if (e == cudaSuccess) e = cudaMalloc(&h->partials, sizeof(double) * reduce_max_blocks());
-    if (e == cudaSuccess) e = cudaMalloc(&h->flags, sizeof(unsigned int) * reduce_max_blocks());
+    const size_t flag_bytes = sizeof(unsigned int) * (reduce_max_blocks() + 1);
+    if (e == cudaSuccess) e = cudaMalloc(&h->flags, flag_bytes);
+    if (e == cudaSuccess) e = cudaMemset(h->flags, 0, flag_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&h->result_dev, 2 * sizeof(double));
     if (e == cudaSuccess) e = cudaMallocHost(&h->result_host, 2 * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&h->cfl_dev, sizeof(unsigned long long));
@@ -902,13 +904,15 @@ extern "C" int ac_reduce(ac_handle *h, int op, int quantity, double *out) {
     L.partials = h->partials;
     L.flags = h->flags;
     L.result = h->result_dev;
+    L.host = h->result_host;
+    L.dx[0] = h->grid.lx / h->grid.nx;
+    L.dx[1] = h->grid.ly / h->grid.ny;
+    L.dx[2] = h->grid.lz / h->grid.nz;
     L.blocks = reduce_max_blocks();
     int nl = 0;
     cudaError_t e = launch_reduce(L, h->stream, &nl);
     h->launches += nl;
     if (e != cudaSuccess) return cuda_fail(e);
-    CK(cudaMemcpyAsync(h->result_host, h->result_dev, 2 * sizeof(double), cudaMemcpyDeviceToHost,
-                       h->stream));
     CK(cudaStreamSynchronize(h->stream));
     *out = h->result_host[0];
     unsigned int flag;

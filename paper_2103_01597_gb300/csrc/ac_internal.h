@@ -146,12 +146,14 @@ struct ReduceLaunch {
     int precision;
     Geom g;
     const void *f[NF];
+    double dx[3];
     StencilCoefs c;
     PhysConsts ph;
     int op, quantity;
     double *partials;      // scratch, >= reduce_max_blocks() doubles
-    unsigned int *flags;   // scratch, >= reduce_max_blocks() words (non-finite seen)
+    unsigned int *flags;   // scratch, reduce_max_blocks() + 1 words, the last one zero
     double *result;        // one double + one flag word after it (device)
+    double *host;          // the same in page-locked host memory, written by the kernel
     int blocks;
 };
 int reduce_max_blocks();

@@ -152,6 +152,26 @@ AC_HD long long fx_mulfrac(long long x, int rh, int rl) {
     return 2 * ((long long)s.hi * rh + (cr >> 31));
 }
 
+// r in (0, 1] as hi 2^-31 + lo 2^-62 (1 as 1 - 2^-62).
+inline void fx_fraction(double r, int *hi, int *lo) {
+    *hi = *lo = 0x7fffffff;
+    if (r < 1.0) {
+        const double t = r * 2147483648.0;
+        *hi = (int)t;
+        *lo = (int)((t - (double)*hi) * 2147483648.0);
+    }
+}
+
+// The normal binary64 with bits b in units of 2^(E - 1078), E at least its biased
+// exponent: magnitude below 2^56 (truncated).  A zero or subnormal b gives 0 for E > 62.
+AC_HD long long fx_align(long long b, int E) {
+    const int e = (int)((b >> 52) & 0x7ff);
+    const fx_u64 m = ((fx_u64)b & 0xfffffffffffffull) | 0x10000000000000ull;
+    const int d = E - e;
+    const long long x = (long long)((m << 3) >> (d > 63 ? 63 : d)), s = b >> 63;
+    return (x ^ s) - s;
+}
+
 // ---- conversion -------------------------------------------------------------------
 // v 2^e as binary64, rounded to nearest from the top 64 significant bits (a
 // negative value is first replaced by its one's complement: half a unit of the

@@ -299,7 +299,9 @@ extern "C" int ac_batch_init(ac_batch **out, int nbox, const ac_box *boxes, cons
     if (e == cudaSuccess) e = cudaMemsetAsync(b->block, 0, 2 * fbytes + wbytes, b->stream);
     if (e == cudaSuccess) e = cudaMalloc(&b->counter, sizeof(unsigned int));
     if (e == cudaSuccess) e = cudaMalloc(&b->partials, sizeof(double) * reduce_max_blocks());
-    if (e == cudaSuccess) e = cudaMalloc(&b->flags, sizeof(unsigned int) * reduce_max_blocks());
+    const size_t flag_bytes = sizeof(unsigned int) * (reduce_max_blocks() + 1);
+    if (e == cudaSuccess) e = cudaMalloc(&b->flags, flag_bytes);
+    if (e == cudaSuccess) e = cudaMemset(b->flags, 0, flag_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&b->result_dev, 2 * sizeof(double));
     if (e == cudaSuccess) e = cudaMallocHost(&b->result_host, 2 * sizeof(double));
     int dev = 0, sms = 152, occ = 1;
@@ -762,12 +764,12 @@ extern "C" int ac_batch_reduce(ac_batch *b, int box, int op, int quantity, doubl
     L.partials = b->partials;
     L.flags = b->flags;
     L.result = b->result_dev;
+    L.host = b->result_host;
+    for (int a = 0; a < 3; ++a) L.dx[a] = dx[a];
     L.blocks = reduce_max_blocks();
     int nl = 0;
     BCK(launch_reduce(L, b->stream, &nl));
     b->launches += nl;
-    BCK(cudaMemcpyAsync(b->result_host, b->result_dev, 2 * sizeof(double), cudaMemcpyDeviceToHost,
-                        b->stream));
     BCK(cudaStreamSynchronize(b->stream));
     *out = b->result_host[0];
     unsigned int flag;

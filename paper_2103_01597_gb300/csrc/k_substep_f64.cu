@@ -31,16 +31,6 @@ static int fx_zchunk(long long tiles, int nz) {
     return best;
 }
 
-// r in (0, 1] as hi 2^-31 + lo 2^-62 (1 as 1 - 2^-62).
-static void fx_fraction(double r, int *hi, int *lo) {
-    *hi = *lo = 0x7fffffff;
-    if (r < 1.0) {
-        const double t = r * 2147483648.0;
-        *hi = (int)t;
-        *lo = (int)((t - (double)*hi) * 2147483648.0);
-    }
-}
-
 // Padded row length (even: the strides of the tensor map are multiples of 16 bytes),
 // bytes of the eight padded int64 arrays, and the tensor map over them: dims (px,
 // py, pz, field), box one plane of a tile with its halo, all fields.
