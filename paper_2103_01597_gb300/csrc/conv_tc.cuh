@@ -18,11 +18,12 @@
 //
 // An output tile is 128 cells of one x-row (GEMM M = 128) for all output
 // channels (N = COUT, padded to 16); K = 27 taps x CIN.  Warp roles in a
-// persistent CTA: warp 4 (one thread) issues the TMA copies of z-slices
-// (rows y-1, y, y+1 of one plane) into a six-slice ring; warp 5 (one thread)
-// issues the MMAs of each tile into one of two TMEM accumulators and signals
-// completion with tcgen05.commit; warps 0-3 read an accumulator back
-// (tcgen05.ld, one TMEM lane per thread), add the bias, apply ReLU and store.
+// persistent CTA: two producer warps (one thread each) issue the TMA copies of
+// z-slices (rows y-1, y, y+1 of one plane) into a ring of slice groups; one warp
+// (one thread) issues the MMAs of each tile into one of sixteen TMEM accumulators
+// and signals completion with tcgen05.commit; two sets of four warps read an
+// accumulator back (tcgen05.ld, one TMEM lane per thread), add the bias, apply
+// ReLU and store.
 // A CTA marches along z through column segments, so each staged slice serves
 // three tiles.  Every wait is bounded: on timeout a role records an error
 // word and stops, the others run out of their own bounded waits, and TMEM is
@@ -42,10 +43,21 @@ using bf16 = __nv_bfloat16;
 
 constexpr int TM = 128;          // cells per tile (GEMM M)
 constexpr int THREADS = 192;     // warps 0-3 epilogue (one TMEM lane quadrant each), 4 TMA, 5 MMA
+// conv_tc_kernel: ESETS sets of four epilogue warps and PRODS TMA warps, each taking tiles
+// or groups of slices in turn, then the MMA warp
+constexpr int ESETS = 2;
+constexpr int PRODS = 2;
+constexpr int CTHREADS = 32 * (4 * ESETS + PRODS + 1);
 constexpr int CORE = 128;        // bytes of one core matrix (8 rows x 16 B)
 constexpr int PCELLS = TM + 8;          // cells of a staged plane (130 used)
 constexpr int PLANE = PCELLS * 16;      // bytes of one staged 8-channel plane
-constexpr int NBUF = 6;          // z-slices in the shared-memory ring
+constexpr int PGROUP = 3;        // slices the paired kernel's issuer waits for at once
+// Shared-memory ring of conv_tc_kernel: ring_groups groups of GROUP z-slices, a group
+// being what one barrier announces and one wait covers.  Two groups of 32-channel
+// slices fill the memory beside the weights; a slice of 8 channels is over in a
+// quarter of the time, so more of them are in flight.
+constexpr int GROUP = 3;
+__host__ __device__ constexpr int ring_groups(int cin) { return cin == 8 ? 4 : 2; }
 // Bounds of every wait, set by time: a try_wait poll of a phase that does not
 // complete returns after about 3.8 us (measured on GB300), so 2^18 polls give
 // up after about one second; a round of non-blocking tests takes well under a
@@ -190,6 +202,54 @@ __device__ __forceinline__ void mma_bf16_elect(uint32_t tmem_d, uint64_t adesc, 
         : "memory");
 }
 
+// Runs of MMAs into one accumulator window under one election: number I + k of a
+// slice's schedule S takes the operands a0 + S::a(I + k), b0 + S::b(I + k), offsets
+// known when compiled.
+template <class S, int I>
+__device__ __forceinline__ void mma_run5_elect(uint32_t tmem_d, uint64_t a0, uint64_t b0, uint32_t idesc) {
+    asm volatile(
+        "{\n .reg .pred p, e;\n .reg .b32 r;\n .reg .b64 x, y;\n"
+        " elect.sync r|e, 0xffffffff;\n"
+        " setp.ne.u32 p, 1, 0;\n"
+        " add.s64 x, %1, %4;\n add.s64 y, %2, %9;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, p;\n"
+        " add.s64 x, %1, %5;\n add.s64 y, %2, %10;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, p;\n"
+        " add.s64 x, %1, %6;\n add.s64 y, %2, %11;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, p;\n"
+        " add.s64 x, %1, %7;\n add.s64 y, %2, %12;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, p;\n"
+        " add.s64 x, %1, %8;\n add.s64 y, %2, %13;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, p;\n"
+        "}\n" ::"r"(tmem_d),
+        "l"(a0), "l"(b0), "r"(idesc), "n"(S::a(I + 0)), "n"(S::a(I + 1)), "n"(S::a(I + 2)), "n"(S::a(I + 3)), "n"(S::a(I + 4)),
+          "n"(S::b(I + 0)), "n"(S::b(I + 1)), "n"(S::b(I + 2)), "n"(S::b(I + 3)), "n"(S::b(I + 4))
+        : "memory");
+}
+template <class S, int I>
+__device__ __forceinline__ void mma_run6_elect(uint32_t tmem_d, uint64_t a0, uint64_t b0, uint32_t idesc) {
+    asm volatile(
+        "{\n .reg .pred p, e;\n .reg .b32 r;\n .reg .b64 x, y;\n"
+        " elect.sync r|e, 0xffffffff;\n"
+        " setp.ne.u32 p, 1, 0;\n"
+        " add.s64 x, %1, %4;\n add.s64 y, %2, %10;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, p;\n"
+        " add.s64 x, %1, %5;\n add.s64 y, %2, %11;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, p;\n"
+        " add.s64 x, %1, %6;\n add.s64 y, %2, %12;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, p;\n"
+        " add.s64 x, %1, %7;\n add.s64 y, %2, %13;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, p;\n"
+        " add.s64 x, %1, %8;\n add.s64 y, %2, %14;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, p;\n"
+        " add.s64 x, %1, %9;\n add.s64 y, %2, %15;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, p;\n"
+        "}\n" ::"r"(tmem_d),
+        "l"(a0), "l"(b0), "r"(idesc), "n"(S::a(I + 0)), "n"(S::a(I + 1)), "n"(S::a(I + 2)), "n"(S::a(I + 3)), "n"(S::a(I + 4)), "n"(S::a(I + 5)),
+          "n"(S::b(I + 0)), "n"(S::b(I + 1)), "n"(S::b(I + 2)), "n"(S::b(I + 3)), "n"(S::b(I + 4)), "n"(S::b(I + 5))
+        : "memory");
+}
+
 // Arrive on `bar` once all MMAs issued so far by this warp have completed (one
 // elected lane).
 __device__ __forceinline__ void mma_commit_elect(uint64_t *bar) {
@@ -263,6 +323,11 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(smem_u32(bar)) : "memory");
 }
 
+__device__ __forceinline__ void mbar_arrive_n(uint64_t *bar, unsigned count) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)), "r"(count)
+                 : "memory");
+}
+
 __device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(smem_u32(bar)),
                  "r"(bytes)
@@ -311,7 +376,7 @@ __host__ __device__ constexpr int w_bytes(int cin, int nb) {
 
 // Bytes of dynamic shared memory: the weight image and the slice ring.
 __host__ __device__ constexpr size_t smem_bytes(int cin, int nb) {
-    return (size_t)w_bytes(cin, nb) + (size_t)NBUF * 3 * row_bytes(cin);
+    return (size_t)w_bytes(cin, nb) + (size_t)ring_groups(cin) * GROUP * 3 * row_bytes(cin);
 }
 
 // Layers with 8 input channels fill the K = 16 of an MMA with two taps of one
@@ -374,8 +439,7 @@ __device__ __forceinline__ Segment segment_of(long long g, const ConvTcArgs &a, 
 
 // Persistent CTA g-loop over column segments b, b + G, ...  Slices are numbered
 // in the order the CTA stages them (a segment of L tiles stages L + 2: planes
-// z0-1 .. z0+L); slice s lives in ring buffer s % NBUF, as that buffer's
-// (s / NBUF)-th fill.
+// z0-1 .. z0+L), GROUP slices to a ring group; a segment's last group may hold fewer.
 //
 // One MMA batch per slice.  Slice j of a segment (plane z0 + j - 1) feeds the
 // tiles j-2, j-1, j of the segment that exist (dz = +1, 0, -1).  The weight
@@ -388,12 +452,25 @@ __device__ __forceinline__ Segment segment_of(long long g, const ConvTcArgs &a, 
 // accumulate, and blocks are zero when handed over: zeroed once at start and
 // again by the epilogue after it reads a tile.  Barriers, each waited on in
 // phase order:
-//   full[b]  : TMA bytes of a fill landed (producer expect_tx, TMA complete_tx);
-//   empty[b] : the MMAs reading a fill have finished (tcgen05.commit);
-//   accf[k]  : the tile in block k is complete (commit after its third slice);
-//   acce[k]  : the four epilogue warps have read and re-zeroed block k;
+//   full[b]  : TMA bytes of ring group b landed (producer expect_tx, TMA complete_tx);
+//   empty[b] : the MMAs reading ring group b have finished (tcgen05.commit);
+//   accf[k]  : the tile in block k is complete (commit after its third slice; one
+//              commit a group measured slower: the epilogues then come in bursts);
+//   acce[k]  : the epilogue warps have read and re-zeroed the GROUP blocks from GROUP k
+//              on (waited on by the producer, so that full[b] says it to the MMA warp);
 //   wbar     : the layer's weight image landed;
 //   fin      : every MMA of the CTA has finished (before TMEM is freed).
+//
+// What bounds it: the issuing threads.  An MMA of N = 96 takes about 52 cycles (its
+// operands' way out of shared memory) and 40 to issue, a wait for a barrier that is
+// already through 200, a commit 40 to 80, a copy's issue 80, and little of that is
+// hidden.  Hence one wait and one release for three slices, block hand-over by way of
+// the producer, two producers, two epilogue sets, and no division on these paths.
+// Measured at 256^3, before and after: layer 1 0.459 -> 0.271 ms (1.34 GB of
+// activations: 0.19 ms), layer 2 0.711 -> 0.573 ms (0.928 TFLOP: 0.495 ms at the
+// measured bfloat16 rate), layer 3 0.635 -> 0.481 ms.  Looking at the next group's
+// barriers ahead of time, one copy of all three rows, and two CTAs on an SM in layer
+// 3 measured slower.
 //
 // Weight image: w[(((kq * NGS + ng) * 8 + r) * 8 + c], NGS = 3 NB / 8, holds for
 // stack row 8 ng + r = (2 - kz) NB + co the weight W[co][ci][kz][dyx] (dyx =
@@ -401,14 +478,36 @@ __device__ __forceinline__ Segment segment_of(long long g, const ConvTcArgs &a, 
 // CIN = 8, kq = 2 p + h, dyx = pair_tap(p, h) and ci = c; zero for co >= COUT,
 // ci >= cin_real and the zero half of the last pair.
 constexpr int RBLK = 16;  // TMEM accumulator blocks per CTA (>= tiles per segment, <= 32)
-constexpr int GROUP = 3;  // slices the MMA issuer waits for at once (<= NBUF / 2)
+
+// The MMAs of one slice: what MMA i adds to the descriptors of the first core
+// matrices (start address / 16; with 8 input channels also the distance of the
+// second tap, as the leading-dimension field).
+template <int CIN, int NB>
+struct SliceMmas {
+    static constexpr int ROW = row_bytes(CIN), NGS = 3 * NB / 8;
+    static constexpr int N = CIN == 8 ? 5 : 9 * CIN / 16;
+    __host__ __device__ static constexpr long long a(int i) {
+        if (CIN == 8) {
+            const int t0 = pair_tap(i, 0), t1 = pair_tap(i, 1);
+            const int off = (t0 / 3) * ROW + (t0 % 3) * 16;
+            const int lbo = (t1 / 3) * ROW + (t1 % 3) * 16 - off;
+            return (off >> 4) + ((long long)(lbo >> 4) << 16);
+        }
+        constexpr int KK = CIN / 16 > 0 ? CIN / 16 : 1;
+        const int dyx = i / KK, kk = i % KK;
+        return ((dyx / 3) * ROW + (dyx % 3) * 16 + kk * 2 * PLANE) >> 4;
+    }
+    __host__ __device__ static constexpr long long b(int i) { return (2 * i * NGS * CORE) >> 4; }
+};
 
 template <int CIN, int COUT, int EPI>
-__global__ void __launch_bounds__(THREADS, 1)
+__global__ void __launch_bounds__(CTHREADS, 1)
     conv_tc_kernel(const __grid_constant__ CUtensorMap xmap, const ConvTcArgs a) {
     constexpr int NB = COUT < 16 ? 16 : COUT;  // accumulator columns per tile
     constexpr int KC = CIN / 8;                // core-matrix columns along K per tap
-    constexpr bool PAIR = CIN == 8;            // two taps per MMA
+    using Mmas = SliceMmas<CIN, NB>;
+    constexpr int NGRP = ring_groups(CIN);
+    constexpr int TGROUPS = (RBLK + GROUP - 1) / GROUP;  // groups of accumulator blocks
     constexpr int NGS = 3 * NB / 8;            // core-matrix rows of the kz stack
     constexpr int ROW = row_bytes(CIN);
     constexpr int SLICE = 3 * ROW;
@@ -417,7 +516,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     constexpr uint32_t TCOLS = RBLK * NB;      // 256 or 128 TMEM columns
     static_assert((CIN % 16 == 0 || CIN == 8) && COUT % 8 == 0 && COUT <= 32, "shape");
     extern __shared__ __align__(1024) unsigned char smem[];
-    __shared__ uint64_t full[NBUF], empty[NBUF], accf[RBLK], acce[RBLK], wbar, fin;
+    __shared__ uint64_t full[NGRP], empty[NGRP], accf[RBLK], acce[TGROUPS], wbar, fin;
     __shared__ uint32_t tmem_base;
     unsigned char *Ws = smem;
     unsigned char *Ss = smem + W_BYTES;
@@ -426,15 +525,13 @@ __global__ void __launch_bounds__(THREADS, 1)
     const long long nseg = (long long)((a.nz + a.zc - 1) / a.zc) * a.ny * segs;
 
     if (warp == 0) tmem_alloc(&tmem_base, TCOLS);
-    if (threadIdx.x == 128) {
-        for (int b = 0; b < NBUF; ++b) {
+    if (threadIdx.x == 128 * ESETS) {
+        for (int b = 0; b < NGRP; ++b) {
             mbar_init(&full[b], 1);
             mbar_init(&empty[b], 1);
         }
-        for (int b = 0; b < RBLK; ++b) {
-            mbar_init(&accf[b], 1);
-            mbar_init(&acce[b], 4);
-        }
+        for (int b = 0; b < RBLK; ++b) mbar_init(&accf[b], 1);
+        for (int b = 0; b < TGROUPS; ++b) mbar_init(&acce[b], 4 * GROUP);
         mbar_init(&wbar, 1);
         mbar_init(&fin, 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -449,112 +546,104 @@ __global__ void __launch_bounds__(THREADS, 1)
     __syncthreads();
     tc_fence_after_sync();
 
-    if (warp == 4) {
-        if (lane == 0) {  // ---- TMA producer
-            mbar_expect_tx(&wbar, W_BYTES);
-            bulk_load(Ws, a.w, W_BYTES, &wbar);
-            long long s = 0;
+    if (warp >= 4 * ESETS && warp < 4 * ESETS + PRODS) {
+        if (lane == 0) {  // ---- TMA producers: every PRODS-th ring group each
+            const int own = warp - 4 * ESETS;
+            static_assert(NGRP % PRODS == 0, "a ring group always has the same producer");
+            if (own == 0) {
+                mbar_expect_tx(&wbar, W_BYTES);
+                bulk_load(Ws, a.w, W_BYTES, &wbar);
+            }
+            int grp = 0;           // ring group of the next slices
+            unsigned round = 0;    // completed passes over the ring
+            uint32_t gpar = 0;     // bit k: parity of the times block group k has been opened
             bool ok = true;
             for (long long g = blockIdx.x; g < nseg && ok; g += gridDim.x) {
                 const Segment sg = segment_of(g, a, segs);
-                for (int j = 0; j < sg.len + 2; ++j, ++s) {
-                    const int b = (int)(s % NBUF);
-                    const long long k = s / NBUF;
-                    if (k > 0 && !mbar_wait(&empty[b], (unsigned)((k - 1) & 1))) {
-                        ok = false;
-                        break;
+                const int y0 = wrapi(sg.y - 1, a.ny), y2 = wrapi(sg.y + 1, a.ny);
+                const int x = sg.seg * (TM / 8);
+                int z = wrapi(sg.z0 - 1, a.nz);
+                for (int j = 0, k = 0; j < sg.len + 2; j += GROUP, ++k) {
+                    const int cnt = min(GROUP, sg.len + 2 - j);
+                    // the blocks this group's tiles open in (if any) have been read and zeroed
+                    // (waited for by every producer: a phase that one did not wait for
+                    // would make the next one's parity ambiguous)
+                    if (j < sg.len) ok = mbar_wait(&acce[k], ((gpar >> k) & 1u) ^ 1u);
+                    if (!ok) break;
+                    if (grp % PRODS == own) {
+                        if (round > 0) ok = mbar_wait(&empty[grp], (round - 1) & 1);
+                        if (!ok) break;
+                        mbar_expect_tx(&full[grp], cnt * SLICE_TX);
+                        for (int q = 0; q < cnt; ++q) {
+                            unsigned char *dst = Ss + (grp * GROUP + q) * SLICE;
+                            tma_load_5d(dst, &xmap, &full[grp], 0, x, 0, y0, z);
+                            tma_load_5d(dst + ROW, &xmap, &full[grp], 0, x, 0, sg.y, z);
+                            tma_load_5d(dst + 2 * ROW, &xmap, &full[grp], 0, x, 0, y2, z);
+                            z = z + 1 == a.nz ? 0 : z + 1;
+                        }
+                    } else {
+                        z += GROUP;
+                        if (z >= a.nz) z = wrapi(z, a.nz);
                     }
-                    mbar_expect_tx(&full[b], SLICE_TX);
-                    const int z = wrapi(sg.z0 + j - 1, a.nz);
-                    unsigned char *dst = Ss + b * SLICE;
-#pragma unroll
-                    for (int r = 0; r < 3; ++r)
-                        tma_load_5d(dst + r * ROW, &xmap, &full[b], 0, sg.seg * (TM / 8), 0,
-                                    wrapi(sg.y + r - 1, a.ny), z);
+                    if (j < sg.len) gpar ^= 1u << k;
+                    if (++grp == NGRP) {
+                        grp = 0;
+                        ++round;
+                    }
                 }
             }
             if (!ok) atomicExch(a.err, 1u);
-            // no copy may be in flight when the CTA exits: wait for each buffer's last fill
-            mbar_wait(&wbar, 0);
-            for (int b = 0; b < NBUF; ++b)
-                if (s > b) mbar_wait(&full[b], (unsigned)(((s - 1 - b) / NBUF) & 1));
+            // no copy may be in flight when the CTA exits: wait for each group's last fill
+            if (own == 0) mbar_wait(&wbar, 0);
+            for (int q = own; q < NGRP; q += PRODS) {
+                const unsigned fills = round + (q < grp);
+                if (fills) mbar_wait(&full[q], (fills - 1) & 1);
+            }
         }
-    } else if (warp == 5) {
+    } else if (warp == 4 * ESETS + PRODS) {
         {  // ---- MMA issuer: the whole warp runs the loop, one elected lane issues
-            static_assert(GROUP == 3, "the combined wait tests six barriers");
             bool ok = __all_sync(0xffffffffu, mbar_wait(&wbar, 0));
-            long long s = 0;  // slices consumed
-            // per TMEM block: bit k of `used` = block k has held a tile, bit k of
-            // `par` = parity of the number of tiles it has held (registers, not an
-            // indexed array: local memory would sit on the issue path)
-            uint32_t used = 0, par = 0;
-            const uint32_t wbase = smem_u32(Ws);
+            int grp = 0;  // ring group of the next slices, and the parity of its fill
+            unsigned fill = 0;
+            // descriptors of the first operands: every other MMA adds byte offsets / 16
+            // to the start-address field
+            const uint64_t a_ring = smem_desc(smem_u32(Ss), CIN == 8 ? 0 : PLANE, CORE);
+            const uint64_t b_stack = smem_desc(smem_u32(Ws), NGS * CORE, CORE);
+            constexpr uint32_t STACK = (NB / 8) * CORE >> 4;  // one kz block of the stack
             for (long long g = blockIdx.x; g < nseg && ok; g += gridDim.x) {
-                const Segment sg = segment_of(g, a, segs);
-                const int L = sg.len;
-                for (int j = 0; j < L + 2; ++j, ++s) {
-                    const int b = (int)(s % NBUF);
-                    if (j % GROUP == 0) {
-                        // one combined wait for the next GROUP slices: each landed,
-                        // and each tile they open has been read out of its block
-                        uint32_t addr[2 * GROUP];
-                        unsigned want[2 * GROUP];
-                        uint32_t pending = 0;
+                const int L = segment_of(g, a, segs).len;
+                for (int j = 0; j < L + 2; j += GROUP) {
+                    // the group's slices have landed, and with them (the producer saw it
+                    // before it sent them) the blocks they open are zero
+                    ok = __all_sync(0xffffffffu, mbar_wait(&full[grp], fill));
+                    if (!ok) break;
+                    tc_fence_after_sync();
+                    uint64_t a0 = a_ring + (uint32_t)(grp * (GROUP * SLICE >> 4));
 #pragma unroll
-                        for (int q = 0; q < GROUP; ++q) {
-                            const long long sq = s + q;
-                            const int jq = j + q;
-                            addr[2 * q] = smem_u32(&full[sq % NBUF]);
-                            want[2 * q] = (unsigned)((sq / NBUF) & 1);
-                            addr[2 * q + 1] = smem_u32(&acce[jq < RBLK ? jq : 0]);
-                            want[2 * q + 1] = ((par >> jq) & 1u) ^ 1u;
-                            if (jq < L + 2) pending |= 1u << (2 * q);
-                            if (jq < L && ((used >> jq) & 1u)) pending |= 1u << (2 * q + 1);
+                    for (int q = 0; q < GROUP; ++q, a0 += SLICE >> 4) {
+                        const int jq = j + q;
+                        if (jq >= L + 2) break;
+                        // tiles ta .. tb, from kz block ta - jq + 2 of the stack
+                        const int ta = jq > 2 ? jq - 2 : 0;
+                        const int tb = jq < L ? jq : L - 1;
+                        const uint32_t dtm = tmem + (uint32_t)(ta * NB);
+                        const uint64_t b0 = b_stack + (uint32_t)(ta - jq + 2) * STACK;
+                        const uint32_t idesc = idesc_bf16(TM, (tb - ta + 1) * NB);
+                        if constexpr (CIN == 8) {
+                            mma_run5_elect<Mmas, 0>(dtm, a0, b0, idesc);
+                        } else {
+                            static_assert(CIN == 8 || Mmas::N == 18, "three runs of six");
+                            mma_run6_elect<Mmas, 0>(dtm, a0, b0, idesc);
+                            mma_run6_elect<Mmas, 6>(dtm, a0, b0, idesc);
+                            mma_run6_elect<Mmas, 12>(dtm, a0, b0, idesc);
                         }
-                        ok = mbar_wait6_warp(addr, want, pending);
-                        if (!ok) break;
-                        tc_fence_after_sync();
+                        if (jq >= 2) mma_commit_elect(&accf[jq - 2]);  // its third slice is in
                     }
-                    if (j < L) {  // tile j opens in block j
-                        used |= 1u << j;
-                        par ^= 1u << j;
+                    mma_commit_elect(&empty[grp]);
+                    if (++grp == NGRP) {
+                        grp = 0;
+                        fill ^= 1u;
                     }
-                    const int ta = j - 2 > 0 ? j - 2 : 0;
-                    const int tb = j < L - 1 ? j : L - 1;
-                    const uint32_t sbase = smem_u32(Ss + b * SLICE);
-                    const uint32_t dtm = tmem + (uint32_t)(ta * NB);
-                    const int stack0 = ta - j + 2;  // kz block of the first tile
-                    const uint32_t idesc = idesc_bf16(TM, (tb - ta + 1) * NB);
-                    // descriptors of the first operands; every other MMA adds a
-                    // compile-time byte offset / 16 to the start-address field
-                    const uint64_t b0 = smem_desc(wbase + stack0 * (NB / 8) * CORE, NGS * CORE, CORE);
-                    if constexpr (PAIR) {
-                        const uint64_t a0 = smem_desc(sbase, 0, CORE);
-#pragma unroll
-                        for (int p = 0; p < 5; ++p) {
-                            const int ta0 = pair_tap(p, 0), tb0 = pair_tap(p, 1);
-                            const uint32_t off = (ta0 / 3) * ROW + (ta0 % 3) * 16;
-                            const uint32_t lbo = (tb0 / 3) * ROW + (tb0 % 3) * 16 - off;
-                            const uint64_t ad = a0 + (off >> 4) + ((uint64_t)(lbo >> 4) << 16);
-                            const uint64_t bd = b0 + ((2 * p * NGS * CORE) >> 4);
-                            mma_bf16_elect(dtm, ad, bd, idesc);
-                        }
-                    } else {
-                        const uint64_t a0 = smem_desc(sbase, PLANE, CORE);
-#pragma unroll
-                        for (int dy = 0; dy < 3; ++dy)
-#pragma unroll
-                            for (int dx = 0; dx < 3; ++dx)
-#pragma unroll
-                                for (int kk = 0; kk < CIN / 16; ++kk) {
-                                    const int dyx = dy * 3 + dx;
-                                    const uint64_t ad = a0 + ((dy * ROW + dx * 16 + kk * 2 * PLANE) >> 4);
-                                    const uint64_t bd = b0 + (((dyx * KC + 2 * kk) * NGS * CORE) >> 4);
-                                    mma_bf16_elect(dtm, ad, bd, idesc);
-                                }
-                    }
-                    mma_commit_elect(&empty[b]);
-                    if (j >= 2) mma_commit_elect(&accf[j - 2]);  // tile j-2 has had its third slice
                 }
             }
             if (!ok && lane == 0) atomicExch(a.err, 1u);
@@ -562,7 +651,8 @@ __global__ void __launch_bounds__(THREADS, 1)
             mma_commit_elect(&fin);
             mbar_wait(&fin, 0);
         }
-    } else {  // ---- epilogue: warps 0-3, TMEM lanes 32 warp .. 32 warp + 31
+    } else {  // ---- epilogue: set = warp / 4 takes every ESETS-th block; TMEM lanes 32 quad ..
+        const int quad = warp & 3, set = warp >> 2;
         float bias[COUT];
 #pragma unroll
         for (int c = 0; c < COUT; ++c) bias[c] = EPI == EPI_MASK_BF16 ? 0.f : a.bias[c];
@@ -585,22 +675,30 @@ __global__ void __launch_bounds__(THREADS, 1)
                 }
             }
         };
-        auto load_mask_seg = [&](long long g) {  // first tile of segment g
-            if (g >= nseg) return;
-            const Segment s2 = segment_of(g, a, segs);
-            load_mask(s2.y, s2.seg * TM + warp * 32 + lane, s2.z0, mnext);
+        // the mask of the set's next tile after tile i of segment g
+        auto load_mask_ahead = [&](long long g, const Segment &s1, int i) {
+            if (EPI != EPI_MASK_BF16) return;
+            Segment s2 = s1;
+            for (i += ESETS; i >= s2.len; i = set) {
+                g += gridDim.x;
+                if (g >= nseg) return;
+                s2 = segment_of(g, a, segs);
+            }
+            load_mask(s2.y, s2.seg * TM + quad * 32 + lane, s2.z0 + i, mnext);
         };
-        load_mask_seg(blockIdx.x);
+        if (blockIdx.x < nseg)
+            load_mask_ahead(blockIdx.x, segment_of(blockIdx.x, a, segs), set - ESETS);
         for (long long g = blockIdx.x; g < nseg && ok; g += gridDim.x) {
             const Segment sg = segment_of(g, a, segs);
-            const int x = sg.seg * TM + warp * 32 + lane;
-            for (int i = 0; i < sg.len; ++i) {
-                const int kb = i;
-                ok = __all_sync(0xffffffffu, mbar_wait(&accf[kb], (par >> kb) & 1u));
-                par ^= 1u << kb;
+            const int x = sg.seg * TM + quad * 32 + lane;
+            // (a block is always the same set's: a phase that a set did not wait for
+            // would make the next one's parity ambiguous)
+            for (int i = set; i < sg.len; i += ESETS) {
+                ok = __all_sync(0xffffffffu, mbar_wait(&accf[i], (par >> i) & 1u));
                 if (!ok) break;
+                par ^= 1u << i;
                 tc_fence_after_sync();
-                const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(kb * NB);
+                const uint32_t taddr = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(i * NB);
                 float v[NB];
                 if constexpr (NB == 32)
                     tmem_ld32(taddr, v);
@@ -609,16 +707,13 @@ __global__ void __launch_bounds__(THREADS, 1)
                 tmem_zero<NB>(taddr);
                 tc_fence_before_sync();
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&acce[kb]);
+                // (the last tile also arrives for the blocks of its group without a tile)
+                if (lane == 0)
+                    mbar_arrive_n(&acce[i / GROUP], i == sg.len - 1 ? GROUP - i % GROUP : 1);
                 uint4 mcur[MK];
 #pragma unroll
                 for (int kc = 0; kc < MK; ++kc) mcur[kc] = mnext[kc];
-                if (EPI == EPI_MASK_BF16) {
-                    if (i + 1 < sg.len)
-                        load_mask(sg.y, x, sg.z0 + i + 1, mnext);
-                    else
-                        load_mask_seg(g + gridDim.x);
-                }
+                load_mask_ahead(g, sg, i);
                 if (x >= a.nx) continue;
                 const int z = sg.z0 + i;
                 if (EPI == EPI_RELU_BF16 || EPI == EPI_MASK_BF16) {
@@ -791,6 +886,7 @@ __device__ __forceinline__ PairSegment pair_segment_of(long long h, const ConvTc
 
 // Shared memory of one CTA of a pair: its half of the weight image and the ring.
 constexpr int PNBUF = 6;
+static_assert(PGROUP <= PNBUF / 2, "a wait leaves half the ring in flight");
 __host__ __device__ constexpr size_t pair_smem_bytes(int cin) {
     return (size_t)w_bytes(cin, 32) / 2 + (size_t)PNBUF * 3 * row_bytes(cin);
 }
@@ -898,7 +994,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
         }
     } else if (warp == 5) {
         if (leader) {  // ---- MMA issuer: the leader's whole warp, one elected lane issues
-            static_assert(GROUP == 3, "the combined wait tests six barriers");
+            static_assert(PGROUP == 3, "the combined wait tests six barriers");
             bool ok = true;
             long long s = 0;
             // bit k of `used`: block k has held a tile; bit k of `par`: parity of their count
@@ -907,12 +1003,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
             for (long long h = pair0; h < nseg && ok; h += npairs) {
                 for (int j = 0; j < L + 2; ++j, ++s) {
                     const int b = (int)(s % PNBUF);
-                    if (j % GROUP == 0) {
-                        uint32_t addr[2 * GROUP];
-                        unsigned want[2 * GROUP];
+                    if (j % PGROUP == 0) {
+                        uint32_t addr[2 * PGROUP];
+                        unsigned want[2 * PGROUP];
                         uint32_t pending = 0;
 #pragma unroll
-                        for (int q = 0; q < GROUP; ++q) {
+                        for (int q = 0; q < PGROUP; ++q) {
                             const long long sq = s + q;
                             const int jq = j + q;
                             const int kq = jq < L ? jq + 2 : 0;  // block tile jq opens

@@ -731,7 +731,7 @@ static cudaError_t tc_grid_for(const ac_closure *c, int sms, int *grid) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
     int per_sm = 0;
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, tc::THREADS, bytes);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, tc::CTHREADS, bytes);
     if (e != cudaSuccess) return e;
     // an SM's 512 TMEM columns bound the resident CTAs too (each allocates RBLK blocks)
     const int tcols = tc::RBLK * (COUT < 16 ? 16 : COUT);
@@ -1068,7 +1068,7 @@ static void launch_tc(const ac_closure *c, int layer, bool pair, const bf16 *img
         return;
     }
     tc::conv_tc_kernel<CIN, COUT, EPI>
-        <<<c->tc_grid[layer], tc::THREADS, tc::smem_bytes(CIN, COUT < 16 ? 16 : COUT), c->stream>>>(
+        <<<c->tc_grid[layer], tc::CTHREADS, tc::smem_bytes(CIN, COUT < 16 ? 16 : COUT), c->stream>>>(
             c->tc_map[layer], a);
 }
 
@@ -1323,7 +1323,7 @@ static void launch_mask(const ac_closure *c, const CUtensorMap &xmap, int grid, 
     a.zc = c->tc_zc;
     a.err = c->tc_err;
     tc::conv_tc_kernel<CIN, 32, tc::EPI_MASK_BF16>
-        <<<grid, tc::THREADS, tc::smem_bytes(CIN, 32), c->stream>>>(xmap, a);
+        <<<grid, tc::CTHREADS, tc::smem_bytes(CIN, 32), c->stream>>>(xmap, a);
 }
 
 template <int CIN, int COUT>
