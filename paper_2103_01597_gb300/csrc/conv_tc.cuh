@@ -404,6 +404,8 @@ struct ConvTcArgs {
     const float *bias;    // [COUT] (not read by EPI_MASK_BF16)
     bf16 *y;              // EPI_RELU_BF16, EPI_MASK_BF16: row-planar output (or null)
     const bf16 *mask;     // EPI_MASK_BF16: row-planar forward activation (COUT channels)
+    double *bpart;        // EPI_MASK_BF16: sums of the output per channel and epilogue warp,
+                          // [COUT / 8][4 ESETS gridDim.x][8]
     float *out[8];        // EPI_SCALED_F32: channel c to out[c][cell]
     const float *out_scale;        // EPI_SCALED_F32: [8]
     unsigned long long *gmax;      // EPI_SCALED_F32: guard word (binary64 bits), or null
@@ -686,6 +688,34 @@ __global__ void __launch_bounds__(CTHREADS, 1)
             }
             load_mask(s2.y, s2.seg * TM + quad * 32 + lane, s2.z0 + i, mnext);
         };
+        // EPI_MASK_BF16: the bias gradient, the sums over cells of what is written.  A
+        // thread adds its cell's COUT channels in binary32 for BTILES tiles, then the
+        // warp adds its lanes in a tree, after which lane c holds channel c and goes on
+        // in binary64.  (As a kernel of its own that read the 134 MB of a 128^3 layer
+        // back: 41 us; here the layer takes as long as without.)
+        constexpr int BTILES = 16;
+        constexpr int BS = EPI == EPI_MASK_BF16 ? COUT : 1;
+        static_assert(EPI != EPI_MASK_BF16 || COUT == 32, "a channel per lane");
+        float bs[BS];
+#pragma unroll
+        for (int c = 0; c < BS; ++c) bs[c] = 0.f;
+        double btotal = 0.0;
+        int btiles = 0;
+        auto fold_bias = [&]() {
+            if constexpr (EPI == EPI_MASK_BF16) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                    for (int i = 0; i < o; ++i) {
+                        const bool up = lane & o;
+                        const float other = __shfl_xor_sync(0xffffffffu, up ? bs[i] : bs[i + o], o);
+                        bs[i] = (up ? bs[i + o] : bs[i]) + other;
+                    }
+                btotal += (double)bs[0];
+#pragma unroll
+                for (int c = 0; c < BS; ++c) bs[c] = 0.f;
+            }
+        };
         if (blockIdx.x < nseg)
             load_mask_ahead(blockIdx.x, segment_of(blockIdx.x, a, segs), set - ESETS);
         for (long long g = blockIdx.x; g < nseg && ok; g += gridDim.x) {
@@ -714,6 +744,10 @@ __global__ void __launch_bounds__(CTHREADS, 1)
 #pragma unroll
                 for (int kc = 0; kc < MK; ++kc) mcur[kc] = mnext[kc];
                 load_mask_ahead(g, sg, i);
+                if (EPI == EPI_MASK_BF16 && ++btiles > BTILES) {
+                    fold_bias();
+                    btiles = 1;
+                }
                 if (x >= a.nx) continue;
                 const int z = sg.z0 + i;
                 if (EPI == EPI_RELU_BF16 || EPI == EPI_MASK_BF16) {
@@ -732,6 +766,8 @@ __global__ void __launch_bounds__(CTHREADS, 1)
                                 o[8 * kc + c] = __bfloat162float(m[c]) > 0.f
                                                     ? __float2bfloat16_rn(v[8 * kc + c])
                                                     : __float2bfloat16_rn(0.f);
+#pragma unroll
+                            for (int c = 0; c < 8; ++c) bs[8 * kc + c] += __bfloat162float(o[8 * kc + c]);
                         } else {
 #pragma unroll
                             for (int c = 0; c < 8; ++c)
@@ -760,6 +796,11 @@ __global__ void __launch_bounds__(CTHREADS, 1)
             }
         }
         if (!ok && lane == 0) atomicExch(a.err, 1u);
+        if (EPI == EPI_MASK_BF16) {
+            fold_bias();
+            const long long rows = (long long)gridDim.x * (4 * ESETS);
+            a.bpart[((lane >> 3) * rows + blockIdx.x * (4 * ESETS) + warp) * 8 + (lane & 7)] = btotal;
+        }
         if (EPI == EPI_SCALED_F32 && a.gmax) {
             unsigned long long bits = (unsigned long long)__double_as_longlong((double)gm);
             for (int o = 16; o > 0; o >>= 1) {
@@ -1151,17 +1192,25 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
 // 32); cin = 8 gives the tap-pair image.  Only the core-matrix rows ng_lo ..
 // ng_lo + ng_cnt - 1 of the kz stack are written, as an image of their own
 // (ng_cnt = 3 nb / 8 for the whole stack; the paired kernel takes the two
-// halves one after the other).
-__global__ void conv_tc_prep_kernel(const float *__restrict__ W, int cout, int cin_real, int cin,
-                                    int nb, int ng_lo, int ng_cnt, bf16 *__restrict__ img) {
-    const int KC = cin / 8;
-    const bool pair = cin == 8;
-    const int total = (pair ? 10 : 9 * KC) * ng_cnt * 64;
+// halves one after the other).  With flip set W is the forward weights
+// [cin_real][cout][27] of the layer whose input gradient this is: channels
+// exchanged, taps mirrored.
+struct ImageJob {
+    const float *w;
+    int cout, cin_real, cin, nb, ng_lo, ng_cnt;
+    bool flip;
+    bf16 *img;
+};
+
+__device__ __forceinline__ void conv_tc_prep(const ImageJob &a) {
+    const int KC = a.cin / 8;
+    const bool pair = a.cin == 8;
+    const int total = (pair ? 10 : 9 * KC) * a.ng_cnt * 64;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
         const int c = i & 7, r = (i >> 3) & 7;
         const int rest = i >> 6;  // kq * ng_cnt + (ng - ng_lo)
-        const int ng = ng_lo + rest % ng_cnt;
-        const int kq = rest / ng_cnt;
+        const int ng = a.ng_lo + rest % a.ng_cnt;
+        const int kq = rest / a.ng_cnt;
         int dyx, ci;
         bool live = true;
         if (pair) {
@@ -1174,11 +1223,13 @@ __global__ void conv_tc_prep_kernel(const float *__restrict__ W, int cout, int c
             ci = 8 * (kq % KC) + c;
         }
         const int row = 8 * ng + r;
-        const int kz = 2 - row / nb, co = row % nb;
-        const float v = (live && co < cout && ci < cin_real)
-                            ? W[((long long)co * cin_real + ci) * 27 + kz * 9 + dyx]
-                            : 0.f;
-        img[i] = __float2bfloat16_rn(v);
+        const int kz = 2 - row / a.nb, co = row % a.nb;
+        const int tap = kz * 9 + dyx;
+        float v = 0.f;
+        if (live && co < a.cout && ci < a.cin_real)
+            v = a.flip ? a.w[((long long)ci * a.cout + co) * 27 + 26 - tap]
+                       : a.w[((long long)co * a.cin_real + ci) * 27 + tap];
+        a.img[i] = __float2bfloat16_rn(v);
     }
 }
 

@@ -416,18 +416,41 @@ __global__ void adam_kernel(float *__restrict__ p, float *__restrict__ m, float 
 // bfloat16 weights from the master copy W[co][ci][tap]:
 //   forward layout    Wf[co][tap][ci_pad]   (ci >= cin stays zero);
 //   transposed layout Wb[ci][26 - tap][co_pad] for the input gradient.
-__global__ void prep_weights_kernel(const float *__restrict__ W, int cout, int cin, int cin_pad,
-                                    bf16 *__restrict__ wf, int cout_pad, bf16 *__restrict__ wb) {
-    const int total = cout * cin * 27;
+struct WeightJob {
+    const float *w;
+    int cout, cin, cin_pad;
+    bf16 *wf;
+    int cout_pad;
+    bf16 *wb;
+};
+
+__device__ __forceinline__ void prep_weights_job(const WeightJob &a) {
+    const int total = a.cout * a.cin * 27;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
-        const int co = t / (cin * 27);
-        const int rem = t - co * cin * 27;
+        const int co = t / (a.cin * 27);
+        const int rem = t - co * a.cin * 27;
         const int ci = rem / 27;
         const int tap = rem - ci * 27;
-        const bf16 w = __float2bfloat16_rn(W[t]);
-        wf[((long long)co * 27 + tap) * cin_pad + ci] = w;
-        if (wb) wb[((long long)ci * 27 + (26 - tap)) * cout_pad + co] = w;
+        const bf16 w = __float2bfloat16_rn(a.w[t]);
+        a.wf[((long long)co * 27 + tap) * a.cin_pad + ci] = w;
+        if (a.wb) a.wb[((long long)ci * 27 + (26 - tap)) * a.cout_pad + co] = w;
     }
+}
+
+// Every weight image in one launch, job blockIdx.y (seventeen launches of about 3 us and
+// the gaps between them took as long as a convolution of the training step).
+struct PrepJobs {
+    WeightJob w[3];
+    tc::ImageJob img[11];
+    int images;
+};
+
+__global__ void prep_kernel(const __grid_constant__ PrepJobs jobs) {
+    const int j = (int)blockIdx.y;
+    if (j < 3)
+        prep_weights_job(jobs.w[j]);
+    else
+        tc::conv_tc_prep(jobs.img[j - 3]);
 }
 
 // Full-weighting restriction: coarse(I) = sum_d w(d) fine(2I + d), w = (1/4, 1/2, 1/4)
@@ -615,11 +638,19 @@ __global__ void bias_grad_rp_kernel(const bf16 *__restrict__ zn, int kcs, int nx
     float s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     for (long long r = blockIdx.x + (long long)ty * G; r < rows; r += 8LL * G) {
         const uint4 *row = reinterpret_cast<const uint4 *>(zn + (r * kcs + kc) * nxp * 8);
-        for (int j = 1 + tx; j <= nx; j += 32) {
-            __align__(16) bf16 v[8];
-            *reinterpret_cast<uint4 *>(v) = row[j];
+        // four loads in flight (8 channels at 128^3: 16.8 -> 13.7 us)
+        for (int j = 1 + tx; j <= nx; j += 128) {
+            uint4 w[4];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) s[c] += __bfloat162float(v[c]);
+            for (int q = 0; q < 4; ++q)
+                if (j + 32 * q <= nx) w[q] = row[j + 32 * q];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (j + 32 * q > nx) break;
+                const bf16 *v = reinterpret_cast<const bf16 *>(&w[q]);
+#pragma unroll
+                for (int c = 0; c < 8; ++c) s[c] += __bfloat162float(v[c]);
+            }
         }
     }
     __shared__ double sh[8][256];
@@ -637,27 +668,16 @@ __global__ void bias_grad_rp_kernel(const bf16 *__restrict__ zn, int kcs, int nx
 
 // gb[co] = sum over blocks of the partials above: one warp per channel, lane l
 // taking blocks l, l + 32, ..., then a fixed shuffle tree.
-__global__ void bias_reduce_kernel(const double *__restrict__ bpart, int G, float *__restrict__ gb) {
-    const int co = blockIdx.x, lane = threadIdx.x;
+__global__ void __launch_bounds__(128)
+    bias_reduce_kernel(const double *__restrict__ bpart, int G, float *__restrict__ gb) {
+    const int co = blockIdx.x, lane = threadIdx.x & 31;
+    __shared__ double sh[4];
     double s = 0.0;
-    for (int b = lane; b < G; b += 32) s += bpart[((long long)(co / 8) * G + b) * 8 + co % 8];
+    for (int b = threadIdx.x; b < G; b += 128) s += bpart[((long long)(co / 8) * G + b) * 8 + co % 8];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) gb[co] = (float)s;
-}
-
-// Weights of the input-gradient convolution: Wt[ci][co][26 - tap] = W[co][ci][tap]
-// (the adjoint of a cross-correlation correlates with the flipped kernel, input
-// and output channels exchanged).
-__global__ void flip_transpose_kernel(const float *__restrict__ W, int cout, int cin,
-                                      float *__restrict__ Wt) {
-    const int total = cout * cin * 27;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
-        const int co = t / (cin * 27);
-        const int rem = t - co * cin * 27;
-        const int ci = rem / 27;
-        const int tap = rem - ci * 27;
-        Wt[((long long)ci * cout + co) * 27 + 26 - tap] = W[t];
-    }
+    if (lane == 0) sh[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x == 0) gb[co] = (float)((sh[0] + sh[1]) + (sh[2] + sh[3]));
 }
 
 }  // namespace ac
@@ -697,7 +717,6 @@ struct ac_closure {
     // tensor maps, per-CTA weight-gradient and bias partials
     void *train_block;
     bf16 *img3b, *img2b, *dyh, *dy2h, *dz2h, *dz1h;
-    float *wt;      // flipped, transposed master weights of layers 3 and 2
     float *wpart;
     double *bpart;
     CUtensorMap tr_map[4];  // dyh, dz2h, dy2h, dz1h
@@ -935,36 +954,29 @@ extern "C" int ac_closure_quit(ac_closure *c) {
     return AC_OK;
 }
 
-// Input-gradient weight images of layers 3 and 2 (the tcgen05 training path):
-// the flipped, transposed weights in the image order of conv_tc_kernel.
-static void prep_train_images(ac_closure *c) {
-    float *wt3 = c->wt, *wt2 = c->wt + 8 * 32 * 27;
-    flip_transpose_kernel<<<32, 256, 0, c->stream>>>(c->params + P_W3, 8, 32, wt3);
-    flip_transpose_kernel<<<128, 256, 0, c->stream>>>(c->params + P_W2, 32, 32, wt2);
-    tc::conv_tc_prep_kernel<<<16, 256, 0, c->stream>>>(wt3, 32, 8, 8, 32, 0, 12, c->img3b);
-    tc::conv_tc_prep_kernel<<<128, 256, 0, c->stream>>>(wt2, 32, 32, 32, 32, 0, 12, c->img2b);
-    c->launches += 4;
-}
-
+// Every weight image from the master weights, the input-gradient images too once
+// training has allocated them.
 static int prep_weights(ac_closure *c) {
-    if (c->train_block) prep_train_images(c);
-    prep_weights_kernel<<<32, 256, 0, c->stream>>>(c->params + P_W1, 32, 8, 16, c->wf1, 0, nullptr);
-    prep_weights_kernel<<<128, 256, 0, c->stream>>>(c->params + P_W2, 32, 32, 32, c->wf2, 32, c->wb2);
-    prep_weights_kernel<<<32, 256, 0, c->stream>>>(c->params + P_W3, 8, 32, 32, c->wf3, 16, c->wb3);
-    tc::conv_tc_prep_kernel<<<16, 256, 0, c->stream>>>(c->params + P_W1, 32, 8, 8, 32, 0, 12, c->img1);
-    tc::conv_tc_prep_kernel<<<128, 256, 0, c->stream>>>(c->params + P_W2, 32, 32, 32, 32, 0, 12,
-                                                        c->img2);
-    tc::conv_tc_prep_kernel<<<64, 256, 0, c->stream>>>(c->params + P_W3, 8, 32, 32, 16, 0, 6, c->img3);
+    const float *W1 = c->params + P_W1, *W2 = c->params + P_W2, *W3 = c->params + P_W3;
+    PrepJobs p = {{{W1, 32, 8, 16, c->wf1, 0, nullptr},
+                   {W2, 32, 32, 32, c->wf2, 32, c->wb2},
+                   {W3, 8, 32, 32, c->wf3, 16, c->wb3}},
+                  {{W1, 32, 8, 8, 32, 0, 12, false, c->img1},
+                   {W2, 32, 32, 32, 32, 0, 12, false, c->img2},
+                   {W3, 8, 32, 32, 16, 0, 6, false, c->img3}},
+                  3};
     // paired kernel: stack rows 0..47 (core rows 0..5) then 48..95, 32 per kz
     for (int h = 0; h < 2; ++h) {
-        tc::conv_tc_prep_kernel<<<16, 256, 0, c->stream>>>(c->params + P_W1, 32, 8, 8, 32, 6 * h, 6,
-                                                           c->pimg1 + h * tc::w_bytes(8, 32) / 4);
-        tc::conv_tc_prep_kernel<<<64, 256, 0, c->stream>>>(c->params + P_W2, 32, 32, 32, 32, 6 * h, 6,
-                                                           c->pimg2 + h * tc::w_bytes(32, 32) / 4);
-        tc::conv_tc_prep_kernel<<<64, 256, 0, c->stream>>>(c->params + P_W3, 8, 32, 32, 32, 6 * h, 6,
-                                                           c->pimg3 + h * tc::w_bytes(32, 32) / 4);
+        p.img[p.images++] = {W1, 32, 8, 8, 32, 6 * h, 6, false, c->pimg1 + h * tc::w_bytes(8, 32) / 4};
+        p.img[p.images++] = {W2, 32, 32, 32, 32, 6 * h, 6, false, c->pimg2 + h * tc::w_bytes(32, 32) / 4};
+        p.img[p.images++] = {W3, 8, 32, 32, 32, 6 * h, 6, false, c->pimg3 + h * tc::w_bytes(32, 32) / 4};
     }
-    c->launches += 12;
+    if (c->train_block) {
+        p.img[p.images++] = {W3, 32, 8, 8, 32, 0, 12, true, c->img3b};
+        p.img[p.images++] = {W2, 32, 32, 32, 32, 0, 12, true, c->img2b};
+    }
+    prep_kernel<<<dim3(64, 3 + p.images), 256, 0, c->stream>>>(p);
+    c->launches++;
     CCK(cudaGetLastError());
     return AC_OK;
 }
@@ -1220,7 +1232,7 @@ static cudaError_t wgrad_grid_for(const ac_closure *c, int sms, int *grid) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
     int per_sm = 0;
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, tc::THREADS, S::SMEM);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, tc::WTHREADS, S::SMEM);
     if (e != cudaSuccess) return e;
     if (per_sm > 512 / S::TCOLS) per_sm = 512 / S::TCOLS;
     const long long segs = (long long)((c->g.nz + c->tc_zc - 1) / c->tc_zc) * c->g.ny *
@@ -1257,14 +1269,15 @@ static int ensure_train(ac_closure *c) {
     c->tr_bias_blocks = (int)(rows / 64 < 1 ? 1 : (rows / 64 > 4096 ? 4096 : rows / 64));
     const long long np2 = (long long)tc::rp_cells(c->g.nx) * rows;
     const size_t b_wpart = align256(sizeof(float) * (size_t)wmax * tc::TM);
-    const size_t b_bpart = align256(sizeof(double) * 4 * (size_t)c->tr_bias_blocks * 8);
-    const size_t b_wt = align256(sizeof(float) * (8 * 32 * 27 + 32 * 32 * 27));
+    // rows of eight bias partials: the output layer's, or the input gradients' epilogue warps'
+    const int brows = 4 * 4 * tc::ESETS * (c->tr_grid[0] > c->tr_grid[1] ? c->tr_grid[0] : c->tr_grid[1]);
+    const size_t b_bpart = align256(sizeof(double) * 8 * (size_t)(brows > c->tr_bias_blocks ? brows : c->tr_bias_blocks));
     const size_t b_img3 = align256((size_t)tc::w_bytes(8, 32));
     const size_t b_img2 = align256((size_t)tc::w_bytes(32, 32));
     // dyh (8 channels), dy2h (16: 8 and a zero plane), dz2h, dz1h (32), row-planar with halo
     const size_t b_act[4] = {align256(2 * 8 * (size_t)np2), align256(2 * 16 * (size_t)np2),
                              align256(2 * 32 * (size_t)np2), align256(2 * 32 * (size_t)np2)};
-    size_t total = b_wpart + b_bpart + b_wt + b_img3 + b_img2;
+    size_t total = b_wpart + b_bpart + b_img3 + b_img2;
     for (int i = 0; i < 4; ++i) total += b_act[i];
     void *blk = nullptr;
     cudaError_t e = cudaMalloc(&blk, total);
@@ -1278,8 +1291,6 @@ static int ensure_train(ac_closure *c) {
     p += b_wpart;
     c->bpart = reinterpret_cast<double *>(p);
     p += b_bpart;
-    c->wt = reinterpret_cast<float *>(p);
-    p += b_wt;
     c->img3b = reinterpret_cast<bf16 *>(p);
     p += b_img3;
     c->img2b = reinterpret_cast<bf16 *>(p);
@@ -1302,21 +1313,20 @@ static int ensure_train(ac_closure *c) {
         return ac_report_cuda(e);
     }
     c->train_block = blk;
-    prep_train_images(c);
-    CCK(cudaGetLastError());
-    return AC_OK;
+    return prep_weights(c);
 }
 
 // One input-gradient convolution through a ReLU on the tcgen05 kernel: from the
 // row-planar gradient behind xmap, with image img, mask = the forward activation;
-// writes y (with its halo cells).
+// writes y (with its halo cells) and its sums over the cells, the bias gradient gb.
 template <int CIN>
 static void launch_mask(const ac_closure *c, const CUtensorMap &xmap, int grid, const bf16 *img,
-                        const bf16 *mask, bf16 *y) {
+                        const bf16 *mask, bf16 *y, float *gb) {
     tc::ConvTcArgs a = {};
     a.w = img;
     a.y = y;
     a.mask = mask;
+    a.bpart = c->bpart;
     a.nx = c->g.nx;
     a.ny = c->g.ny;
     a.nz = c->g.nz;
@@ -1324,6 +1334,7 @@ static void launch_mask(const ac_closure *c, const CUtensorMap &xmap, int grid, 
     a.err = c->tc_err;
     tc::conv_tc_kernel<CIN, 32, tc::EPI_MASK_BF16>
         <<<grid, tc::CTHREADS, tc::smem_bytes(CIN, 32), c->stream>>>(xmap, a);
+    bias_reduce_kernel<<<32, 128, 0, c->stream>>>(c->bpart, 4 * tc::ESETS * grid, gb);
 }
 
 template <int CIN, int COUT>
@@ -1337,20 +1348,16 @@ static void launch_wgrad(const ac_closure *c, const CUtensorMap &xmap, const CUt
     a.zc = c->tc_zc;
     a.err = c->tc_err;
     tc::wgrad_tc_kernel<CIN, COUT>
-        <<<grid, tc::THREADS, tc::WgradShape<CIN, COUT>::SMEM, c->stream>>>(xmap, dmap, a);
-    tc::wgrad_tc_reduce_kernel<CIN, COUT><<<152, 256, 0, c->stream>>>(c->wpart, grid, cin_real, gW);
-}
-
-static void launch_bias(const ac_closure *c, const bf16 *zn, int kcs, int cout, float *gb) {
-    const long long rows = (long long)c->g.ny * c->g.nz;
-    bias_grad_rp_kernel<<<dim3((unsigned)c->tr_bias_blocks, (unsigned)(cout / 8)), 256, 0, c->stream>>>(
-        zn, kcs, c->g.nx, rows, c->bpart);
-    bias_reduce_kernel<<<cout, 32, 0, c->stream>>>(c->bpart, c->tr_bias_blocks, gb);
+        <<<grid, tc::WTHREADS, tc::WgradShape<CIN, COUT>::SMEM, c->stream>>>(xmap, dmap, a);
+    constexpr int entries = tc::WgradShape<CIN, COUT>::NACC * tc::WgradShape<CIN, COUT>::N3 * tc::TM;
+    tc::wgrad_tc_reduce_kernel<CIN, COUT>
+        <<<entries / tc::RENTRIES, tc::RSPLIT * tc::RENTRIES, 0, c->stream>>>(c->wpart, grid, cin_real, gW);
 }
 
 // Backward pass on the tcgen05 kernels: forward (row-planar activations kept),
 // loss and dY, the two input gradients through the ReLUs (flipped, transposed
-// weights), the three weight gradients and the three bias gradients.
+// weights) with the bias gradients of their layers, the three weight gradients
+// and the output layer's bias gradient.
 static int run_backward_tc(ac_closure *c, const float *const in[8], const float *const target[8]) {
     int rc = ensure_train(c);
     if (rc) return rc;
@@ -1361,15 +1368,15 @@ static int run_backward_tc(ac_closure *c, const float *const in[8], const float 
     for (int i = 0; i < 8; ++i) t.p[i] = target[i];
     loss_grad_rp_kernel<<<c->lossblocks, 256, 0, c->stream>>>(c->y, t, c->scales + 16, g.nx, g.n,
                                                               c->dyh, c->dy2h, c->lossp);
-    launch_mask<8>(c, c->tr_map[0], c->tr_grid[0], c->img3b, c->a2, c->dz2h);
-    launch_mask<32>(c, c->tr_map[1], c->tr_grid[1], c->img2b, c->a1, c->dz1h);
+    launch_mask<8>(c, c->tr_map[0], c->tr_grid[0], c->img3b, c->a2, c->dz2h, c->grads + P_B2);
+    launch_mask<32>(c, c->tr_map[1], c->tr_grid[1], c->img2b, c->a1, c->dz1h, c->grads + P_B1);
     launch_wgrad<32, 8>(c, c->tc_map[2], c->tr_map[2], c->tr_grid[2], 32, c->grads + P_W3);
     launch_wgrad<32, 32>(c, c->tc_map[1], c->tr_map[1], c->tr_grid[3], 32, c->grads + P_W2);
     launch_wgrad<8, 32>(c, c->tc_map[0], c->tr_map[3], c->tr_grid[4], 8, c->grads + P_W1);
-    launch_bias(c, c->dy2h, 2, 8, c->grads + P_B3);
-    launch_bias(c, c->dz2h, 4, 32, c->grads + P_B2);
-    launch_bias(c, c->dz1h, 4, 32, c->grads + P_B1);
-    c->launches += 15;
+    bias_grad_rp_kernel<<<c->tr_bias_blocks, 256, 0, c->stream>>>(c->dy2h, 2, g.nx, (long long)g.ny * g.nz,
+                                                                  c->bpart);
+    bias_reduce_kernel<<<8, 128, 0, c->stream>>>(c->bpart, c->tr_bias_blocks, c->grads + P_B3);
+    c->launches += 13;
     CCK(cudaGetLastError());
     return AC_OK;
 }

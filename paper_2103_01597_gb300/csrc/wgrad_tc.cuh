@@ -29,16 +29,18 @@
 // the epilogue warps write per-CTA partial sums, which a second kernel adds in
 // binary64 in a fixed order.
 //
-// Warp roles: warp 4 (one thread) issues the TMA copies, warp 5 the MMAs, warps
-// 0-3 zero the accumulators, prepare each dZ tile's shifted copies and read the
-// accumulators at the end.  Every wait is bounded; on timeout the role records
-// an error word and stops.
+// Warp roles: warp 8 (one thread) issues the TMA copies, warp 9 the MMAs; warps 0-7, two
+// sets, prepare the dZ tiles' shifted copies in turn and read the accumulators at the end
+// (warps 0-3 zero them).  Every wait is bounded; on timeout the role records an error word
+// and stops.
 #pragma once
 
 #include "conv_tc.cuh"
 
 namespace ac {
 namespace tc {
+
+constexpr int WTHREADS = 32 * (4 * 2 + 2);  // two sets of copy warps, TMA, MMA
 
 struct WgradTcArgs {
     float *part;  // [grid][NACC][N3][128] per-CTA partial sums
@@ -88,7 +90,7 @@ __host__ __device__ constexpr uint32_t idesc_bf16_mn(int m, int n) {
 }
 
 template <int CIN, int COUT>
-__global__ void __launch_bounds__(THREADS, 1)
+__global__ void __launch_bounds__(WTHREADS, 1)
     wgrad_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap dmap,
                     const WgradTcArgs a) {
     using S = WgradShape<CIN, COUT>;
@@ -115,7 +117,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     ga.zc = a.zc;
 
     if (warp == 0) tmem_alloc(&tmem_base, S::TCOLS);
-    if (threadIdx.x == 128) {
+    if (threadIdx.x == 256) {
         for (int b = 0; b < NSLOT; ++b) {
             mbar_init(&full[b], 1);
             mbar_init(&empty[b], 1);
@@ -132,7 +134,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     // the ring bytes past the slots are only read into discarded rows: keep them finite
-    for (int i = S::RING_S + 16 * (int)threadIdx.x; i < S::RING; i += 16 * THREADS)
+    for (int i = S::RING_S + 16 * (int)threadIdx.x; i < S::RING; i += 16 * WTHREADS)
         *reinterpret_cast<uint4 *>(Ss + i) = make_uint4(0, 0, 0, 0);
     fence_proxy_async_smem();
     __syncthreads();  // barriers initialised, TMEM address published
@@ -146,14 +148,13 @@ __global__ void __launch_bounds__(THREADS, 1)
     __syncthreads();
     tc_fence_after_sync();
 
-    if (warp == 4) {
+    if (warp == 8) {
         if (lane == 0) {  // ---- TMA producer: slices 0, 1, then (slice i + 2, dZ tile i)
-            long long s = 0, t = 0;
+            int b = 0, l = 0;         // slot of the next slice, buffer of the next dZ tile
+            unsigned round = 0, lround = 0;  // completed passes over the slots, the buffers
             bool ok = true;
             auto slice = [&](const Segment &sg, int j) {
-                const int b = (int)(s % NSLOT);
-                const long long k = s / NSLOT;
-                if (k > 0 && !mbar_wait(&empty[b], (unsigned)((k - 1) & 1))) return false;
+                if (round > 0 && !mbar_wait(&empty[b], (round - 1) & 1)) return false;
                 const int copies = S::MIRROR && b < 2 ? 2 : 1;
                 mbar_expect_tx(&full[b], copies * SLICE_TX);
                 const int z = wrapi(sg.z0 + j - 1, a.nz);
@@ -164,7 +165,10 @@ __global__ void __launch_bounds__(THREADS, 1)
                         tma_load_5d(dst + r * ROW, &xmap, &full[b], 0, sg.seg * (TM / 8), 0,
                                     wrapi(sg.y + r - 1, a.ny), z);
                 }
-                ++s;
+                if (++b == NSLOT) {
+                    b = 0;
+                    ++round;
+                }
                 return true;
             };
             for (long long g = blockIdx.x; g < nseg && ok; g += gridDim.x) {
@@ -173,9 +177,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 for (int i = 0; i < sg.len && ok; ++i) {
                     ok = slice(sg, i + 2);
                     if (!ok) break;
-                    const int l = (int)(t % NL);
-                    const long long k = t / NL;
-                    if (k > 0 && !mbar_wait(&lempty[l], (unsigned)((k - 1) & 1))) {
+                    if (lround > 0 && !mbar_wait(&lempty[l], (lround - 1) & 1)) {
                         ok = false;
                         break;
                     }
@@ -183,19 +185,27 @@ __global__ void __launch_bounds__(THREADS, 1)
                     // landed row r = slot x0 + r, cell x0 + r - 1
                     tma_load_5d(Ls + l * COPY, &dmap, &lfull[l], 0, sg.seg * (TM / 8), 0, sg.y,
                                 sg.z0 + i);
-                    ++t;
+                    if (++l == NL) {
+                        l = 0;
+                        ++lround;
+                    }
                 }
             }
             if (!ok) atomicExch(a.err, 1u);
             // no copy may be in flight when the CTA exits: wait for each buffer's last fill
-            for (int b = 0; b < NSLOT; ++b)
-                if (s > b) mbar_wait(&full[b], (unsigned)(((s - 1 - b) / NSLOT) & 1));
-            for (int l = 0; l < NL; ++l)
-                if (t > l) mbar_wait(&lfull[l], (unsigned)(((t - 1 - l) / NL) & 1));
+            for (int q = 0; q < NSLOT; ++q) {
+                const unsigned fills = round + (q < b);
+                if (fills) mbar_wait(&full[q], (fills - 1) & 1);
+            }
+            for (int q = 0; q < NL; ++q) {
+                const unsigned fills = lround + (q < l);
+                if (fills) mbar_wait(&lfull[q], (fills - 1) & 1);
+            }
         }
-    } else if (warp == 5) {
+    } else if (warp == 9) {
         // ---- MMA issuer: the whole warp runs the loop, one elected lane issues
-        long long s = 0, t = 0;  // first slice of the current tile's run; dZ tiles consumed
+        int b = 0, c = 0;             // slot of the run's first slice, copy set of the tile
+        unsigned fill = 0, cfill = 0;  // parities of their fills
         bool ok = true;
         const uint32_t idesc = idesc_bf16_mn(TM, N3);
         for (long long g = blockIdx.x; g < nseg && ok; g += gridDim.x) {
@@ -204,22 +214,26 @@ __global__ void __launch_bounds__(THREADS, 1)
             const int valid = a.nx - sg.seg * TM;
             const int nks = valid >= TM ? TM / 16 : (valid + 15) / 16;  // K-steps with cells < nx
             for (int i = 0; i < L; ++i) {
-                // slices s .. s + 2 have landed (the first two were waited for by the
-                // previous tile of the segment, or are waited now); tile t's copies are ready
-                for (int q = (i == 0 ? 0 : 2); q < 3 && ok; ++q)
-                    ok = __all_sync(0xffffffffu,
-                                    mbar_wait(&full[(s + q) % NSLOT], (unsigned)(((s + q) / NSLOT) & 1)));
-                const int c = (int)(t % NC);
-                if (ok)
-                    ok = __all_sync(0xffffffffu, mbar_wait(&cready[c], (unsigned)((t / NC) & 1)));
+                // the run's three slices have landed (the first two were waited for by the
+                // previous tile of the segment, or are waited now); the tile's copies are ready
+                int slot[3];
+                bool here = true;
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    slot[q] = b + q < NSLOT ? b + q : b + q - NSLOT;
+                    if (i == 0 || q == 2)
+                        here = mbar_wait(&full[slot[q]], b + q < NSLOT ? fill : fill ^ 1u) && here;
+                }
+                here = mbar_wait(&cready[c], cfill) && here;
+                ok = __all_sync(0xffffffffu, here);
                 if (!ok) break;
                 tc_fence_after_sync();
                 // A: the tile's cells x0 + k are staged rows k + 1 of every plane of the run;
                 // block mb starts at plane 0 of the run's (mb)-th slice
                 uint64_t a0[NMB];
 #pragma unroll
-                for (int mb = 0; mb < NMB; ++mb)  // block mb: slice s + mb, in its own slot
-                    a0[mb] = smem_desc(smem_u32(Ss + (int)((s + mb) % NSLOT) * SLICE) + 16, CORE, PLANE);
+                for (int mb = 0; mb < NMB; ++mb)  // block mb: the run's slice mb, in its own slot
+                    a0[mb] = smem_desc(smem_u32(Ss + slot[mb] * SLICE) + 16, CORE, PLANE);
                 const uint64_t b0 = smem_desc(smem_u32(Cs + c * 3 * COPY), CORE, PLANE);
                 for (int ks = 0; ks < nks; ++ks) {
                     const uint64_t step = (uint32_t)(ks * 256) >> 4;
@@ -228,67 +242,86 @@ __global__ void __launch_bounds__(THREADS, 1)
                         mma_bf16_elect(tmem + (uint32_t)(mb * N3), a0[mb] + step, b0 + step, idesc);
                 }
                 mma_commit_elect(&cempty[c]);
-                mma_commit_elect(&empty[s % NSLOT]);  // slice s serves no later tile
+                mma_commit_elect(&empty[slot[0]]);  // the run's first slice serves no later tile
                 if (i == L - 1) {
-                    mma_commit_elect(&empty[(s + 1) % NSLOT]);
-                    mma_commit_elect(&empty[(s + 2) % NSLOT]);
-                    s += 3;
-                } else {
-                    s += 1;
+                    mma_commit_elect(&empty[slot[1]]);
+                    mma_commit_elect(&empty[slot[2]]);
                 }
-                ++t;
+                b += i == L - 1 ? 3 : 1;
+                if (b >= NSLOT) {
+                    b -= NSLOT;
+                    fill ^= 1u;
+                }
+                if (++c == NC) {
+                    c = 0;
+                    cfill ^= 1u;
+                }
             }
         }
         if (!ok && lane == 0) atomicExch(a.err, 1u);
         mma_commit_elect(&done);  // every MMA of the CTA, before the epilogue reads TMEM
-    } else {  // ---- warps 0-3: the dZ tiles' shifted copies, then TMEM lanes 32 warp ..
-        const int tid = threadIdx.x;  // 0 .. 127
+    } else {  // ---- warps 0-7: the dZ tiles' shifted copies, then TMEM lanes 32 quad ..
+        // Two sets of four warps, each with its own landed tile and copy set, so that one
+        // tile's waits and fence overlap the other's copies (128^3, with 8 input channels:
+        // 98 -> 92 us; with 32, where the MMAs' operands bound it: 116 -> 115, 135 -> 134).
+        const int tid = threadIdx.x & 127, set = warp >> 2, quad = warp & 3;
         bool ok = true;
-        long long t = 0;
+        static_assert(NL == 2 && NC == 2, "a landed tile and a copy set for each set of warps");
+        const int c = set;
+        int turn = 0;        // set whose turn the next tile is
+        unsigned round = 0;  // tiles this set has copied
         for (long long g = blockIdx.x; g < nseg && ok; g += gridDim.x) {
             const Segment sg = segment_of(g, ga, segs);
             const int valid = a.nx - sg.seg * TM;  // rows r < valid are cells < nx
-            for (int i = 0; i < sg.len; ++i, ++t) {
-                const int l = (int)(t % NL), c = (int)(t % NC);
-                ok = __all_sync(0xffffffffu, mbar_wait(&lfull[l], (unsigned)((t / NL) & 1)));
-                if (ok && t >= NC)  // the MMAs of tile t - NC have read this copy set
-                    ok = __all_sync(0xffffffffu,
-                                    mbar_wait(&cempty[c], (unsigned)(((t / NC) - 1) & 1)));
+            for (int i = 0; i < sg.len; ++i) {
+                turn ^= 1;
+                if (turn == set) continue;  // (set 0 takes the first)
+                bool here = mbar_wait(&lfull[c], round & 1);
+                if (round > 0)  // the MMAs that read this copy set last are done
+                    here = mbar_wait(&cempty[c], (round - 1) & 1) && here;
+                ok = __all_sync(0xffffffffu, here);
                 if (!ok) break;
                 unsigned char *base = Cs + c * 3 * COPY;  // copy kx at base + kx * COPY
-                const unsigned char *landed = Ls + l * COPY;
+                const unsigned char *landed = Ls + c * COPY;
                 // copy kx, row r = landed row r + 2 - kx (cell x0 + r + 1 - kx); rows of
-                // cells past nx (r >= valid) zero
-                for (int e = tid; e < DKC * TM; e += 128) {
-                    const int pl = e / TM, r = e - pl * TM;
-                    const uint4 *src = reinterpret_cast<const uint4 *>(landed + pl * PLANE);
+                // cells past nx (r >= valid) zero.  Each landed row is read once: row tid
+                // of each plane, then the two rows past the tile.
+                auto spread = [&](int pl, int row) {
+                    const uint4 v = reinterpret_cast<const uint4 *>(landed + pl * PLANE)[row];
                     const uint4 z = make_uint4(0, 0, 0, 0);
-                    const bool in = r < valid;
-                    reinterpret_cast<uint4 *>(base + 2 * COPY + pl * PLANE)[r] = in ? src[r] : z;
-                    reinterpret_cast<uint4 *>(base + COPY + pl * PLANE)[r] = in ? src[r + 1] : z;
-                    reinterpret_cast<uint4 *>(base + pl * PLANE)[r] = in ? src[r + 2] : z;
-                }
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        const int r = row - k;  // copy 2 - k
+                        if (r >= 0 && r < TM)
+                            reinterpret_cast<uint4 *>(base + (2 - k) * COPY + pl * PLANE)[r] =
+                                r < valid ? v : z;
+                    }
+                };
+#pragma unroll
+                for (int pl = 0; pl < DKC; ++pl) spread(pl, tid);
+                if (tid < 2 * DKC) spread(tid >> 1, TM + (tid & 1));
                 // generic reads of the landed tile before the TMA refills it, generic
                 // writes of the copies before the tensor core reads them
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) {
-                    mbar_arrive(&lempty[l]);
+                    mbar_arrive(&lempty[c]);
                     mbar_arrive(&cready[c]);
                 }
+                ++round;
             }
         }
         if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&done, 0));
         tc_fence_after_sync();
         if (ok) {
-            const int m = warp * 32 + lane;
+            const int m = quad * 32 + lane;
             constexpr int CH = N3 % 32 == 0 ? 32 : 16;
 #pragma unroll 1
             for (int k = 0; k < NACC; ++k)
 #pragma unroll 1
-                for (int c0 = 0; c0 < N3; c0 += CH) {
+                for (int c0 = set * CH; c0 < N3; c0 += 2 * CH) {
                     const uint32_t taddr =
-                        tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(k * N3 + c0);
+                        tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(k * N3 + c0);
                     float v[CH];
                     if constexpr (CH == 32)
                         tmem_ld32(taddr, v);
@@ -312,23 +345,35 @@ __global__ void __launch_bounds__(THREADS, 1)
 // that the CTAs' blocks are read coalesced; entries that hold no gradient (padded
 // columns, rows past a block's planes) are skipped.  Row m of block mb is plane
 // P = mb BLK + m / 8 of the run, channel 8 (P % KC) + m % 8, tap row P / KC = 3 kz + ky.
-// Binary64 sums in CTA order.
+// Binary64 sums, RSPLIT runs of CTAs at once, added in order: one chain of 152 additions
+// took 23 us at any layer's size, eight take 13 us with 128 x 48 and 128 x 96 entries
+// and 27 us with 3 x 128 x 96, where the FP64 pipe bounds them.
+constexpr int RSPLIT = 8, RENTRIES = 32;
+
 template <int CIN, int COUT>
-__global__ void wgrad_tc_reduce_kernel(const float *__restrict__ part, int ctas, int cin_real,
-                                       float *__restrict__ gW) {
+__global__ void __launch_bounds__(RSPLIT * RENTRIES)
+    wgrad_tc_reduce_kernel(const float *__restrict__ part, int ctas, int cin_real, float *__restrict__ gW) {
     using S = WgradShape<CIN, COUT>;
     constexpr int PER_CTA = S::NACC * S::N3 * TM;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < PER_CTA; t += gridDim.x * blockDim.x) {
-        const int m = t % TM, n = (t / TM) % S::N3, mb = t / (TM * S::N3);
-        const int kx = n / S::NB, co = n % S::NB;
-        const int P = mb * S::BLK + m / 8;
-        if (co >= COUT || P >= S::NPL || (S::BLK > 0 && m / 8 >= S::BLK)) continue;
-        const int ci = 8 * (P % S::KC) + m % 8;
-        if (ci >= cin_real) continue;
-        const int tr = P / S::KC;
-        double s = 0.0;
-        for (int b = 0; b < ctas; ++b) s += part[(long long)b * PER_CTA + t];
-        gW[(co * cin_real + ci) * 27 + tr * 3 + kx] = (float)s;
+    static_assert(PER_CTA % RENTRIES == 0, "whole blocks");
+    __shared__ double sh[RSPLIT][RENTRIES];
+    const int e = threadIdx.x % RENTRIES, run = threadIdx.x / RENTRIES;
+    const int t = blockIdx.x * RENTRIES + e;
+    const int m = t % TM, n = (t / TM) % S::N3, mb = t / (TM * S::N3);
+    const int kx = n / S::NB, co = n % S::NB;
+    const int P = mb * S::BLK + m / 8;
+    const int ci = 8 * (P % S::KC) + m % 8;
+    const bool live = co < COUT && P < S::NPL && (S::BLK == 0 || m / 8 < S::BLK) && ci < cin_real;
+    const int chunk = (ctas + RSPLIT - 1) / RSPLIT;
+    double s = 0.0;
+    if (live)
+        for (int b = run * chunk; b < min(ctas, (run + 1) * chunk); ++b)
+            s += part[(long long)b * PER_CTA + t];
+    sh[run][e] = s;
+    __syncthreads();
+    if (run == 0 && live) {
+        for (int q = 1; q < RSPLIT; ++q) s += sh[q][e];
+        gW[(co * cin_real + ci) * 27 + (P / S::KC) * 3 + kx] = (float)s;
     }
 }
 
