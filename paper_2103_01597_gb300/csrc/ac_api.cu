@@ -62,7 +62,7 @@ struct ac_handle {
     int stencil_mode;             // AC_STENCIL_*
     void *fx_block;               // int64 copies of the fields (integer stencil sums)
     CUtensorMap fx_map;           // tensor map over them
-    unsigned long long *fx_stats; // per-field extremes (16 words) of the substep's input
+    unsigned long long *fx_stats; // per-field extremes of the substep's input (16 words, and a count)
     void *fx_plan;                // device plan of the integer-sum path (mode, scales)
     double *stage;       // float64 staging for load/store
     size_t stage_elems;
@@ -547,8 +547,9 @@ extern "C" int ac_set_forcing(ac_handle *h, const int k[3], const double e[3], d
 }
 
 // Measured, us per step with unequal spacings, integer form against plain stencils:
-// 11520 cells 115 against 84, 17472 cells 115 against 147, 32768 cells 115 against 147,
-// 215040 cells 321 against 812 (the integer form's preparation launches set its floor).
+// 11520 cells 115 against 84 (with two launches a substep more than now), 17472 cells 114
+// against 146, 32768 cells 114 against 147, 215040 cells 316 against 811 (the integer form's
+// preparation launches set its floor).
 constexpr long long FX_UNEQUAL_MIN_CELLS = 16384;
 
 // Integer stencil sums apply to binary64 fields on a periodic grid with equal
@@ -623,15 +624,16 @@ static int ensure_fx(ac_handle *h) {
     unsigned long long *stats = nullptr;
     void *plan = nullptr;
     cudaError_t e = cudaMalloc(&blk, fx_copy_bytes(h->g));
-    if (e == cudaSuccess) e = cudaMalloc(&stats, 2 * NF * sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaMalloc(&stats, (2 * NF + 1) * sizeof(unsigned long long));
     if (e == cudaSuccess) e = fx_encode_map(blk, h->g, &h->fx_map);
     if (e == cudaSuccess) e = cudaMalloc(&plan, fx_plan_bytes());
     if (e == cudaSuccess) e = cudaMemsetAsync(plan, 0, fx_plan_bytes(), h->stream);
-    // extremes: largest keys start at 0, smallest at all ones (the plan kernel
-    // restores this after every read)
+    // extremes: largest keys start at 0, smallest at all ones, then the count of
+    // finished CTAs (the plan restores this after every read)
     if (e == cudaSuccess) e = cudaMemsetAsync(stats, 0, NF * sizeof(unsigned long long), h->stream);
     if (e == cudaSuccess)
         e = cudaMemsetAsync(stats + NF, 0xff, NF * sizeof(unsigned long long), h->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(stats + 2 * NF, 0, sizeof(unsigned long long), h->stream);
     if (e != cudaSuccess) {
         if (blk) cudaFree(blk);
         if (stats) cudaFree(stats);

@@ -144,8 +144,8 @@ cudaError_t launch_substep_f64(const SubstepLaunch &L, cudaStream_t st, int *lau
     const long long n = L.g.elems;
     FxPlan *plan = static_cast<FxPlan *>(L.fx_plan);
     cudaError_t e;
-    fx_stats_kernel<<<fx_grid(n / 2), 256, 0, st>>>(fx, n, L.fx_stats);
-    fx_plan_kernel<<<1, 32, 0, st>>>(L.fx_stats, plan, L.ph.inv_cp, L.ph.gamma_cp, L.ph.gm1, aniso);
+    fx_stats_kernel<<<fx_grid(n / 2), 256, 0, st>>>(fx, n, L.fx_stats, plan, L.ph.inv_cp, L.ph.gamma_cp,
+                                                   L.ph.gm1, aniso);
     fx_quantize_kernel<<<fx_grid(32ll * fx.py * fx.pz), 256, 0, st>>>(fx, L.g, plan);
     if (L.ev_mid) {
         e = cudaEventRecord(L.ev_mid, st);
@@ -167,13 +167,13 @@ cudaError_t launch_substep_f64(const SubstepLaunch &L, cudaStream_t st, int *lau
         e = aniso ? launch_fx_group<C, X, true>(a, *L.fx_map, fc, plan, st)        \
                   : launch_fx_group<C, X, false>(a, *L.fx_map, fc, plan, st);      \
         if (e != cudaSuccess) return e;                                            \
-        if (!aniso) substep_fx_field_kernel<C, X><<<grid, block, 0, st>>>(a, fx, fc, plan); \
-        substep_fx_plain_kernel<C, X><<<grid, block, 0, st>>>(a, plan);            \
+        if (aniso) substep_fx_fallback_kernel<C, X, false><<<grid, block, 0, st>>>(a, fx, fc, plan); \
+        else substep_fx_fallback_kernel<C, X, true><<<grid, block, 0, st>>>(a, fx, fc, plan); \
     } while (0)
     if (ext) { if (cfl) AC_FX(true, true); else AC_FX(false, true); }
     else { if (cfl) AC_FX(true, false); else AC_FX(false, false); }
 #undef AC_FX
-    *launches += aniso ? 5 : 6;
+    *launches += 4;
     return cudaGetLastError();
 }
 

@@ -1,5 +1,5 @@
 // Binary64 substep with exact integer stencil sums and fixed-point products
-// (cubic periodic grids).
+// (periodic grids).
 //
 // GB300 executes two FP64 lanes per SM per cycle: an FP64-pipe instruction holds
 // its sub-partition's pipe for about 78 cycles per warp, a 64-bit integer addition
@@ -9,7 +9,7 @@
 // with c the midpoint of the field's range and 2^E above its half-range.  Every
 // weight set of Eq. 13 sums to zero, so the offset changes no derivative.
 //
-// A plan kernel picks one of three kernels per substep from the fields' ranges,
+// A plan picks one of three forms per substep from the fields' ranges,
 // on the device (no host round trip):
 //  * FX_GROUP (b = 56): the exponents E of the three components of u (and of A)
 //    lie within FX_GROUP_SLACK binades of each other and share the largest as one
@@ -17,7 +17,7 @@
 //    numerators are exact integers, the products of the right-hand side (u . grad,
 //    S . grad ln rho, S : S, j x B, j^2, u x B) exact integer dot products
 //    (fx_arith.cuh), the exponentials fixed point; what remains on the FP64 pipe
-//    is one multiply-add per term of Eqs. B.1-B.4 and the Runge-Kutta update (54
+//    is one multiply-add per term of Eqs. B.1-B.4 and the Runge-Kutta update (58
 //    instructions per cell).
 //  * FX_FIELD (b = 50): some component lies further below its group's largest, so
 //    every field keeps its own scale; integer numerators are converted one by one
@@ -94,7 +94,7 @@ struct FxPtrs {
 };
 
 // The quantisation plan of one substep (device memory, written by
-// fx_plan_kernel, read by the quantisation and substep kernels).
+// fx_stats_kernel, read by the quantisation and substep kernels).
 struct FxPlan {
     int kern;                  // the kernel that runs: FX_GROUP, FX_FIELD or FX_PLAIN
     int zero[NF];              // constant field: F = 0
@@ -109,77 +109,16 @@ struct FxPlan {
     int err;                   // set if a bounded wait of the substep kernel ran out
 };
 
-// Per-field extremes of the current state: stats[q] = largest key of field q,
-// stats[NF + q] = its smallest key (the plan kernel resets both for the next
-// substep).  Two cells per thread and iteration (16-byte loads; the arrays are
-// 16-byte aligned), one CTA-wide reduction, then 16 atomics per CTA.
-__global__ void __launch_bounds__(256) fx_stats_kernel(FxPtrs p, long long n,
-                                                       unsigned long long *stats) {
-    unsigned long long hi[NF], lo[NF];
-#pragma unroll
-    for (int q = 0; q < NF; ++q) {
-        hi[q] = 0ull;
-        lo[q] = ~0ull;
-    }
-    const long long n2 = n >> 1;
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n2;
-         t += (long long)gridDim.x * blockDim.x) {
-#pragma unroll
-        for (int q = 0; q < NF; ++q) {
-            const double2 v = __ldg(reinterpret_cast<const double2 *>(p.f[q]) + t);
-            const unsigned long long k0 = fx_key((unsigned long long)__double_as_longlong(v.x));
-            const unsigned long long k1 = fx_key((unsigned long long)__double_as_longlong(v.y));
-            const unsigned long long kh = k0 > k1 ? k0 : k1, kl = k0 > k1 ? k1 : k0;
-            hi[q] = kh > hi[q] ? kh : hi[q];
-            lo[q] = kl < lo[q] ? kl : lo[q];
-        }
-    }
-    if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
-#pragma unroll
-        for (int q = 0; q < NF; ++q) {
-            const unsigned long long k =
-                fx_key((unsigned long long)__double_as_longlong(p.f[q][n - 1]));
-            hi[q] = k > hi[q] ? k : hi[q];
-            lo[q] = k < lo[q] ? k : lo[q];
-        }
-    }
-    __shared__ unsigned long long red[2 * NF];
-    if (threadIdx.x < NF) {
-        red[threadIdx.x] = 0ull;
-        red[NF + threadIdx.x] = ~0ull;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < NF; ++q) {
-        unsigned long long a = hi[q], b = lo[q];
-        for (int o = 16; o > 0; o >>= 1) {
-            const unsigned long long x = __shfl_xor_sync(0xffffffffu, a, o);
-            const unsigned long long y = __shfl_xor_sync(0xffffffffu, b, o);
-            a = x > a ? x : a;
-            b = y < b ? y : b;
-        }
-        if ((threadIdx.x & 31) == 0) {
-            atomicMax(&red[q], a);
-            atomicMin(&red[NF + q], b);
-        }
-    }
-    __syncthreads();
-    if (threadIdx.x < NF)
-        atomicMax(&stats[threadIdx.x], red[threadIdx.x]);
-    else if (threadIdx.x < 2 * NF)
-        atomicMin(&stats[threadIdx.x], red[threadIdx.x]);
-}
-
 // One warp: lane q < NF plans field q (offset, exponent), then the lanes agree
 // on the kernel.  Thread 0 also counts the substep under its mode: plain,
 // per-field (a component more than one binade below its group's largest) or group.
-__global__ void fx_plan_kernel(unsigned long long *stats, FxPlan *plan, double inv_cp,
-                               double gamma_cp, double gm1, int aniso) {
+__device__ __forceinline__ void fx_plan(unsigned long long *stats, FxPlan *plan, double inv_cp,
+                                        double gamma_cp, double gm1, int aniso) {
     const int q = threadIdx.x;
     int bad = 0, zero = 1, e = -100000, ec = -100000;
     double c = 0.0, big = 0.0;
     if (q < NF) {
-        const double hi = fx_unkey(stats[q]), lo = fx_unkey(stats[NF + q]);
+        const double hi = fx_unkey(__ldcg(&stats[q])), lo = fx_unkey(__ldcg(&stats[NF + q]));
         stats[q] = 0ull;        // ready for the next substep's extremes
         stats[NF + q] = ~0ull;
         if (!isfinite(hi) || !isfinite(lo)) {
@@ -254,6 +193,79 @@ __global__ void fx_plan_kernel(unsigned long long *stats, FxPlan *plan, double i
         }
         if (!aniso) plan->taken[mode] += 1ull;
     }
+}
+
+// Per-field extremes of the current state: stats[q] = largest key of field q,
+// stats[NF + q] = its smallest key.  Two cells per thread and iteration (16-byte
+// loads; the arrays are 16-byte aligned), one CTA-wide reduction, then 16 atomics per
+// CTA.  The last CTA to finish (stats[2 NF] counts them) makes the plan of them and
+// resets the words for the next substep: as a kernel of its own the plan was 5 us of a
+// 32^3 substep's 42.
+__global__ void __launch_bounds__(256) fx_stats_kernel(FxPtrs p, long long n, unsigned long long *stats,
+                                                       FxPlan *plan, double inv_cp, double gamma_cp,
+                                                       double gm1, int aniso) {
+    unsigned long long hi[NF], lo[NF];
+#pragma unroll
+    for (int q = 0; q < NF; ++q) {
+        hi[q] = 0ull;
+        lo[q] = ~0ull;
+    }
+    const long long n2 = n >> 1;
+    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < n2;
+         t += (long long)gridDim.x * blockDim.x) {
+#pragma unroll
+        for (int q = 0; q < NF; ++q) {
+            const double2 v = __ldg(reinterpret_cast<const double2 *>(p.f[q]) + t);
+            const unsigned long long k0 = fx_key((unsigned long long)__double_as_longlong(v.x));
+            const unsigned long long k1 = fx_key((unsigned long long)__double_as_longlong(v.y));
+            const unsigned long long kh = k0 > k1 ? k0 : k1, kl = k0 > k1 ? k1 : k0;
+            hi[q] = kh > hi[q] ? kh : hi[q];
+            lo[q] = kl < lo[q] ? kl : lo[q];
+        }
+    }
+    if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
+#pragma unroll
+        for (int q = 0; q < NF; ++q) {
+            const unsigned long long k =
+                fx_key((unsigned long long)__double_as_longlong(p.f[q][n - 1]));
+            hi[q] = k > hi[q] ? k : hi[q];
+            lo[q] = k < lo[q] ? k : lo[q];
+        }
+    }
+    __shared__ unsigned long long red[2 * NF];
+    if (threadIdx.x < NF) {
+        red[threadIdx.x] = 0ull;
+        red[NF + threadIdx.x] = ~0ull;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < NF; ++q) {
+        unsigned long long a = hi[q], b = lo[q];
+        for (int o = 16; o > 0; o >>= 1) {
+            const unsigned long long x = __shfl_xor_sync(0xffffffffu, a, o);
+            const unsigned long long y = __shfl_xor_sync(0xffffffffu, b, o);
+            a = x > a ? x : a;
+            b = y < b ? y : b;
+        }
+        if ((threadIdx.x & 31) == 0) {
+            atomicMax(&red[q], a);
+            atomicMin(&red[NF + q], b);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < NF)
+        atomicMax(&stats[threadIdx.x], red[threadIdx.x]);
+    else if (threadIdx.x < 2 * NF)
+        atomicMin(&stats[threadIdx.x], red[threadIdx.x]);
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&stats[2 * NF], 1ull) == gridDim.x - 1;
+    __syncthreads();
+    if (!last || threadIdx.x >= 32) return;
+    __threadfence();
+    fx_plan(stats, plan, inv_cp, gamma_cp, gm1, aniso);
+    if (threadIdx.x == 0) stats[2 * NF] = 0ull;
 }
 
 // F = round(f 2^s) - round(c 2^s) by integer operations on the binary64 bits, with
@@ -636,25 +648,6 @@ __device__ __forceinline__ void fx_field_column(const SubstepArgs<double, double
             a.fout[q][o] = ldg(a.fin[q] + o) + a.beta * wn;
         }
     }
-}
-
-// Kernel of FX_FIELD.  Each of the plan's three kernels is launched every substep
-// (its own register allocation: with all bodies in one kernel ptxas spilled and it
-// ran 3-10% slower); the two that the plan did not choose return at once.  Two CTAs
-// of 128 threads per SM (8 warps, as many as 255 registers allow).
-template <bool CFL, bool EXT = false>
-__global__ void __launch_bounds__(128, 2) substep_fx_field_kernel(const SubstepArgs<double, double> a,
-                                                                  const FxPtrs fx, FxCoefs fc,
-                                                                  const FxPlan *plan) {
-    if (plan->kern != FX_FIELD) return;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y * blockDim.y + threadIdx.y;
-    const bool active = i < a.g.nx && j < a.g.ny;
-    __shared__ double etab[512];
-    exp_tab_stage(etab);
-    double cfl = 0.0;
-    if (active) fx_field_column<CFL, EXT>(a, fx, fc, plan, etab, i, j, cfl);
-    if (CFL) block_max_to_global(cfl, a.cfl_max);
 }
 
 // ---- FX_GROUP: integer stencils, integer products --------------------------------
@@ -1333,12 +1326,30 @@ __global__ void __launch_bounds__(2 * FXT * FXT, 1)
     if (CFL) block_max_to_global(cfl, a.cfl_max);
 }
 
-// FX_PLAIN: plain binary64 stencils, the arithmetic of AC_STENCIL_FP64.
-template <bool CFL, bool EXT = false>
-__global__ void __launch_bounds__(128) substep_fx_plain_kernel(const SubstepArgs<double, double> a,
-                                                              const FxPlan *plan) {
-    if (plan->kern != FX_PLAIN) return;
-    substep_body<double, double, IdxPeriodic32, CFL, 3, EXT>(a);
+// What FX_GROUP does not take: FX_FIELD (equal spacing only: FIELD), and FX_PLAIN, plain
+// binary64 stencils, the arithmetic of AC_STENCIL_FP64.  Launched every substep beside
+// substep_fx_kernel (its own register allocation: with the group body in one kernel
+// ptxas spilled); whichever the plan did not choose returns at once, which costs a
+// small grid 3.7 us a launch, so these two share one.  Two CTAs of 128 threads per SM
+// (8 warps, as many as 255 registers allow).
+template <bool CFL, bool EXT, bool FIELD>
+__global__ void __launch_bounds__(128, 2) substep_fx_fallback_kernel(const SubstepArgs<double, double> a,
+                                                                     const FxPtrs fx, FxCoefs fc,
+                                                                     const FxPlan *plan) {
+    const int kern = plan->kern;
+    if (kern == FX_GROUP) return;
+    if (!FIELD || kern == FX_PLAIN) {
+        substep_body<double, double, IdxPeriodic32, CFL, 3, EXT>(a);
+        return;
+    }
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = blockIdx.y * blockDim.y + threadIdx.y;
+    const bool active = i < a.g.nx && j < a.g.ny;
+    __shared__ double etab[512];
+    exp_tab_stage(etab);
+    double cfl = 0.0;
+    if (active) fx_field_column<CFL, EXT>(a, fx, fc, plan, etab, i, j, cfl);
+    if (CFL) block_max_to_global(cfl, a.cfl_max);
 }
 
 }  // namespace ac
