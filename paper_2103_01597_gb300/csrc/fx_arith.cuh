@@ -175,7 +175,7 @@ AC_HD long long fx_align(long long b, int E) {
 // ---- conversion -------------------------------------------------------------------
 // v 2^e as binary64, rounded to nearest from the top 64 significant bits (a
 // negative value is first replaced by its one's complement: half a unit of the
-// 96 bits); values below 2^32 units become zero.  eb = e + FX_EB.
+// 96 bits).  eb = e + FX_EB.
 constexpr int FX_EB = 1023 + 95 - 1;
 AC_HD double fx_to_double(const Fx96 &v, int eb) {
     const int th = (int)(v.top >> 32);
@@ -185,9 +185,14 @@ AC_HD double fx_to_double(const Fx96 &v, int eb) {
     h = up ? m : h;
     m = up ? l : m;
     l = up ? 0u : l;
+    // the middle word too: rare, but not rare enough to call it zero (a Laplacian on a
+    // fine grid is some 2^53 units, one in 2^20 of them below 2^32)
+    const bool up2 = h == 0;
+    h = up2 ? m : h;
+    m = up2 ? 0u : m;
     const int c = fx_clz(h);
     const unsigned H = fx_shl_hi(m, h, c), M = fx_shl_hi(l, m, c);  // top bit of H set
-    const int e = eb - c - (up ? 32 : 0);
+    const int e = eb - c - (up ? 32 : 0) - (up2 ? 32 : 0);
     fx_u64 b = (((fx_u64)H << 32) | M) >> 11;
     b += (M >> 10) & 1u;
     b += (fx_u64)(((unsigned)e << 20) + (s & 0x80000000u)) << 32;

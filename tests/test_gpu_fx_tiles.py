@@ -191,3 +191,16 @@ def test_unequal_spacing_left_to_the_plain_stencils(case):
         sim.close()
     for a, b in zip(out, plain):
         assert np.array_equal(a, b, equal_nan=True)
+
+
+def test_small_laplacians():
+    """One cell sets the scale and the rest of u and A lies 2^33 below it, so that the
+    Laplacians' 96-bit numerators there stay below 2^32 units: taken for zero they would
+    be 8e-11 of the largest off."""
+    n = (21, 18, 20)
+    f = np.zeros((8,) + n[::-1])
+    noise = synthetic.noise_state(n, 9, sigma=3.5e-11)
+    for q in (1, 2, 3, 5, 6, 7):
+        f[q] = noise[q]
+        f[q][7, 5, 11] = 0.3 if q % 2 else -0.2
+    _parity(n, f, force_amp=0.0)
