@@ -51,16 +51,16 @@ def bytes_per_cell(elem_f, elem_w, s):
 
 # Nominal dense FP64 rate of one GB300 (no measured FP64 peak is provided).
 FP64_NOMINAL_TFLOPS = 1.25
-# DRAM bytes per cell of one launch of the integer-sum FP64 substep kernel
-# (ncu, 128^3, substep-1/2 variant, over 2,097,152 cells): group scales (forced
-# noise state) 424.2 MB read + 236.7 MB written, per-field scales (u_z scaled by
+# DRAM bytes per cell of one launch of the integer FP64 substep kernel (ncu, 128^3,
+# substep-1/2 variant, over 2,097,152 cells): group scales (forced state) 452.7 MB
+# read + 229.1 MB written; the per-field form of the fallback kernel (u_z scaled by
 # 1e-3) 429.3 + 236.7 MB.
-FX_TRAFFIC_PER_CELL = {"group": (424206592 + 236677888) / 2097152,
+FX_TRAFFIC_PER_CELL = {"group": (452677120 + 229116288) / 2097152,
                        "field": (429260800 + 236704256) / 2097152}
 # FP64-pipe thread instructions per cell of that kernel (ncu
 # sm__inst_executed_pipe_fp64 x 32 / cells, 128^3 forced; the instruction stream
-# does not depend on the grid), per mode: substep-0 (CFL) and substep-1/2 variants.
-FX_FP64_PIPE_INST_PER_CELL = {"group": (206.3125, 179.3125), "field": (236.3125, 209.3125)}
+# does not depend on the grid), per form: substep-0 (CFL) and substep-1/2 variants.
+FX_FP64_PIPE_INST_PER_CELL = {"group": (59.6774, 58.3281), "field": (236.3125, 209.3125)}
 # DRAM bytes per cell of one launch of the binary32 tiled substep, the mean over
 # substeps 0, 1, 2 (ncu, 256^3 forced, one step: 1970.1 MB read + written per
 # launch on average over 16,777,216 cells; algorithmic 96, 128, 128 B/cell)
@@ -543,12 +543,15 @@ def run_ours(args, wl):
         # measured denominator: the library's DFMA-chain probe (2 flops per FMA)
         dfma = ac.ac_diag_fma_rate(ac.AC_FP64, stream.cuda_stream)
         peak = 2 * dfma / 1e12
-        # the count per cell weighted by the modes the timed substeps ran (none
-        # for plain binary64 stencils, which this table does not cover)
+        # the count per cell of the form the timed substeps ran (none for plain
+        # binary64 stencils, which this table does not cover).  A substep counted
+        # under field scales (components more than one binade apart) still runs the
+        # group form up to six binades, so the per-field counts, the larger ones, are
+        # taken only where every substep was counted so.
         inst = None
         traffic = None
         if fixed and order == 6 and sum(modes) and not modes[2] and not wl.get("entropy"):
-            fg = modes[0] / sum(modes)
+            fg = 1.0 if modes[0] else 0.0
             G, F = FX_FP64_PIPE_INST_PER_CELL["group"], FX_FP64_PIPE_INST_PER_CELL["field"]
             inst = [fg * G[v] + (1 - fg) * F[v] for v in range(2)]
             traffic = (fg * FX_TRAFFIC_PER_CELL["group"] +
@@ -567,11 +570,10 @@ def run_ours(args, wl):
                 "peak_source": "measured: ac_diag_fma_rate(AC_FP64), the library's own DFMA "
                                "chains, x 2 flops (nominal: %.2f TFLOP/s)" % FP64_NOMINAL_TFLOPS,
                 # dram read + write per launch of the substep-1/2 variant, from the
-                # 128^3 ncu captures of the same kernels scaled by cells, weighted by
-                # the modes the timed substeps ran
+                # 128^3 ncu captures of the same kernels scaled by cells
                 "traffic": traffic,
-                "kernel": ("fx_stats + fx_plan + fx_quantize + substep_fx_kernel (int64 "
-                           "stencil sums)" if fixed else
+                "kernel": ("fx_stats + fx_quantize + substep_fx_kernel (integer stencils "
+                           "and products)" if fixed else
                            "substep_kernel<double,double,IdxPeriodicR<%d>>" % (order // 2)),
                 "prep_ms": {str(s): prep_ms[s] for s in range(3)},
                 "method_flops_equiv": {
@@ -579,8 +581,8 @@ def run_ours(args, wl):
                     "alg_flops_per_cell_substep": {s: flops_per_cell(order, s)
                                                    for s in range(3)},
                     "note": ("the method's binary64 flops per cell-substep over the launch "
-                             "time; on the integer-sum path the 540 stencil flops run as "
-                             "exact int64 operations on the integer pipes, so this rate can "
+                             "time; on the integer path the stencils and products run as "
+                             "integer operations off the FP64 pipe, so this rate can "
                              "exceed the FP64 peak" if fixed else
                              "all arithmetic on the FP64 pipe")},
                 "fp64_dgemm_measured_tflops": dg,
@@ -1189,8 +1191,8 @@ CF_FLOPS = {1: 2 * 27 * 8 * 32, 2: 2 * 27 * 32 * 32, 3: 2 * 27 * 32 * 8}
 # algorithmic flops per cell (8 real input channels, 8 real output channels)
 CF_ALGO_FLOPS = 2 * 27 * (8 * 32 + 32 * 32 + 32 * 8)
 # DRAM bytes per cell of one launch of the 32 -> 32 tcgen05 layer (ncu, 128^3:
-# 144.9 MB read + 89.0 MB written over 2,097,152 cells)
-CF_TRAFFIC_PER_CELL = (144.937728e6 + 89.045248e6) / 2097152
+# 145.0 MB read + 92.1 MB written over 2,097,152 cells)
+CF_TRAFFIC_PER_CELL = (144.959488e6 + 92.069632e6) / 2097152
 
 
 def _closure_oracle_sample(params, n, seed):
