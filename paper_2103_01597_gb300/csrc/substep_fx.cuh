@@ -664,7 +664,7 @@ __device__ __forceinline__ void fx_field_column(const SubstepArgs<double, double
 // the FP64 pipe, 179 instructions a cell); these integer products with stencil points
 // loaded through L1 5.95 (load latency at 2 warps per scheduler); one thread per cell
 // on the ring 3.72; two threads in lockstep between CTA barriers 4.11; without CTA
-// barriers (FxMarch) 3.40; with the halves balanced 3.18.  Bound now by the issue of
+// barriers (FxMarch) 3.40; with the halves balanced 3.18, 3.22 since conversions take every size.  Bound now by the issue of
 // its 3900 instructions a cell (about half the issue slots; ALU 48%, FP64 pipe 55%).
 constexpr int FXT = 16;                            // tile edge
 constexpr int FXR = FXT + 2 * R;                   // staged row
