@@ -459,7 +459,8 @@ __device__ __forceinline__ Segment segment_of(long long g, const ConvTcArgs &a, 
 //   accf[k]  : the tile in block k is complete (commit after its third slice; one
 //              commit a group measured slower: the epilogues then come in bursts);
 //   acce[k]  : the epilogue warps have read and re-zeroed the GROUP blocks from GROUP k
-//              on (waited on by the producer, so that full[b] says it to the MMA warp);
+//              on, and every producer has seen the phase before (waited on by the
+//              producers, so that full[b] says it to the MMA warp);
 //   wbar     : the layer's weight image landed;
 //   fin      : every MMA of the CTA has finished (before TMEM is freed).
 //
@@ -533,7 +534,7 @@ __global__ void __launch_bounds__(CTHREADS, 1)
             mbar_init(&empty[b], 1);
         }
         for (int b = 0; b < RBLK; ++b) mbar_init(&accf[b], 1);
-        for (int b = 0; b < TGROUPS; ++b) mbar_init(&acce[b], 4 * GROUP);
+        for (int b = 0; b < TGROUPS; ++b) mbar_init(&acce[b], 4 * GROUP + PRODS);
         mbar_init(&wbar, 1);
         mbar_init(&fin, 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -569,8 +570,13 @@ __global__ void __launch_bounds__(CTHREADS, 1)
                     const int cnt = min(GROUP, sg.len + 2 - j);
                     // the blocks this group's tiles open in (if any) have been read and zeroed
                     // (waited for by every producer: a phase that one did not wait for
-                    // would make the next one's parity ambiguous)
-                    if (j < sg.len) ok = mbar_wait(&acce[k], ((gpar >> k) & 1u) ^ 1u);
+                    // would make the next one's parity ambiguous; and each says that it
+                    // has seen the phase, so that the next one cannot complete under a
+                    // producer that lags, whose parity would then mean the one after)
+                    if (j < sg.len) {
+                        ok = mbar_wait(&acce[k], ((gpar >> k) & 1u) ^ 1u);
+                        if (ok) mbar_arrive(&acce[k]);
+                    }
                     if (!ok) break;
                     if (grp % PRODS == own) {
                         if (round > 0) ok = mbar_wait(&empty[grp], (round - 1) & 1);
