@@ -494,6 +494,14 @@ int ac_closure_status(ac_closure *c);
  * usable; AC_OK would mean the wait completed.  `stream` may be NULL;
  * synchronises it. */
 int ac_diag_wait_timeout(unsigned polls, void *stream);
+
+/*
+ * Polls (up to 2^18, the default; about 3.8 us each) after which the handle's
+ * integer-sum substeps give up waiting for their own copies.  A substep that gives up
+ * leaves the state undefined and is reported as AC_ERR_TIMEOUT (ac_set_stencil_mode).
+ * Diagnostic (no counterpart in the paper): 0 makes a substep's first wait run out at once.
+ */
+int ac_diag_substep_polls(ac_handle *h, unsigned polls);
 /* Diagnostic of the table-driven binary64 exp that the binary64 substep
  * kernels use for exp(-ln rho), exp(xi) and exp(-xi) (Tang's method with a
  * 256-entry table; the library exp where |x| >= 700 or x is not finite).

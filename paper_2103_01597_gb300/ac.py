@@ -177,6 +177,7 @@ def load_library(path=None):
         "ac_closure_launch_count": ([_vp, ctypes.POINTER(_c.c_ulonglong)], _c.c_int),
         "ac_closure_set_conv_path": ([_vp, _c.c_int], _c.c_int),
         "ac_diag_wait_timeout": ([_c.c_uint, _vp], _c.c_int),
+        "ac_diag_substep_polls": ([_vp, _c.c_uint], _c.c_int),
         "ac_diag_exp_table": ([_vp, _c.c_longlong, _vp, _vp], _c.c_int),
         "ac_bounds_check_take": ([ctypes.POINTER(_c.c_ulonglong)], _c.c_int),
         "ac_bounds_check_selftest": ([ctypes.POINTER(_c.c_longlong)], _c.c_int),
@@ -520,6 +521,11 @@ def ac_diag_wait_timeout(polls, stream=None):
     """Run the bounded-wait diagnostic; returns the library's status code
     (AC_ERR_TIMEOUT is the expected outcome)."""
     return load_library().ac_diag_wait_timeout(int(polls), stream)
+
+
+def ac_diag_substep_polls(h, polls):
+    """Polls after which the handle's integer-sum substeps give up a wait."""
+    _check(load_library().ac_diag_substep_polls(h, int(polls)), "ac_diag_substep_polls")
 
 
 def ac_diag_exp_table(x, y, stream=None):

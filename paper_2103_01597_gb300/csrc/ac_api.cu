@@ -64,6 +64,7 @@ struct ac_handle {
     CUtensorMap fx_map;           // tensor map over them
     unsigned long long *fx_stats; // per-field extremes of the substep's input (16 words, and a count)
     void *fx_plan;                // device plan of the integer-sum path (mode, scales)
+    unsigned fx_polls;            // polls of a device wait of the integer-sum substep
     double *stage;       // float64 staging for load/store
     size_t stage_elems;
     int next_s;
@@ -158,6 +159,7 @@ extern "C" int ac_init(ac_handle **out, const ac_grid *grid, const ac_params *pa
     h->stream = static_cast<cudaStream_t>(stream);
     h->elem_f = params->precision == AC_FP64 ? 8 : 4;
     h->elem_w = params->precision == AC_FP32 ? 4 : 8;
+    h->fx_polls = FX_WAIT_LIMIT;
     const int ntab = grid->nx + grid->ny + grid->nz;
     cudaError_t e = cudaMalloc(&h->ftab, (size_t)ntab * (sizeof(double2) + sizeof(float2)));
     if (e == cudaSuccess) e = cudaMalloc(&h->partials, sizeof(double) * reduce_max_blocks());
@@ -654,6 +656,12 @@ extern "C" int ac_get_stencil_modes(ac_handle *h, unsigned long long counts[3]) 
     return AC_OK;
 }
 
+extern "C" int ac_diag_substep_polls(ac_handle *h, unsigned polls) {
+    if (!h || polls > FX_WAIT_LIMIT) return AC_ERR_ARG;
+    h->fx_polls = polls;
+    return AC_OK;
+}
+
 extern "C" int ac_get_step(const ac_handle *h, unsigned long long *step, int *next_substep) {
     if (!h) return AC_ERR_ARG;
     if (step) *step = h->step;
@@ -785,6 +793,7 @@ extern "C" int ac_integrate_substep(ac_handle *h, double dt, int s) {
         L.fx_stats = h->fx_stats;
         L.fx_plan = h->fx_plan;
     }
+    L.fx_polls = h->fx_polls;
     L.ev_mid = nullptr;
     cudaEvent_t *tev = nullptr;
     if (h->timing && h->nrec < AC_TIMING_MAX) {

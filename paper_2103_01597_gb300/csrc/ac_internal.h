@@ -103,19 +103,21 @@ struct SubstepLaunch {
     int s;
     unsigned long long *cfl_max;  // substep 0: device word for the max CFL speed (or NULL)
     // binary64 with integer stencil sums (periodic grids): use_fx = 1 for equal spacing,
-    // 2 for unequal; int64 copies of
-    // the fields, padded by their periodic halo, with their tensor map, 16 words of per-field extremes and the device plan of the
-    // substep (fx_plan_bytes()); use_fx = 0 selects plain binary64 sums.
+    // 2 for unequal; int64 copies of the fields, padded by their periodic halo, with their
+    // tensor map, 17 words of per-field extremes and the device plan of the substep
+    // (fx_plan_bytes()); use_fx = 0 selects plain binary64 sums.
     int use_fx;
     void *fx_copies;           // fx_copy_bytes()
     const CUtensorMap *fx_map;
     unsigned long long *fx_stats;
     void *fx_plan;
+    unsigned fx_polls;         // polls of a device wait before it gives up
     double dx[3];
     // optional: recorded after the preparation kernels (integer-sum path:
     // extremes, plan, quantisation), before the substep kernel itself
     cudaEvent_t ev_mid;
 };
+constexpr unsigned FX_WAIT_LIMIT = 1u << 18;  // polls (3.8 us each): a second
 size_t fx_plan_bytes();
 size_t fx_copy_bytes(const Geom &g);
 cudaError_t fx_encode_map(void *base, const Geom &g, CUtensorMap *map);

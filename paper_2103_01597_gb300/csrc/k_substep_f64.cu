@@ -59,14 +59,15 @@ cudaError_t fx_encode_map(void *base, const Geom &g, CUtensorMap *map) {
 
 template <bool CFL, bool EXT, bool ANISO>
 static cudaError_t launch_fx_group(SubstepArgs<double, double> a, const CUtensorMap &map,
-                                   const FxCoefs &fc, FxPlan *plan, cudaStream_t st) {
+                                   const FxCoefs &fc, FxPlan *plan, unsigned polls,
+                                   cudaStream_t st) {
     auto k = substep_fx_kernel<CFL, EXT, ANISO>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FX_SMEM);
     if (e != cudaSuccess) return e;
     const unsigned gx = (a.g.nx + FXT - 1) / FXT, gy = (a.g.ny + FXT - 1) / FXT;
     a.zchunk = fx_zchunk((long long)gx * gy, a.g.nz);
     const dim3 grid(gx, gy, (a.g.nz + a.zchunk - 1) / a.zchunk);
-    k<<<grid, dim3(FXT, FXT, 2), FX_SMEM, st>>>(a, map, fc, plan);
+    k<<<grid, dim3(FXT, FXT, 2), FX_SMEM, st>>>(a, map, fc, plan, polls);
     return cudaGetLastError();
 }
 
@@ -164,8 +165,8 @@ cudaError_t launch_substep_f64(const SubstepLaunch &L, cudaStream_t st, int *lau
     // one kernel per plan; those the plan did not choose return at once
 #define AC_FX(C, X)                                                                \
     do {                                                                           \
-        e = aniso ? launch_fx_group<C, X, true>(a, *L.fx_map, fc, plan, st)        \
-                  : launch_fx_group<C, X, false>(a, *L.fx_map, fc, plan, st);      \
+        e = aniso ? launch_fx_group<C, X, true>(a, *L.fx_map, fc, plan, L.fx_polls, st)   \
+                  : launch_fx_group<C, X, false>(a, *L.fx_map, fc, plan, L.fx_polls, st); \
         if (e != cudaSuccess) return e;                                            \
         if (aniso) substep_fx_fallback_kernel<C, X, false><<<grid, block, 0, st>>>(a, fx, fc, plan); \
         else substep_fx_fallback_kernel<C, X, true><<<grid, block, 0, st>>>(a, fx, fc, plan); \

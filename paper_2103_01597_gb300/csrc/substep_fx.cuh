@@ -676,7 +676,6 @@ constexpr int FX_WARPS = 2 * FXT * FXT / 32;
 constexpr int FX_XCH = 6;                          // doubles a cell's A thread hands to its u thread
 constexpr size_t FX_SMEM =
     (size_t)FX_SLOTS * FX_PLANE_BYTES + 8 * (256 + FX_XCH * FXT * FXT);
-constexpr unsigned FX_WAIT_LIMIT = 1u << 18;       // try_wait polls (3.8 us each) before giving up
 
 __device__ __forceinline__ unsigned fx_smem_u32(const void *p) {
     return (unsigned)__cvta_generic_to_shared(p);
@@ -687,20 +686,23 @@ __device__ __forceinline__ double fx_load_now(const double *p) {
     asm volatile("ld.global.f64 %0, [%1];\n" : "=d"(v) : "l"(p));
     return v;
 }
-// Wait for the phase of `bar` with the given parity; false after FX_WAIT_LIMIT polls.
-__device__ __forceinline__ bool fx_wait(fx_u64 *bar, unsigned parity) {
-    const unsigned a = fx_smem_u32(bar);
-    for (unsigned it = 0; it < FX_WAIT_LIMIT; ++it) {
-        unsigned done;
-        asm volatile(
-            "{\n .reg .pred p;\n"
-            " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-            " selp.u32 %0, 1, 0, p;\n}\n"
-            : "=r"(done)
-            : "r"(a), "r"(parity)
-            : "memory");
-        if (done) return true;
-    }
+// Whether the phase of `bar` with the given parity has completed (a poll that does not
+// find it so returns after about 3.8 us).
+__device__ __forceinline__ bool fx_poll(fx_u64 *bar, unsigned parity) {
+    unsigned done;
+    asm volatile(
+        "{\n .reg .pred p;\n"
+        " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(fx_smem_u32(bar)), "r"(parity)
+        : "memory");
+    return done != 0;
+}
+// Wait for it; false after `polls` polls.
+__device__ __forceinline__ bool fx_wait(fx_u64 *bar, unsigned parity, unsigned polls) {
+    for (unsigned it = 0; it < polls; ++it)
+        if (fx_poll(bar, parity)) return true;
     return false;
 }
 // One plane (padded plane index pz) of the tile whose first staged cell is (x, y).
@@ -923,6 +925,8 @@ struct FxShared {
     fx_u64 given[FX_WARPS / 2];      // the A warp's exchange values are written ...
     fx_u64 taken[FX_WARPS / 2];      // ... and read by the u warp of the same cells
     unsigned done;                   // warps that have finished their stencils (cumulative)
+    unsigned polls;                  // of a wait before it gives up
+    unsigned fetched;                // planes asked for, plane n of them into slot n % FX_SLOTS
     int cfl_low;                     // the CTA's cfl_low below (bits of a positive float)
 };
 struct FxMarch {
@@ -934,9 +938,13 @@ struct FxMarch {
     int last;            // the slot that plane z + 3 is in, and the parity of its fill
     unsigned parity;
     bool ok;             // false once a bounded wait has run out
+    // wait in the march: the limit is only read where the first poll finds nothing
+    __device__ __forceinline__ bool wait(fx_u64 *bar, unsigned p) {
+        return fx_poll(bar, p) || fx_wait(bar, p, *(volatile unsigned *)&sh->polls);
+    }
     // plane z + 3 has landed
     __device__ __forceinline__ bool arrive() {
-        ok = __all_sync(0xffffffffu, fx_wait(&sh->full[last], parity));
+        ok = __all_sync(0xffffffffu, wait(&sh->full[last], parity));
         return ok;
     }
     // this warp has taken its stencils of plane z; once all have, plane z - 3's slot
@@ -948,6 +956,7 @@ struct FxMarch {
             const unsigned n = atomicAdd(&sh->done, 1u) + 1u;
             if (n == FX_WARPS * (unsigned)(z - z0 + 1) && z + 1 < z1) {
                 __threadfence_block();
+                atomicAdd(&sh->fetched, 1u);
                 fx_fetch(sm + slot[0], map, &sh->full[last == FX_SLOTS - 1 ? 0 : last + 1], x0, y0,
                          z + 7);
             }
@@ -1092,7 +1101,7 @@ __device__ __forceinline__ void fx_march_a(const SubstepArgs<double, double> &a,
             rs += rho_inv * (fc.K_dt * lapxi + fc.K_c1sq * gxi2);
         }
         // the u warp has read the values of the plane before
-        if (z > z0) m.ok = __all_sync(0xffffffffu, fx_wait(taken, (z - z0 - 1) & 1)) && m.ok;
+        if (z > z0) m.ok = __all_sync(0xffffffffu, m.wait(taken, (z - z0 - 1) & 1)) && m.ok;
 #pragma unroll
         for (int q = 0; q < 3; ++q) xch[q * FXT * FXT] = pl[q];
         xch[3 * FXT * FXT] = h;
@@ -1253,7 +1262,7 @@ __device__ __forceinline__ void fx_march_u(const SubstepArgs<double, double> &a,
         }
         if (EXT) h = fma(fc.inv_T_ref * fc.zeta_c1sq * divu, divu, h);
         // the other thread's terms
-        m.ok = __all_sync(0xffffffffu, fx_wait(given, (z - z0) & 1)) && m.ok;
+        m.ok = __all_sync(0xffffffffu, m.wait(given, (z - z0) & 1)) && m.ok;
         double x[FX_XCH];
 #pragma unroll
         for (int q = 0; q < FX_XCH; ++q) x[q] = xch[q * FXT * FXT];
@@ -1271,7 +1280,7 @@ __device__ __forceinline__ void fx_march_u(const SubstepArgs<double, double> &a,
 template <bool CFL, bool EXT, bool ANISO>
 __global__ void __launch_bounds__(2 * FXT * FXT, 1)
     substep_fx_kernel(const SubstepArgs<double, double> a, const __grid_constant__ CUtensorMap map,
-                      const FxCoefs fc, FxPlan *plan) {
+                      const FxCoefs fc, FxPlan *plan, unsigned polls) {
     if (plan->kern != FX_GROUP) return;
     extern __shared__ __align__(128) unsigned char fx_smem[];
     __shared__ FxShared sh;
@@ -1292,6 +1301,8 @@ __global__ void __launch_bounds__(2 * FXT * FXT, 1)
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(fx_smem_u32(bars + b))
                          : "memory");
         sh.done = 0;
+        sh.fetched = FX_SLOTS;
+        sh.polls = polls;
         if (CFL) {
             const double g = __longlong_as_double(
                 (long long)*reinterpret_cast<volatile unsigned long long *>(a.cfl_max));
@@ -1307,7 +1318,7 @@ __global__ void __launch_bounds__(2 * FXT * FXT, 1)
 #pragma unroll
     for (int d = 0; d < FX_SLOTS; ++d) m.slot[d] = d * FX_PLANE;
     m.ok = true;
-    for (int d = 0; d < FX_SLOTS - 1; ++d) m.ok = fx_wait(&sh.full[d], 0) && m.ok;
+    for (int d = 0; d < FX_SLOTS - 1; ++d) m.ok = fx_wait(&sh.full[d], 0, polls) && m.ok;
     m.ok = __all_sync(0xffffffffu, m.ok);
     m.last = FX_SLOTS - 1;
     m.parity = 0;
@@ -1319,9 +1330,13 @@ __global__ void __launch_bounds__(2 * FXT * FXT, 1)
         else
             fx_march_u<EXT, ANISO>(a, fc, plan, xch, m, i, j);
     }
-    if (!m.ok) {  // report, and let no copy be in flight when the CTA ends
+    // a wait that ran out is reported, and no copy may be in flight when the CTA ends: with
+    // every warp out of the march no plane is asked for any more, and the last fill of
+    // each slot is waited for
+    if (__syncthreads_or(!m.ok) && tid == 0) {
         atomicExch(&plan->err, 1);
-        for (int d = 0; d < FX_SLOTS; ++d) fx_wait(&sh.full[d], d <= m.last ? m.parity : m.parity ^ 1);
+        for (unsigned n = sh.fetched - FX_SLOTS; n < sh.fetched; ++n)
+            fx_wait(&sh.full[n % FX_SLOTS], (n / FX_SLOTS) & 1, FX_WAIT_LIMIT);
     }
     if (CFL) block_max_to_global(cfl, a.cfl_max);
 }
