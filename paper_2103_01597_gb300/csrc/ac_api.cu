@@ -121,6 +121,15 @@ int ac::valid_params(const ac_params *p) {
     return 1;
 }
 
+cudaError_t ac::zero_now(void *p, size_t bytes) {
+    cudaStream_t st = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return e;
+    e = cudaMemsetAsync(p, 0, bytes, st);
+    const cudaError_t s = cudaStreamSynchronize(st), d = cudaStreamDestroy(st);
+    return e != cudaSuccess ? e : (s != cudaSuccess ? s : d);
+}
+
 static void free_timing(ac_handle *h) {
     if (!h->tev) return;
     for (int i = 0; i < 3 * AC_TIMING_MAX; ++i)
@@ -165,11 +174,11 @@ extern "C" int ac_init(ac_handle **out, const ac_grid *grid, const ac_params *pa
     if (e == cudaSuccess) e = cudaMalloc(&h->partials, sizeof(double) * reduce_max_blocks());
     const size_t flag_bytes = sizeof(unsigned int) * (reduce_max_blocks() + 1);
     if (e == cudaSuccess) e = cudaMalloc(&h->flags, flag_bytes);
-    if (e == cudaSuccess) e = cudaMemset(h->flags, 0, flag_bytes);
+    if (e == cudaSuccess) e = zero_now(h->flags, flag_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&h->result_dev, 2 * sizeof(double));
     if (e == cudaSuccess) e = cudaMallocHost(&h->result_host, 2 * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&h->cfl_dev, sizeof(unsigned long long));
-    if (e == cudaSuccess) e = cudaMemset(h->cfl_dev, 0, sizeof(unsigned long long));
+    if (e == cudaSuccess) e = zero_now(h->cfl_dev, sizeof(unsigned long long));
     if (e != cudaSuccess) {
         int rc = cuda_fail(e);
         free_handle_memory(h);

@@ -159,6 +159,10 @@ struct ReduceLaunch {
     int blocks;
 };
 int reduce_max_blocks();
+// Zeroes new device memory before it returns, behind no other stream's work: what a
+// kernel on any stream relies on later (a memset on the default stream would be ordered
+// with neither a non-blocking stream nor the host).
+cudaError_t zero_now(void *p, size_t bytes);
 cudaError_t launch_reduce(const ReduceLaunch &L, cudaStream_t st, int *launches);
 
 // Record a CUDA error for ac_last_cuda_error() and map it to an AC_ERR_* code.

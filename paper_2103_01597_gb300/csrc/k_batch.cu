@@ -301,7 +301,7 @@ extern "C" int ac_batch_init(ac_batch **out, int nbox, const ac_box *boxes, cons
     if (e == cudaSuccess) e = cudaMalloc(&b->partials, sizeof(double) * reduce_max_blocks());
     const size_t flag_bytes = sizeof(unsigned int) * (reduce_max_blocks() + 1);
     if (e == cudaSuccess) e = cudaMalloc(&b->flags, flag_bytes);
-    if (e == cudaSuccess) e = cudaMemset(b->flags, 0, flag_bytes);
+    if (e == cudaSuccess) e = zero_now(b->flags, flag_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&b->result_dev, 2 * sizeof(double));
     if (e == cudaSuccess) e = cudaMallocHost(&b->result_host, 2 * sizeof(double));
     int dev = 0, sms = 152, occ = 1;
