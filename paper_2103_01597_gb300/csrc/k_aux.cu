@@ -601,6 +601,14 @@ __device__ __forceinline__ void red_cfl_exact(const double *const *f, const IX &
     if (v == v) atomicMax(word, (fx_u64)__double_as_longlong(v));
 }
 
+// A block's non-finite cells noted in the flag word after the maximum.  Every kernel that
+// takes exact speeds notes its own: once an infinity is in the word, later cells of the
+// search compare against it.
+__device__ __forceinline__ void red_cfl_flag(unsigned int bad, fx_u64 *word) {
+    if (__syncthreads_or(bad) && threadIdx.x + threadIdx.y == 0)
+        atomicOr(reinterpret_cast<unsigned int *>(word + 1), 1u);
+}
+
 // A first guess: the speeds of one cell in 8 x 8 x 4 (y, z, x).
 template <class IX>
 __global__ void __launch_bounds__(RED_THREADS) reduce_cfl_sample_kernel(PtrPack<const double> pk,
@@ -617,6 +625,7 @@ __global__ void __launch_bounds__(RED_THREADS) reduce_cfl_sample_kernel(PtrPack<
         ix.set_z((int)(r / ny) * 8, g);
         red_cfl_exact(pk.p, ix, k, word, bad);
     }
+    red_cfl_flag(bad, word);
 }
 
 // v in binary32 towards zero; infinite or NaN, and |v| from 2^128 on, as infinity.
@@ -680,8 +689,7 @@ __global__ void __launch_bounds__(RED_THREADS, 2)
             if (!(up <= known)) red_cfl_exact(f, ix, k, word, bad);
         }
     }
-    if (__syncthreads_or(bad) && threadIdx.x + threadIdx.y == 0)
-        atomicOr(reinterpret_cast<unsigned int *>(word + 1), 1u);
+    red_cfl_flag(bad, word);
     if (red_last_block(out.flags + RED_MAX_BLOCKS) && threadIdx.x + threadIdx.y == 0) {
         const fx_u64 w = __ldcg(word);
         const unsigned int b = __ldcg(reinterpret_cast<unsigned int *>(word + 1));
