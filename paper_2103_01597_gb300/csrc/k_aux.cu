@@ -1,6 +1,7 @@
 // Auxiliary kernels: periodic halo fill (Sec. 3.3), forcing phase tables,
 // host-format staging (load/store with precision conversion), and binary64
 // reductions of fields and derived quantities.
+#include <float.h>
 #include <math.h>
 
 #include "fx_arith.cuh"
@@ -628,7 +629,8 @@ __global__ void __launch_bounds__(RED_THREADS) reduce_cfl_sample_kernel(PtrPack<
     red_cfl_flag(bad, word);
 }
 
-// v in binary32 towards zero; infinite or NaN, and |v| from 2^128 on, as infinity.
+// v in binary32 towards zero, but infinite or NaN, and |v| from 2^128 on, as infinity:
+// a bound formed of such values is infinite or NaN.
 __device__ __forceinline__ float red_float(double v) {
     const int hi = __double2hiint(v), a = hi & 0x7fffffff;
     int r = ((a - 0x38000000) << 3) | (int)((unsigned)__double2loint(v) >> 29);
@@ -684,8 +686,10 @@ __global__ void __launch_bounds__(RED_THREADS, 2)
             float up = 1.0001f * (sqrtf(ux * ux + uy * uy + uz * uz + 1e-37f) +
                                   sqrtf(cs2 + (Bx * Bx + By * By + Bz * Bz + 1e-37f) * ri));
             if (!(fabsf(a + b) <= 60.f && fabsf(l) <= 60.f)) up = INFINITY;
-            const float known = red_float(__longlong_as_double(
-                (long long)*reinterpret_cast<volatile fx_u64 *>(word)));
+            // (at most binary32's largest number: an infinite bound is never below it, and
+            // the cell's exact speed is taken, however large the known one)
+            const float known = fminf(red_float(__longlong_as_double((long long)*
+                                      reinterpret_cast<volatile fx_u64 *>(word))), FLT_MAX);
             if (!(up <= known)) red_cfl_exact(f, ix, k, word, bad);
         }
     }

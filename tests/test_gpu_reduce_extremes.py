@@ -1,8 +1,10 @@
 """The search for the largest CFL speed of binary64 states, where a cell of its first guess
-is not finite.
+is not finite and where speeds leave binary32's range (1e-12 relative, the bound of
+test_gpu_substep.py).
 """
 import math
 
+import numpy as np
 import pytest
 import torch
 
@@ -12,6 +14,7 @@ pytestmark = pytest.mark.gpu
 
 PHYS = dict(nu=5e-3, eta=5e-3, cs0=1.2, gamma=1.4, cp=1.1, lnrho0=0.1)
 LARGE = (48, 40, 36)  # 69120 cells: the search starts from a guess on every 4th, 8th, 8th cell
+SMALL = (20, 18, 16)
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -45,4 +48,27 @@ def test_nonfinite_cell_of_the_first_guess_is_reported(bad, at):
             with pytest.raises(ac.AcError) as ei:
                 sim.reduce(ac.AC_MAX, ac.AC_Q_CFL)
             assert ei.value.code == ac.AC_ERR_NONFINITE, q
+        sim.close()
+
+
+CELLS = [(0, 0, 0), (1, 2, 3), (8, 8, 8), (9, 7, 5), (15, 17, 19)]
+
+
+@pytest.mark.parametrize("n", [SMALL, LARGE])
+@pytest.mark.parametrize("low", CELLS)
+def test_speeds_beyond_binary32(n, low):
+    """A speed of 1e40 at one cell, a larger one or an infinity at another."""
+    for high in CELLS:
+        if high == low:
+            continue
+        f = _state(n)
+        f[1][low], f[2][high] = 1e40, 1e50
+        sim = _sim(n, f)
+        got = sim.reduce(ac.AC_MAX, ac.AC_Q_CFL)
+        assert abs(got - 1e50) <= 1e-12 * 1e50, (high, got)
+        f[2][high] = np.inf
+        sim.load(f)
+        with pytest.raises(ac.AcError) as ei:
+            sim.reduce(ac.AC_MAX, ac.AC_Q_CFL)
+        assert ei.value.code == ac.AC_ERR_NONFINITE, high
         sim.close()
