@@ -273,9 +273,7 @@ cudaError_t launch_gather_f32(const void *src, int elem_size, const Geom &g, int
 // reduce_cells_kernel, bound by memory.  E_M sums and, in binary32, the CFL speed go
 // through reduce_curl_kernel, whose threads march along z (the periodic offsets of x and
 // y are set once).  In binary64 an FP64-pipe instruction costs a warp about 78 cycles, so
-// the curl is taken in integers there: the 36 values around a cell are aligned to the
-// largest exponent among them (56 bits), their numerators and |B|^2 are exact
-// (fx_arith.cuh).  The largest CFL speed (reduce_cfl_max_kernel) is searched with a
+// the six derivatives of the curl are taken in integers there (fx_arith.cuh).  The largest CFL speed (reduce_cfl_max_kernel) is searched with a
 // binary32 upper bound, exact binary64 speeds only where it exceeds the largest known.
 // The rest (max and min of E_K and E_M, other orders, CFL sums) takes the general kernel.
 // Measured at 256^3 in binary64, host time of one call each: E_K 245 us, E_M 883, rms |u|
@@ -509,18 +507,15 @@ static long long red_tiles(const Geom &g) {
     return (long long)((g.nx + 31) / 32) * ((g.ny + 7) / 8) * ((g.nz + RED_Z - 1) / RED_Z);
 }
 
-// Spacing factors of the integer curl: numerators of axis a times h / dx_a, h the smallest
-// spacing (hi 2^-31 + lo 2^-62), and 1 / (60 h).
-struct RedCurl {
-    int rh[3], rl[3];
-    double c1;
-};
-
 // |B|^2 at a cell from integers; binary64 stencils where an exponent is out of range
-// (non-finite values among them).
+// (non-finite values among them).  Each derivative has a scale of its own, the largest
+// exponent among its six values: a uniform part of A, or another component's size, then
+// takes no bits from it.  Values within three binades of that exponent are exact (a
+// smaller one keeps the bits that a binary64 difference with the largest would keep, and
+// three more), the numerator is their exact sum, rounded once to binary64.
 template <class IX>
 __device__ __forceinline__ double red_curl2(const double *const *f, const IX &ix,
-                                            const DevCoefs<double> &k, const RedCurl &rc) {
+                                            const DevCoefs<double> &k) {
     // derivative of A_q along axis a, d = 0..5 for the points -3 .. 3
     constexpr int Q[6] = {2, 1, 0, 2, 1, 0}, A[6] = {1, 2, 2, 0, 0, 1};
     double v[6][6];
@@ -531,42 +526,49 @@ __device__ __forceinline__ double red_curl2(const double *const *f, const IX &ix
             const int m = d < 3 ? d - 3 : d - 2;
             v[t][d] = ldg(f[5 + Q[t]] + ix(A[t] == 0 ? m : 0, A[t] == 1 ? m : 0, A[t] == 2 ? m : 0));
         }
-    int top = 0;
+    int E[6];
+    bool out = false;  // beyond 2^+-200
 #pragma unroll
-    for (int t = 0; t < 6; ++t)
+    for (int t = 0; t < 6; ++t) {
+        int top = 0;
 #pragma unroll
         for (int d = 0; d < 6; ++d) {
             const int h = __double2hiint(v[t][d]) & 0x7fffffff;
             top = h > top ? h : top;
         }
-    const int E = top >> 20;
-    if (E >= 1223 || E < 823) {  // beyond 2^+-200
-        if (top == 0) return 0.0;
+        E[t] = top >> 20;
+        out |= E[t] >= 1223 || (E[t] < 823 && top > 0);
+        E[t] = E[t] < 823 ? 823 : E[t];  // all zero
+    }
+    double B[3];
+    if (out) {
         const GlobalView<double, IX> ax{f[5], ix}, ay{f[6], ix}, az{f[7], ix};
-        const double Bx = op_d1<1>(az, k.d1[1]) - op_d1<2>(ay, k.d1[2]);
-        const double By = op_d1<2>(ax, k.d1[2]) - op_d1<0>(az, k.d1[0]);
-        const double Bz = op_d1<0>(ay, k.d1[0]) - op_d1<1>(ax, k.d1[1]);
-        return Bx * Bx + By * By + Bz * Bz;
-    }
-    long long d[6];
+        B[0] = op_d1<1>(az, k.d1[1]) - op_d1<2>(ay, k.d1[2]);
+        B[1] = op_d1<2>(ax, k.d1[2]) - op_d1<0>(az, k.d1[0]);
+        B[2] = op_d1<0>(ay, k.d1[0]) - op_d1<1>(ax, k.d1[1]);
+    } else {
+        double d[6];
 #pragma unroll
-    for (int t = 0; t < 6; ++t) {
-        long long F[6];
+        for (int t = 0; t < 6; ++t) {
+            long long F[6];
 #pragma unroll
-        for (int p = 0; p < 6; ++p) F[p] = fx_align(fx_double_to_bits(v[t][p]), E);
-        const long long n = 45 * (F[3] - F[2]) + 9 * (F[1] - F[4]) + (F[5] - F[0]);
-        d[t] = fx_mulfrac(n >> 3, rc.rh[A[t]], rc.rl[A[t]]);
+            for (int p = 0; p < 6; ++p) F[p] = fx_align(fx_double_to_bits(v[t][p]), E[t]);
+            const long long n = 45 * (F[3] - F[2]) + 9 * (F[1] - F[4]) + (F[5] - F[0]);
+            d[t] = fx_to_double(n, FX_EB64 + E[t] - 1078);
+        }
+        // (the weight of the outermost points is 1 / (60 dx))
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            B[q] = d[2 * q] * k.d1[A[2 * q]][2] - d[2 * q + 1] * k.d1[A[2 * q + 1]][2];
     }
-    const FxSplit B[3] = {fx_split(d[0] - d[1]), fx_split(d[2] - d[3]), fx_split(d[4] - d[5])};
-    const double b2 = fx_to_double(fx_dot3(B, B), FX_EB + 38 + 2 * (E - 1078));
-    return b2 * (rc.c1 * rc.c1);
+    return B[0] * B[0] + B[1] * B[1] + B[2] * B[2];
 }
 
 // E_M (CFL = false), or the CFL speed of binary32 fields, over marching threads.
 template <typename R, class IX, bool CFL>
 __global__ void __launch_bounds__(RED_THREADS, 2)
-    reduce_curl_kernel(PtrPack<const R> pk, Geom g, DevCoefs<R> k, RedCurl rc, int op, double count,
-                       long long tiles, RedOut out) {
+    reduce_curl_kernel(PtrPack<const R> pk, Geom g, DevCoefs<R> k, int op, double count, long long tiles,
+                       RedOut out) {
     double acc = red_init(op);
     unsigned int bad = 0;
     for (long long t = blockIdx.x; t < tiles; t += gridDim.x) {
@@ -578,7 +580,7 @@ __global__ void __launch_bounds__(RED_THREADS, 2)
             ix.set_z(z, g);
             double v;
             if constexpr (sizeof(R) == 8)
-                v = 0.5 * red_curl2(pk.p, ix, k, rc);
+                v = 0.5 * red_curl2(pk.p, ix, k);
             else
                 v = cell_quantity<R, IX>(pk.p, ix, k, CFL ? AC_Q_CFL : AC_Q_EMAG);
             if (red_nonfinite(v)) bad = 1;
@@ -730,30 +732,22 @@ static bool launch_curl(const ReduceLaunch &L, const PtrPack<const R> &pk, const
     const long long tiles = red_tiles(L.g);
     const unsigned nb = (unsigned)(tiles < RED_MAX_BLOCKS ? tiles : RED_MAX_BLOCKS);
     const bool sum = L.op == AC_SUM || L.op == AC_RMS;
-    RedCurl rc = {};
-    if (sizeof(R) == 8) {
-        double lo = L.dx[0], hi = L.dx[0];
-        for (int a = 1; a < 3; ++a) {
-            lo = fmin(lo, L.dx[a]);
-            hi = fmax(hi, L.dx[a]);
-        }
-        if (!(hi <= 8.0 * lo) || !(lo >= 1e-12 && hi <= 1e12)) return false;
-        for (int a = 0; a < 3; ++a) fx_fraction(lo / L.dx[a], &rc.rh[a], &rc.rl[a]);
-        rc.c1 = 1.0 / (60.0 * lo);
-    }
     if (L.quantity == AC_Q_EMAG) {
         if (!sum) return false;
-        reduce_curl_kernel<R, IX, false><<<nb, dim3(32, 8), 0, st>>>(pk, L.g, k, rc, L.op, count, tiles, out);
+        reduce_curl_kernel<R, IX, false><<<nb, dim3(32, 8), 0, st>>>(pk, L.g, k, L.op, count, tiles, out);
         ++*launches;
         *err = cudaGetLastError();
         return true;
     }
     if constexpr (sizeof(R) == 8) {
-        // (the binary32 bound wants c_s of ordinary magnitude)
-        if (L.op != AC_MAX || !(L.ph.cs2_ref >= 1e-10 && L.ph.cs2_ref <= 1e10)) return false;
+        // (the binary32 bound wants c_s and the spacings of ordinary magnitude)
+        const double lo = fmin(L.dx[0], fmin(L.dx[1], L.dx[2])), hi = fmax(L.dx[0], fmax(L.dx[1], L.dx[2]));
+        if (L.op != AC_MAX || !(L.ph.cs2_ref >= 1e-10 && L.ph.cs2_ref <= 1e10) || !(hi <= 8.0 * lo) ||
+            !(lo >= 1e-12 && hi <= 1e12))
+            return false;
         *err = launch_cfl_max<IX>(L, pk, k, out, nb, tiles, st, launches);
     } else {
-        reduce_curl_kernel<R, IX, true><<<nb, dim3(32, 8), 0, st>>>(pk, L.g, k, rc, L.op, count, tiles, out);
+        reduce_curl_kernel<R, IX, true><<<nb, dim3(32, 8), 0, st>>>(pk, L.g, k, L.op, count, tiles, out);
         ++*launches;
         *err = cudaGetLastError();
     }

@@ -1,6 +1,10 @@
-"""The search for the largest CFL speed of binary64 states, where a cell of its first guess
-is not finite and where speeds leave binary32's range (1e-12 relative, the bound of
-test_gpu_substep.py).
+"""The binary64 reductions that search or align: the largest CFL speed where a cell of the
+first guess is not finite and where speeds leave binary32's range, and E_M where a part
+of A is uniform or one component is far smaller than another.
+
+CFL speeds: 1e-12 relative to the oracle, the bound of test_gpu_substep.py.  E_M: 1e-14
+relative to the same stencils in extended precision on the stored values (a cell's |B|^2
+carries some eight roundings, its sum over the cells some forty).
 """
 import math
 
@@ -72,3 +76,37 @@ def test_speeds_beyond_binary32(n, low):
             sim.reduce(ac.AC_MAX, ac.AC_Q_CFL)
         assert ei.value.code == ac.AC_ERR_NONFINITE, high
         sim.close()
+
+
+def _b2(A, h):
+    """|curl A|^2 in extended precision, sixth order."""
+    A = A.astype(np.longdouble)
+
+    def d1(f, a):
+        ax = 2 - a
+        s = sum(w * (np.roll(f, -m, ax) - np.roll(f, m, ax)) for m, w in ((1, 45), (2, -9), (3, 1)))
+        return s / (60 * np.longdouble(h[a]))
+
+    B = [d1(A[2], 1) - d1(A[1], 2), d1(A[0], 2) - d1(A[2], 0), d1(A[1], 0) - d1(A[0], 1)]
+    return B[0] ** 2 + B[1] ** 2 + B[2] ** 2
+
+
+@pytest.mark.parametrize("offset,amps", [((0, 0, 0), (1, 1, 1)), ((0, 0, 1e4), (1, 1, 1)),
+                                         ((0, 0, 1e6), (1, 1, 1)), ((1, 1, 1), (1e-8, 1e-8, 1e-8)),
+                                         ((1, 0, 0), (0, 1e-4, 1e-4)), ((1, 0, 0), (0, 1e-8, 1e-8)),
+                                         ((0, 0, 0), (1, 1e-8, 1e-8)), ((3, 0, 0), (0, 0, 1e-10))])
+@pytest.mark.parametrize("L", [(2 * math.pi,) * 3, (2 * math.pi, 3.0, 11.0), (2.0, 40.0, 3.0)])
+def test_magnetic_energy_with_uniform_parts(offset, amps, L):
+    """A_x varies along x only where it is the large one, so that it adds nothing to B."""
+    n = (32, 30, 28)
+    f = np.zeros((8,) + n[::-1])
+    z, y, x = np.meshgrid(*[np.arange(m) * 2 * np.pi / m for m in n[::-1]], indexing="ij")
+    waves = (np.cos(x + 0.3) if amps[1] < amps[0] else np.sin(y - 2 * z + 0.4) + 0.5 * np.cos(z + 1.0),
+             np.sin(z + 2 * x + 0.1) + 0.3 * np.cos(x - 1.2), np.cos(x - y + 0.7) + 0.4 * np.sin(2 * y))
+    for q in range(3):
+        f[5 + q] = offset[q] + amps[q] * waves[q]
+    want = float(0.5 * np.sum(_b2(f[5:8], [L[a] / n[a] for a in range(3)])))
+    sim = _sim(n, f, L=L)
+    got = sim.reduce(ac.AC_SUM, ac.AC_Q_EMAG)
+    sim.close()
+    assert want > 0 and abs(got - want) <= 1e-14 * want, (got, want, abs(got - want) / want)
