@@ -145,8 +145,8 @@ cudaError_t launch_substep_f64(const SubstepLaunch &L, cudaStream_t st, int *lau
     const long long n = L.g.elems;
     FxPlan *plan = static_cast<FxPlan *>(L.fx_plan);
     cudaError_t e;
-    fx_stats_kernel<<<fx_grid(n / 2), 256, 0, st>>>(fx, n, L.fx_stats, plan, L.ph.inv_cp, L.ph.gamma_cp,
-                                                   L.ph.gm1, aniso);
+    fx_stats_kernel<<<fx_grid(n / 2), 256, 0, st>>>(fx, n, L.fx_stats, plan, L.ph.gamma_cp, L.ph.gm1,
+                                                   aniso);
     fx_quantize_kernel<<<fx_grid(32ll * fx.py * fx.pz), 256, 0, st>>>(fx, L.g, plan);
     if (L.ev_mid) {
         e = cudaEventRecord(L.ev_mid, st);

@@ -100,11 +100,6 @@ struct FxPlan {
     int zero[NF];              // constant field: F = 0
     int s[NF];                 // F = round((f - c) 2^s), s = b - E
     unsigned long long C[NF];  // round(c 2^s) modulo 2^64
-    // grad(ln rho + s / c_p) = pi_f 2^-s (big + rho small), big the larger-scaled of
-    // the two gradients, rho = pi_rh 2^-31 + pi_rl 2^-62 <= 1 (FX_GROUP)
-    int pi_s;                  // 1: s is the larger-scaled one
-    int pi_rh, pi_rl;
-    double pi_f;
     unsigned long long taken[3];  // substeps counted in each mode (cumulative)
     int err;                   // set if a bounded wait of the substep kernel ran out
 };
@@ -112,8 +107,8 @@ struct FxPlan {
 // One warp: lane q < NF plans field q (offset, exponent), then the lanes agree
 // on the kernel.  Thread 0 also counts the substep under its mode: plain,
 // per-field (a component more than one binade below its group's largest) or group.
-__device__ __forceinline__ void fx_plan(unsigned long long *stats, FxPlan *plan, double inv_cp,
-                                        double gamma_cp, double gm1, int aniso) {
+__device__ __forceinline__ void fx_plan(unsigned long long *stats, FxPlan *plan, double gamma_cp,
+                                        double gm1, int aniso) {
     const int q = threadIdx.x;
     int bad = 0, zero = 1, e = -100000, ec = -100000;
     double c = 0.0, big = 0.0;
@@ -171,26 +166,8 @@ __device__ __forceinline__ void fx_plan(unsigned long long *stats, FxPlan *plan,
         plan->s[q] = s;
         plan->C[q] = fx_round_grid((unsigned long long)__double_as_longlong(c), s);
     }
-    const int s0 = __shfl_sync(0xffffffffu, s, 0), s4 = __shfl_sync(0xffffffffu, s, 4);
-    const int z0 = __shfl_sync(0xffffffffu, zero, 0), z4 = __shfl_sync(0xffffffffu, zero, 4);
     if (q == 0) {
         plan->kern = kern;
-        if (kern == FX_GROUP) {
-            // ratio of the scales of grad s / c_p and grad ln rho
-            const double ratio = ldexp(inv_cp, s0 - s4);
-            const int pi_s = z0 ? 1 : (z4 ? 0 : ratio >= 1.0);
-            const double rho = z0 || z4 ? 0.0 : (pi_s ? 1.0 / ratio : ratio);
-            int rh = 0x7fffffff, rl = 0x7fffffff;
-            if (rho < 1.0) {
-                const double t = rho * 2147483648.0;
-                rh = (int)t;
-                rl = (int)((t - (double)rh) * 2147483648.0);
-            }
-            plan->pi_s = pi_s;
-            plan->pi_rh = rh;
-            plan->pi_rl = rl;
-            plan->pi_f = pi_s ? inv_cp : 1.0;
-        }
         if (!aniso) plan->taken[mode] += 1ull;
     }
 }
@@ -202,8 +179,8 @@ __device__ __forceinline__ void fx_plan(unsigned long long *stats, FxPlan *plan,
 // resets the words for the next substep: as a kernel of its own the plan was 5 us of a
 // 32^3 substep's 42.
 __global__ void __launch_bounds__(256) fx_stats_kernel(FxPtrs p, long long n, unsigned long long *stats,
-                                                       FxPlan *plan, double inv_cp, double gamma_cp,
-                                                       double gm1, int aniso) {
+                                                       FxPlan *plan, double gamma_cp, double gm1,
+                                                       int aniso) {
     unsigned long long hi[NF], lo[NF];
 #pragma unroll
     for (int q = 0; q < NF; ++q) {
@@ -264,7 +241,7 @@ __global__ void __launch_bounds__(256) fx_stats_kernel(FxPtrs p, long long n, un
     __syncthreads();
     if (!last || threadIdx.x >= 32) return;
     __threadfence();
-    fx_plan(stats, plan, inv_cp, gamma_cp, gm1, aniso);
+    fx_plan(stats, plan, gamma_cp, gm1, aniso);
     if (threadIdx.x == 0) stats[2 * NF] = 0ull;
 }
 
@@ -988,10 +965,8 @@ __device__ __forceinline__ void fx_march_a(const SubstepArgs<double, double> &a,
                                            FxMarch &m, int i, int j, double &cfl) {
     const bool active = i < a.g.nx && j < a.g.ny;
     const int kl = -plan->s[0], ku = -plan->s[1], ks = -plan->s[4], ka = -plan->s[5];
-    const bool pi_s = plan->pi_s != 0;
-    const int pi_rh = plan->pi_rh, pi_rl = plan->pi_rl;
     const long long Cu[3] = {(long long)plan->C[1], (long long)plan->C[2], (long long)plan->C[3]};
-    const double c1cs2_ref = fc.c1dt * a.k.cs2_ref * plan->pi_f;
+    const double c1cs2_ref = fc.c1dt * a.k.cs2_ref;
     // sh->cfl_low: the largest CFL speed known so far, rounded down (the CTA's own and,
     // from the start, what other CTAs have reported); cells whose upper bound lies below
     // it need no exact speed (two square roots: 1150 FP64-pipe cycles)
@@ -1068,7 +1043,9 @@ __device__ __forceinline__ void fx_march_a(const SubstepArgs<double, double> &a,
         const double rho_inv = fx_exp55(-fx_from_double55(lnrho), etab, FX_L70);
         const double exi = fx_exp55(xx, etab, FX_L70), emxi = fx_exp55(-xx, etab, FX_L70);
         const double cjb = rho_inv * fc.jb, cp = exi * c1cs2_ref;
-        // pressure, from grad(ln rho + s / c_p), and Lorentz force
+        // pressure and Lorentz force.  The two gradients are converted each with its own
+        // scale: in a direction in which only the smaller-scaled field varies, a sum in the
+        // other's units would keep only the bits left of those.
         const int ej = FX_EB + 44 + 2 * ka;
         double pl[3] = {cjb * fx_to_double(fx_det2(J[1], B[2], J[2], B[1]), ej),
                         cjb * fx_to_double(fx_det2(J[2], B[0], J[0], B[2]), ej),
@@ -1076,9 +1053,9 @@ __device__ __forceinline__ void fx_march_a(const SubstepArgs<double, double> &a,
         FxSplit SS[3];
 #pragma unroll
         for (int q = 0; q < 3; ++q) {
-            const long long big = pi_s ? GS[q] : GL[q], small = pi_s ? GL[q] : GS[q];
-            pl[q] = fma(-cp, fx_to_double(big + fx_mulfrac(small, pi_rh, pi_rl),
-                                          FX_EB64 + 2 + (pi_s ? ks : kl)), pl[q]);
+            const double g = fma(a.k.inv_cp, fx_to_double(GS[q], FX_EB64 + 2 + ks),
+                                 fx_to_double(GL[q], FX_EB64 + 2 + kl));
+            pl[q] = fma(-cp, g, pl[q]);
             SS[q] = fx_split(GS[q]);
         }
         // entropy: advection, conduction, eta j^2 / rho
