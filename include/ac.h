@@ -225,9 +225,10 @@ int ac_get_stencil_order(const ac_handle *h, int *order);
  * their exponents E; the stencil numerators and the products of the right-hand
  * side are then exact integers, rounded once when a term is converted to binary64.
  * That form runs while the components' exponents lie within six binades of each
- * other (a component keeps at least 50 bits of its own range), every |E| <= 200, a
- * mean flow is at most 2^4 times its range and |ln rho| and |xi| (the exponent of
- * c_s^2) stay below 64; otherwise b = 50, every field keeps its own scale and the
+ * other (a component keeps at least 50 bits of its own range; a uniform component of u
+ * counts with its value unless that is zero), every |E| <= 200, a mean flow is at most
+ * 2^4 times its range and |ln rho| and |xi| (the exponent of c_s^2) stay below 64;
+ * otherwise b = 50, every field keeps its own scale and the
  * sums across components and the products run in binary64; a state that holds a NaN
  * or an infinity, or a range outside [2^-960, 2^960), takes plain binary64 stencils
  * (the AC_STENCIL_FP64 arithmetic, so non-finite values propagate as the definition

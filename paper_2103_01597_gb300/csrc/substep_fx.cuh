@@ -148,12 +148,13 @@ __device__ __forceinline__ void fx_plan(unsigned long long *stats, FxPlan *plan,
     if (eg == -100000) eg = egc > -100000 ? egc : 0;
     const int any_bad = __any_sync(0xffffffffu, bad);
     const int far = __any_sync(0xffffffffu, q < NF && !zero && e < eg - FX_MODE_SLACK);
-    // what FX_GROUP is sized for: the slack, the exponents, |u| < 2^(E + 4) (u is
-    // taken from F + C), |ln rho| and |xi| below 64 (the fixed-point exp)
+    // what FX_GROUP is sized for: the slack, the exponents, |u| < 2^(E + 4) (u is taken
+    // from F + C, so that a constant component has to lie within the slack too, or be
+    // zero), |ln rho| and |xi| below 64 (the fixed-point exp)
     const double xb = gamma_cp * __shfl_sync(0xffffffffu, big, 4) +
                       fabs(gm1) * __shfl_sync(0xffffffffu, big, 0);
     int out = q < NF && ((!zero && e < eg - FX_GROUP_SLACK) || eg > FX_EMAX || eg < -FX_EMAX);
-    if (g == 1) out |= ec > eg + 4;
+    if (g == 1) out |= ec > eg + 4 || (zero && c != 0.0 && ec < eg - FX_GROUP_SLACK);
     if (q == 0) out |= !(big < 64.0) || !(xb < 64.0);
     const int any_out = __any_sync(0xffffffffu, out);
     // (FX_FIELD wants equal spacing: without it the plain stencils take its place)

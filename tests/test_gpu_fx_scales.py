@@ -1,5 +1,6 @@
 """Terms of the binary64 substep whose operands have scales far apart: the pressure
-gradient where ln rho and s vary along different axes.  One substep at 1e-12 relative per field
+gradient where ln rho and s vary along different axes, and advection by a uniform
+velocity component far below the others' range.  One substep at 1e-12 relative per field
 in the max norm against the FP64 oracle (the bound the method is held to;
 test_gpu_substep.py): here only the small operand reaches the component that is looked at.
 """
@@ -54,3 +55,30 @@ def test_pressure_of_fields_on_different_axes(eps, small, n, hs, entropy):
     err, wo = _w(n, f, hs, **terms)
     assert np.max(np.abs(wo[2])) > 1e-6 * eps * 1e-3
     assert np.all(err[1:3] <= 1e-12), err
+
+
+@pytest.mark.parametrize("uz", [0.3, 1e-2, 1e-5, 1e-6, 1e-8])
+@pytest.mark.parametrize("n,hs", [(N, (1.0, 1.0, 1.0)), ((26, 28, 25), (1.0, 1.5, 0.75))])
+def test_advection_by_a_small_uniform_component(uz, n, hs):
+    """u = (sin y, sin x, u_z): divergence-free, and only u_z meets the gradients of
+    ln rho(z) and (s being at its reference) A(z)."""
+    f = np.zeros((8,) + n[::-1])
+    x, y, z = _axes(n)
+    f[0] = 0.3 * np.sin(z + 0.1)
+    f[1], f[2], f[3] = np.sin(y), np.sin(x), uz
+    err, wo = _w(n, f, hs)
+    assert np.max(np.abs(wo[0])) > 1e-2 * uz * 1e-3
+    assert err[0] <= 1e-12, err
+
+
+@pytest.mark.parametrize("u", [(1.0, 1e-8, 0.0), (1e-9, 0.0, 2.0), (1e-3, 1e-3, 1e-3)])
+def test_advection_by_a_uniform_flow(u):
+    """Every component constant: ln rho varies along the axis of the smallest."""
+    f = np.zeros((8,) + N[::-1])
+    axes = _axes(N)
+    small = min((abs(v), a) for a, v in enumerate(u) if v)[1]
+    f[0] = 0.3 * np.sin(axes[small] + 0.1)
+    for a in range(3):
+        f[1 + a] = u[a]
+    err, _ = _w(N, f)
+    assert err[0] <= 1e-12, err
