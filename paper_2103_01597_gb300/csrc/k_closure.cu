@@ -486,10 +486,20 @@ __device__ __forceinline__ long long restrict_bits(float v) {
 // fine plane it reads three rows, a lane its two cells (the third comes from the lane
 // below), aligns them to the largest exponent in the warp (56 bits) and keeps the
 // plane's weighted sum P, so that a coarse cell is P(2K-1) + 2 P(2K) + P(2K+1) and costs
-// two new planes.  Cells whose sum comes out below 2^-26 of the scale, planes with
-// exponents out of range (zeros, non-finite values) go through restrict_cell, so every
-// result carries binary32's rounding and no more.  Measured, 256^3 binary64 to 128^3, eight
-// fields in one launch: 951 us in binary64 (27 additions a cell), 495 us so.
+// two new planes.  Where the exact sum might round to the other binary32 neighbour
+// (restrict_sure), and for planes with exponents out of range (zeros, non-finite values),
+// the cell goes through restrict_cell, so a result is the exact sum's rounding or that
+// function's.  Measured, 256^3 binary64 to 128^3, eight fields in one launch: 951 us in
+// binary64 (27 additions a cell), 502 us so.
+// Whether the integer sum s, of value d, has the exact sum's binary32 rounding.  Alignment
+// drops less than 68 units (one of each value, whose weights add up to 64, and the
+// planes' shifts); with |s| from 2^46 on these are 68 2^6 units in the last place of d at
+// most, and the rounding is sure unless d's last 29 bits lie that near a midpoint.
+__device__ __forceinline__ bool restrict_sure(long long s, double d) {
+    const int t = (int)((unsigned)__double2loint(d) & 0x1fffffffu) - 0x10000000;
+    return (s < 0 ? -s : s) >= (1ll << 46) && (t > 5000 || t < -5000);
+}
+
 struct RestrictPlane {
     long long p;
     int E;  // biased exponent of the scale; 0: not representable here, 1: all zero
@@ -564,12 +574,12 @@ __global__ void __launch_bounds__(256) restrict_kernel(R8<T> fine8, int nxf, int
         const int E = max(a.E, max(b.E, c.E));
         const long long s = (a.p >> min(E - a.E, 63)) + 2 * (b.p >> min(E - b.E, 63)) +
                             (c.p >> min(E - c.E, 63));
-        const long long m = s < 0 ? -s : s;
+        const double d = fx_to_double(s, FX_EB64 + E - 1078 - 6);
         float r;
         if (E == 1 && a.E && b.E && c.E)
             r = 0.f;
-        else if (a.E && b.E && c.E && m >= (1ll << 36))
-            r = (float)fx_to_double(s, FX_EB64 + E - 1078 - 6);
+        else if (a.E && b.E && c.E && restrict_sure(s, d))
+            r = (float)d;
         else
             r = restrict_cell(fine, nxf, nyf, nzf, Ic, Jc, K);
         if (active) coarse[((long long)K * nyc + J) * nxc + I] = r;
