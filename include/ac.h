@@ -240,7 +240,10 @@ int ac_get_stencil_order(const ac_handle *h, int *order);
  * AC_STENCIL_FP64: binary64 arithmetic throughout.  AC_STENCIL_FIXED: integer
  * sums, AC_ERR_ARG where they do not apply.  Extra device memory for integer
  * sums: one int64 copy of the eight fields with a radius-3 halo, allocated on first
- * use.  Its kernel's waits for that copy are bounded: if one runs out, ac_store,
+ * use.  Where AC_STENCIL_AUTO cannot have it (no memory left; the handle's first such
+ * substep under stream capture) it goes on with plain binary64 stencils, after a lack of
+ * memory until the next ac_set_stencil_mode; AC_STENCIL_FIXED returns the error.  Its
+ * kernel's waits for that copy are bounded: if one runs out, ac_store,
  * ac_store_f32 and ac_last_cfl return AC_ERR_TIMEOUT.
  */
 #define AC_STENCIL_AUTO 0

@@ -64,6 +64,7 @@ struct ac_handle {
     CUtensorMap fx_map;           // tensor map over them
     unsigned long long *fx_stats; // per-field extremes of the substep's input (16 words, and a count)
     void *fx_plan;                // device plan of the integer-sum path (mode, scales)
+    int fx_refused;               // AUTO: its memory could not be had, plain stencils instead
     unsigned fx_polls;            // polls of a device wait of the integer-sum substep
     double *stage;       // float64 staging for load/store
     size_t stage_elems;
@@ -587,6 +588,7 @@ extern "C" int ac_set_stencil_mode(ac_handle *h, int mode) {
     if (!h || mode < AC_STENCIL_AUTO || mode > AC_STENCIL_FIXED) return AC_ERR_ARG;
     if (mode == AC_STENCIL_FIXED && !fx_applicable(h)) return AC_ERR_ARG;
     h->stencil_mode = mode;
+    h->fx_refused = 0;  // asked for anew
     return AC_OK;
 }
 
@@ -623,7 +625,7 @@ extern "C" int ac_get_stencil_order(const ac_handle *h, int *order) {
 
 extern "C" int ac_get_stencil_path(const ac_handle *h, int *fixed) {
     if (!h || !fixed) return AC_ERR_ARG;
-    *fixed = h->stencil_mode != AC_STENCIL_FP64 && fx_applicable(h);
+    *fixed = h->stencil_mode != AC_STENCIL_FP64 && !h->fx_refused && fx_applicable(h);
     return AC_OK;
 }
 
@@ -654,6 +656,28 @@ static int ensure_fx(ac_handle *h) {
     h->fx_block = blk;
     h->fx_stats = stats;
     h->fx_plan = plan;
+    return AC_OK;
+}
+
+// Whether the handle's stream is being captured into a graph (nothing can be allocated).
+static bool capturing(const ac_handle *h) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &st) == cudaSuccess) return st != cudaStreamCaptureStatusNone;
+    (void)cudaGetLastError();  // the default stream beside a capture
+    return true;
+}
+
+// The same for AC_STENCIL_AUTO, which has the plain stencils to go on with where the work
+// areas are not there and cannot be had: no memory left for them (remembered), or a first
+// substep under capture.  *use is cleared then.
+static int ensure_fx_auto(ac_handle *h, int *use) {
+    if (h->stencil_mode == AC_STENCIL_FIXED || h->fx_block) return ensure_fx(h);
+    if (!h->fx_refused && !capturing(h)) {
+        const int rc = ensure_fx(h);
+        if (rc != AC_ERR_OOM) return rc;
+        h->fx_refused = 1;
+    }
+    *use = 0;
     return AC_OK;
 }
 
@@ -795,8 +819,10 @@ extern "C" int ac_integrate_substep(ac_handle *h, double dt, int s) {
     L.fx_copies = nullptr;
     L.fx_map = nullptr;
     if (L.use_fx) {
-        rc = ensure_fx(h);
+        rc = ensure_fx_auto(h, &L.use_fx);
         if (rc) return rc;
+    }
+    if (L.use_fx) {
         L.fx_copies = h->fx_block;
         L.fx_map = &h->fx_map;
         L.fx_stats = h->fx_stats;
