@@ -555,9 +555,9 @@ __device__ __forceinline__ RestrictPlane restrict_plane(const T *__restrict__ fi
 
 template <typename T, bool VEC>
 __global__ void __launch_bounds__(256) restrict_kernel(R8<T> fine8, int nxf, int nyf, int nzf, W8 coarse8,
-                                                       int zc) {
+                                                       int zc, int lgf) {
     const int nxc = nxf / 2, nyc = nyf / 2, nzc = nzf / 2;
-    const int q = blockIdx.z & 7, k0 = (int)(blockIdx.z >> 3) * zc;
+    const int q = blockIdx.z & ((1 << lgf) - 1), k0 = (int)(blockIdx.z >> lgf) * zc;  // 2^lgf fields
     const int gx = (nxc + 31) / 32;
     const T *__restrict__ fine = fine8.p[q];
     float *__restrict__ coarse = coarse8.p[q];
@@ -1506,19 +1506,35 @@ extern "C" int ac_restrict(const void *const fine[8], int fine_precision, int nx
         if (!fine[q] || !coarse[q]) return AC_ERR_ARG;
     // coarse planes of a march: 16, more only where the grid's z extent asks for it
     const int nzc = nz / 2, zc = nzc > 16 * 8191 ? (nzc + 8190) / 8191 : 16;
-    const dim3 block(32, 8, 1), grid((unsigned)((long long)((nx / 2 + 31) / 32) * ((ny / 2 + 7) / 8)), 1,
-                                     8 * ((nzc + zc - 1) / zc));
+    const dim3 block(32, 8, 1);
+    const unsigned tiles = (unsigned)((long long)((nx / 2 + 31) / 32) * ((ny / 2 + 7) / 8));
     // pairs of fine cells in one load where every row starts on such a boundary
-    const size_t pair = fine_precision == AC_FP64 ? 16 : 8;
+    const size_t elem = fine_precision == AC_FP64 ? 8 : 4, cells = (size_t)nx * ny * nz;
     bool vec = true;
-    for (int q = 0; q < 8; ++q) vec = vec && (uintptr_t)fine[q] % pair == 0;
-    W8 out;
-    for (int q = 0; q < 8; ++q) out.p[q] = coarse[q];
+    for (int q = 0; q < 8; ++q) vec = vec && (uintptr_t)fine[q] % (2 * elem) == 0;
+    // One launch for all fields, unless an output lies in another field's input or output:
+    // then one after the other, so that such a field finds what the ones before it left.
+    auto meet = [](const void *a, size_t na, const void *b, size_t nb) {
+        return (uintptr_t)a < (uintptr_t)b + nb && (uintptr_t)b < (uintptr_t)a + na;
+    };
+    int lgf = 3;
+    for (int q = 0; q < 8; ++q)
+        for (int p = 0; p < 8; ++p)
+            if (p != q && (meet(coarse[q], cells / 2, fine[p], cells * elem) ||
+                           meet(coarse[q], cells / 2, coarse[p], cells / 2)))
+                lgf = 0;
+    const dim3 grid(tiles, 1, (unsigned)((nzc + zc - 1) / zc) << lgf);
     auto launch = [&](auto t, auto v) {
         using T = decltype(t);
-        R8<T> in;
-        for (int q = 0; q < 8; ++q) in.p[q] = static_cast<const T *>(fine[q]);
-        restrict_kernel<T, decltype(v)::value><<<grid, block, 0, st>>>(in, nx, ny, nz, out, zc);
+        for (int q0 = 0; q0 < 8; q0 += 1 << lgf) {
+            R8<T> in;
+            W8 out;
+            for (int q = 0; q < 8; ++q) {
+                in.p[q] = static_cast<const T *>(fine[(q0 + q) & 7]);
+                out.p[q] = coarse[(q0 + q) & 7];
+            }
+            restrict_kernel<T, decltype(v)::value><<<grid, block, 0, st>>>(in, nx, ny, nz, out, zc, lgf);
+        }
     };
     if (fine_precision == AC_FP64) {
         if (vec) launch(double{}, std::true_type{}); else launch(double{}, std::false_type{});
