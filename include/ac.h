@@ -243,8 +243,10 @@ int ac_get_stencil_order(const ac_handle *h, int *order);
  * use.  Where AC_STENCIL_AUTO cannot have it (no memory left; the handle's first such
  * substep under stream capture) it goes on with plain binary64 stencils, after a lack of
  * memory until the next ac_set_stencil_mode; AC_STENCIL_FIXED returns the error.  Its
- * kernel's waits for that copy are bounded: if one runs out, ac_store,
- * ac_store_f32 and ac_last_cfl return AC_ERR_TIMEOUT.
+ * kernel's waits for that copy are bounded: if one runs out, the state is undefined and
+ * the next of ac_store, ac_store_w, ac_store_f32, ac_last_cfl, ac_reduce,
+ * ac_get_stencil_modes and (where it has happened by then) substep 0 of a step returns
+ * AC_ERR_TIMEOUT, once.
  */
 #define AC_STENCIL_AUTO 0
 #define AC_STENCIL_FP64 1

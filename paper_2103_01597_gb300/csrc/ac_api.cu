@@ -57,7 +57,7 @@ struct ac_handle {
     double *partials;
     unsigned int *flags;
     double *result_dev;  // [value, flag word]
-    double *result_host; // page-locked copy of result_dev
+    double *result_host; // page-locked copy of result_dev, and the substep's timeout word
     unsigned long long *cfl_dev;  // max CFL speed of the last substep-0 input (bits of a double)
     int stencil_mode;             // AC_STENCIL_*
     void *fx_block;               // int64 copies of the fields (integer stencil sums)
@@ -131,6 +131,8 @@ cudaError_t ac::zero_now(void *p, size_t bytes) {
     return e != cudaSuccess ? e : (s != cudaSuccess ? s : d);
 }
 
+static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
+
 static void free_timing(ac_handle *h) {
     if (!h->tev) return;
     for (int i = 0; i < 3 * AC_TIMING_MAX; ++i)
@@ -148,7 +150,6 @@ static void free_handle_memory(ac_handle *h) {
     if (h->result_dev) cudaFree(h->result_dev);
     if (h->result_host) cudaFreeHost(h->result_host);
     if (h->stage) cudaFree(h->stage);
-    if (h->cfl_dev) cudaFree(h->cfl_dev);
     if (h->fx_block) cudaFree(h->fx_block);
     if (h->fx_stats) cudaFree(h->fx_stats);
     if (h->fx_plan) cudaFree(h->fx_plan);
@@ -173,13 +174,14 @@ extern "C" int ac_init(ac_handle **out, const ac_grid *grid, const ac_params *pa
     const int ntab = grid->nx + grid->ny + grid->nz;
     cudaError_t e = cudaMalloc(&h->ftab, (size_t)ntab * (sizeof(double2) + sizeof(float2)));
     if (e == cudaSuccess) e = cudaMalloc(&h->partials, sizeof(double) * reduce_max_blocks());
-    const size_t flag_bytes = sizeof(unsigned int) * (reduce_max_blocks() + 1);
-    if (e == cudaSuccess) e = cudaMalloc(&h->flags, flag_bytes);
-    if (e == cudaSuccess) e = zero_now(h->flags, flag_bytes);
+    // the words that have to be zero at first in one block: flags, their count, cfl_dev
+    const size_t flag_bytes = align_up(sizeof(unsigned int) * (reduce_max_blocks() + 1), 8);
+    if (e == cudaSuccess) e = cudaMalloc(&h->flags, flag_bytes + sizeof(unsigned long long));
+    if (e == cudaSuccess) e = zero_now(h->flags, flag_bytes + sizeof(unsigned long long));
+    h->cfl_dev = reinterpret_cast<unsigned long long *>(reinterpret_cast<char *>(h->flags) + flag_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&h->result_dev, 2 * sizeof(double));
-    if (e == cudaSuccess) e = cudaMallocHost(&h->result_host, 2 * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&h->cfl_dev, sizeof(unsigned long long));
-    if (e == cudaSuccess) e = zero_now(h->cfl_dev, sizeof(unsigned long long));
+    if (e == cudaSuccess) e = cudaMallocHost(&h->result_host, 3 * sizeof(double));
+    if (e == cudaSuccess) h->result_host[2] = 0.0;
     if (e != cudaSuccess) {
         int rc = cuda_fail(e);
         free_handle_memory(h);
@@ -209,8 +211,6 @@ extern "C" int ac_field_elems(const ac_handle *h, size_t *elems) {
     *elems = (size_t)h->g.elems;
     return AC_OK;
 }
-
-static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // Allocate the library-owned state on first use (zero-filled).
 static int ensure_state(ac_handle *h) {
@@ -338,16 +338,18 @@ static int load_common(ac_handle *h, int field, const double *src, int to_w) {
     return AC_OK;
 }
 
-// Wait for the stream; AC_ERR_TIMEOUT if a bounded device wait of the integer-sum
-// substep ran out since the last such report (the state is then undefined).
-static int sync_checked(ac_handle *h) {
-    int *err = reinterpret_cast<int *>(h->result_host + 1);
-    *err = 0;
-    if (h->fx_plan) CK(fx_plan_err(h->fx_plan, err, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
+// AC_ERR_TIMEOUT if a bounded device wait of the integer-sum substep is known to have run
+// out since the last such report (the state is then undefined).
+static int timed_out(ac_handle *h) {
+    volatile int *err = reinterpret_cast<volatile int *>(h->result_host + 2);
     if (!*err) return AC_OK;
-    CK(fx_plan_err(h->fx_plan, nullptr, h->stream));
+    *err = 0;
     return AC_ERR_TIMEOUT;
+}
+// Wait for the stream, after which every such wait before it is known.
+static int sync_checked(ac_handle *h) {
+    CK(cudaStreamSynchronize(h->stream));
+    return timed_out(h);
 }
 
 static int store_common(ac_handle *h, int field, double *dst, int from_w) {
@@ -686,7 +688,7 @@ extern "C" int ac_get_stencil_modes(ac_handle *h, unsigned long long counts[3]) 
     counts[0] = counts[1] = counts[2] = 0;
     if (!h->fx_plan) return AC_OK;
     CK(fx_plan_taken(h->fx_plan, counts, h->stream));
-    return AC_OK;
+    return timed_out(h);
 }
 
 extern "C" int ac_diag_substep_polls(ac_handle *h, unsigned polls) {
@@ -770,6 +772,7 @@ extern "C" int ac_integrate_substep(ac_handle *h, double dt, int s) {
     if (!h || s < 0 || s > 2 || !isfinite(dt)) return AC_ERR_ARG;
     if (s != h->next_s) return AC_ERR_STATE;
     int rc = ensure_state(h);
+    if (!rc && s == 0) rc = timed_out(h);  // (what has reached the host: no wait for the device)
     if (rc) return rc;
     const int forcing = h->params.force_amp != 0.0;
     if (forcing) {
@@ -829,6 +832,7 @@ extern "C" int ac_integrate_substep(ac_handle *h, double dt, int s) {
         L.fx_plan = h->fx_plan;
     }
     L.fx_polls = h->fx_polls;
+    L.fx_err = reinterpret_cast<int *>(h->result_host + 2);
     L.ev_mid = nullptr;
     cudaEvent_t *tev = nullptr;
     if (h->timing && h->nrec < AC_TIMING_MAX) {
@@ -959,8 +963,9 @@ extern "C" int ac_reduce(ac_handle *h, int op, int quantity, double *out) {
     cudaError_t e = launch_reduce(L, h->stream, &nl);
     h->launches += nl;
     if (e != cudaSuccess) return cuda_fail(e);
-    CK(cudaStreamSynchronize(h->stream));
+    rc = sync_checked(h);
     *out = h->result_host[0];
+    if (rc) return rc;
     unsigned int flag;
     memcpy(&flag, &h->result_host[1], sizeof flag);
     return flag ? AC_ERR_NONFINITE : AC_OK;

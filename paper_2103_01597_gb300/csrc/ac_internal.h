@@ -111,7 +111,8 @@ struct SubstepLaunch {
     const CUtensorMap *fx_map;
     unsigned long long *fx_stats;
     void *fx_plan;
-    unsigned fx_polls;         // polls of a device wait before it gives up
+    unsigned fx_polls;         // polls of a device wait before it gives up ...
+    int *fx_err;               // ... and sets this word (page-locked host memory)
     double dx[3];
     // optional: recorded after the preparation kernels (integer-sum path:
     // extremes, plan, quantisation), before the substep kernel itself
@@ -121,9 +122,6 @@ constexpr unsigned FX_WAIT_LIMIT = 1u << 18;  // polls (3.8 us each): a second
 size_t fx_plan_bytes();
 size_t fx_copy_bytes(const Geom &g);
 cudaError_t fx_encode_map(void *base, const Geom &g, CUtensorMap *map);
-// Enqueues a copy of the plan's timeout word (a bounded wait of the tiled kernel ran
-// out) to page-locked *err, or, with err null, clears it.
-cudaError_t fx_plan_err(void *plan, int *err, cudaStream_t st);
 // Substeps run in each mode (group scales, per-field scales, plain binary64)
 // since the plan was zeroed; synchronises `st`.
 cudaError_t fx_plan_taken(const void *plan, unsigned long long taken[3], cudaStream_t st);

@@ -59,7 +59,7 @@ cudaError_t fx_encode_map(void *base, const Geom &g, CUtensorMap *map) {
 
 template <bool CFL, bool EXT, bool ANISO>
 static cudaError_t launch_fx_group(SubstepArgs<double, double> a, const CUtensorMap &map,
-                                   const FxCoefs &fc, FxPlan *plan, unsigned polls,
+                                   const FxCoefs &fc, const FxPlan *plan, unsigned polls, int *err,
                                    cudaStream_t st) {
     auto k = substep_fx_kernel<CFL, EXT, ANISO>;
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FX_SMEM);
@@ -67,7 +67,7 @@ static cudaError_t launch_fx_group(SubstepArgs<double, double> a, const CUtensor
     const unsigned gx = (a.g.nx + FXT - 1) / FXT, gy = (a.g.ny + FXT - 1) / FXT;
     a.zchunk = fx_zchunk((long long)gx * gy, a.g.nz);
     const dim3 grid(gx, gy, (a.g.nz + a.zchunk - 1) / a.zchunk);
-    k<<<grid, dim3(FXT, FXT, 2), FX_SMEM, st>>>(a, map, fc, plan, polls);
+    k<<<grid, dim3(FXT, FXT, 2), FX_SMEM, st>>>(a, map, fc, plan, polls, err);
     return cudaGetLastError();
 }
 
@@ -165,8 +165,8 @@ cudaError_t launch_substep_f64(const SubstepLaunch &L, cudaStream_t st, int *lau
     // one kernel per plan; those the plan did not choose return at once
 #define AC_FX(C, X)                                                                \
     do {                                                                           \
-        e = aniso ? launch_fx_group<C, X, true>(a, *L.fx_map, fc, plan, L.fx_polls, st)   \
-                  : launch_fx_group<C, X, false>(a, *L.fx_map, fc, plan, L.fx_polls, st); \
+        e = aniso ? launch_fx_group<C, X, true>(a, *L.fx_map, fc, plan, L.fx_polls, L.fx_err, st)   \
+                  : launch_fx_group<C, X, false>(a, *L.fx_map, fc, plan, L.fx_polls, L.fx_err, st); \
         if (e != cudaSuccess) return e;                                            \
         if (aniso) substep_fx_fallback_kernel<C, X, false><<<grid, block, 0, st>>>(a, fx, fc, plan); \
         else substep_fx_fallback_kernel<C, X, true><<<grid, block, 0, st>>>(a, fx, fc, plan); \
@@ -180,13 +180,6 @@ cudaError_t launch_substep_f64(const SubstepLaunch &L, cudaStream_t st, int *lau
 
 // Size of the device plan of the integer-sum path (allocated by the handle).
 size_t fx_plan_bytes() { return sizeof(FxPlan); }
-
-// Enqueue a copy of the plan's timeout word to page-locked *err, or clear it.
-cudaError_t fx_plan_err(void *plan, int *err, cudaStream_t st) {
-    FxPlan *p = static_cast<FxPlan *>(plan);
-    return err ? cudaMemcpyAsync(err, &p->err, sizeof(int), cudaMemcpyDeviceToHost, st)
-               : cudaMemsetAsync(&p->err, 0, sizeof(int), st);
-}
 
 // Substeps run in each mode of the integer-sum path, read from a plan.
 cudaError_t fx_plan_taken(const void *plan, unsigned long long taken[3], cudaStream_t st) {

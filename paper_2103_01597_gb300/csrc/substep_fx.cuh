@@ -101,7 +101,6 @@ struct FxPlan {
     int s[NF];                 // F = round((f - c) 2^s), s = b - E
     unsigned long long C[NF];  // round(c 2^s) modulo 2^64
     unsigned long long taken[3];  // substeps counted in each mode (cumulative)
-    int err;                   // set if a bounded wait of the substep kernel ran out
 };
 
 // One warp: lane q < NF plans field q (offset, exponent), then the lanes agree
@@ -1258,7 +1257,7 @@ __device__ __forceinline__ void fx_march_u(const SubstepArgs<double, double> &a,
 template <bool CFL, bool EXT, bool ANISO>
 __global__ void __launch_bounds__(2 * FXT * FXT, 1)
     substep_fx_kernel(const SubstepArgs<double, double> a, const __grid_constant__ CUtensorMap map,
-                      const FxCoefs fc, FxPlan *plan, unsigned polls) {
+                      const FxCoefs fc, const FxPlan *plan, unsigned polls, int *err) {
     if (plan->kern != FX_GROUP) return;
     extern __shared__ __align__(128) unsigned char fx_smem[];
     __shared__ FxShared sh;
@@ -1312,7 +1311,7 @@ __global__ void __launch_bounds__(2 * FXT * FXT, 1)
     // every warp out of the march no plane is asked for any more, and the last fill of
     // each slot is waited for
     if (__syncthreads_or(!m.ok) && tid == 0) {
-        atomicExch(&plan->err, 1);
+        *reinterpret_cast<volatile int *>(err) = 1;  // page-locked host memory
         for (unsigned n = sh.fetched - FX_SLOTS; n < sh.fetched; ++n)
             fx_wait(&sh.full[n % FX_SLOTS], (n / FX_SLOTS) & 1, FX_WAIT_LIMIT);
     }

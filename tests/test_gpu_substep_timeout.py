@@ -48,3 +48,32 @@ def test_substep_gives_up_and_the_next_one_is_sound(n, polls):
         sim.store()  # reported once
     sim.close()
     assert np.array_equal(_reference(n), want)
+
+
+REPORTS = {
+    "store_w": lambda sim: sim.store_w(),
+    "reduce": lambda sim: sim.reduce(ac.AC_MAX, ac.AC_UX),
+    "last_cfl": lambda sim: ac.ac_last_cfl(sim.h),
+    "modes": lambda sim: ac.ac_get_stencil_modes(sim.h),
+    "next_step": lambda sim: (torch.cuda.synchronize(), sim.step(1e-3)),
+}
+
+
+@pytest.mark.parametrize("call", sorted(REPORTS))
+def test_every_call_that_waits_reports_it_once(call):
+    """The step's last substep gives up; a program that never stores the state still learns
+    of it."""
+    sim = _sim((40, 24, 20))
+    sim.substep(1e-3, 0)
+    sim.substep(1e-3, 1)
+    ac.ac_diag_substep_polls(sim.h, 0)
+    sim.substep(1e-3, 2)
+    ac.ac_diag_substep_polls(sim.h, 1 << 18)
+    with pytest.raises(ac.AcError) as ei:
+        REPORTS[call](sim)
+    assert ei.value.code == ac.AC_ERR_TIMEOUT
+    try:
+        REPORTS[call](sim)
+    except ac.AcError as e:  # (the undefined state may hold anything)
+        assert e.code == ac.AC_ERR_NONFINITE
+    sim.close()
