@@ -214,9 +214,10 @@ int ac_get_stencil_order(const ac_handle *h, int *order);
  * spacing dx = dy = dz, stencil order 6, a step dt with |dt| in [1e-100, 1e100]:
  * those kernels fold dt into their coefficients), plain binary64 sums
  * otherwise.  (Unequal spacings no more than a factor of 8 apart, from 16384 cells
- * on, use them too, each axis's numerators scaled to the smallest spacing, while the
- * state lies in the ranges of the form b = 56 below; ac_get_stencil_path and
- * ac_get_stencil_modes do not count that form.)  With
+ * on but for thin boxes, where the plain stencils are the faster, use them too, each
+ * axis's numerators scaled to the smallest spacing, while the state lies in the ranges
+ * of the form b = 56 below; ac_get_stencil_path and ac_get_stencil_modes do not count
+ * that form.)  With
  * integer sums every field is first written, on the device before each
  * substep, as int64 fixed point about its own offset: F = round((f - c)
  * 2^(b - E)), c the midpoint of the field's range and 2^E above its half-range
@@ -228,10 +229,12 @@ int ac_get_stencil_order(const ac_handle *h, int *order);
  * other (a component keeps at least 50 bits of its own range; a uniform component of u
  * counts with its value unless that is zero), every |E| <= 200, a mean flow is at most
  * 2^4 times its range and |ln rho| and |xi| (the exponent of c_s^2) stay below 64;
- * otherwise b = 50, every field keeps its own scale and the
- * sums across components and the products run in binary64; a state that holds a NaN
- * or an infinity, or a range outside [2^-960, 2^960), takes plain binary64 stencils
- * (the AC_STENCIL_FP64 arithmetic, so non-finite values propagate as the definition
+ * otherwise b = 50, every field keeps its own scale and the sums across components
+ * and the products run in binary64.  (Thin boxes, which the tiles of that form would
+ * mostly pad, have b = 50 throughout: a common scale for components within one binade
+ * of each other, else their own, products in binary64.)  A state that holds a NaN or
+ * an infinity, or a range outside [2^-960, 2^960), takes plain binary64 stencils (the
+ * AC_STENCIL_FP64 arithmetic, so non-finite values propagate as the definition
  * does and show in ac_last_cfl).  The result stays within the 1e-12 relative bound
  * of the exact-rounding definition.  ac_get_stencil_modes counts the substeps by the
  * state they met: AC_STENCIL_MODE_GROUP, the exponents of the components of u (and
@@ -239,10 +242,11 @@ int ac_get_stencil_order(const ac_handle *h, int *order);
  * further below its group's largest; AC_STENCIL_MODE_PLAIN as above.
  * AC_STENCIL_FP64: binary64 arithmetic throughout.  AC_STENCIL_FIXED: integer
  * sums, AC_ERR_ARG where they do not apply.  Extra device memory for integer
- * sums: one int64 copy of the eight fields with a radius-3 halo, allocated on first
- * use.  Where AC_STENCIL_AUTO cannot have it (no memory left; the handle's first such
- * substep under stream capture) it goes on with plain binary64 stencils, after a lack of
- * memory until the next ac_set_stencil_mode; AC_STENCIL_FIXED returns the error.  Its
+ * sums: one int64 copy of the eight fields, but for thin boxes with a radius-3 halo,
+ * allocated on first use.  Where AC_STENCIL_AUTO cannot have it (no memory left; the
+ * handle's first such substep under stream capture) it goes on with plain binary64
+ * stencils, after a lack of memory until the next ac_set_stencil_mode;
+ * AC_STENCIL_FIXED returns the error.  The
  * kernel's waits for that copy are bounded: if one runs out, the state is undefined and
  * the next of ac_store, ac_store_w, ac_store_f32, ac_last_cfl, ac_reduce,
  * ac_get_stencil_modes and (where it has happened by then) substep 0 of a step returns

@@ -64,6 +64,7 @@ struct ac_handle {
     CUtensorMap fx_map;           // tensor map over them
     unsigned long long *fx_stats; // per-field extremes of the substep's input (16 words, and a count)
     void *fx_plan;                // device plan of the integer-sum path (mode, scales)
+    int fx_shape;                 // form of it that the box's shape asks for (fx_form), -1: not asked yet
     int fx_refused;               // AUTO: its memory could not be had, plain stencils instead
     unsigned fx_polls;            // polls of a device wait of the integer-sum substep
     double *stage;       // float64 staging for load/store
@@ -170,6 +171,7 @@ extern "C" int ac_init(ac_handle **out, const ac_grid *grid, const ac_params *pa
     h->stream = static_cast<cudaStream_t>(stream);
     h->elem_f = params->precision == AC_FP64 ? 8 : 4;
     h->elem_w = params->precision == AC_FP32 ? 4 : 8;
+    h->fx_shape = -1;
     h->fx_polls = FX_WAIT_LIMIT;
     const int ntab = grid->nx + grid->ny + grid->nz;
     cudaError_t e = cudaMalloc(&h->ftab, (size_t)ntab * (sizeof(double2) + sizeof(float2)));
@@ -560,12 +562,6 @@ extern "C" int ac_set_forcing(ac_handle *h, const int k[3], const double e[3], d
     return AC_OK;
 }
 
-// Measured, us per step with unequal spacings, integer form against plain stencils:
-// 11520 cells 115 against 84 (with two launches a substep more than now), 17472 cells 114
-// against 146, 32768 cells 114 against 147, 215040 cells 316 against 811 (the integer form's
-// preparation launches set its floor).
-constexpr long long FX_UNEQUAL_MIN_CELLS = 16384;
-
 // Integer stencil sums apply to binary64 fields on a periodic grid with equal
 // spacing on every axis (so numerators of different axes share a coefficient).
 static int fx_applicable(const ac_handle *h) {
@@ -576,14 +572,14 @@ static int fx_applicable(const ac_handle *h) {
 }
 
 // Unequal spacings: the integer form of AC_STENCIL_AUTO, whose numerators are scaled
-// axis by axis (ratios up to 8, so that the coarsest axis keeps its precision), from a
-// size on where it is the faster one.
+// axis by axis (ratios up to 8, so that the coarsest axis keeps its precision), for the
+// boxes where it is the faster one (fx_form).
 static int fx_unequal(const ac_handle *h) {
     const double dx = h->grid.lx / h->grid.nx, dy = h->grid.ly / h->grid.ny,
                  dz = h->grid.lz / h->grid.nz;
     const double lo = fmin(dx, fmin(dy, dz)), hi = fmax(dx, fmax(dy, dz));
     return h->params.precision == AC_FP64 && h->grid.layout == AC_LAYOUT_PERIODIC &&
-           h->coefs.radius == 3 && hi <= 8.0 * lo && h->g.elems >= FX_UNEQUAL_MIN_CELLS;
+           h->coefs.radius == 3 && hi <= 8.0 * lo;
 }
 
 extern "C" int ac_set_stencil_mode(ac_handle *h, int mode) {
@@ -633,14 +629,14 @@ extern "C" int ac_get_stencil_path(const ac_handle *h, int *fixed) {
 
 // Work areas of the integer-sum path, on first use: the int64 copies of the
 // fields, the extremes words and the plan (zeroed, so its mode counts start at 0).
-static int ensure_fx(ac_handle *h) {
+static int ensure_fx(ac_handle *h, int form) {
     if (h->fx_block) return AC_OK;
     void *blk = nullptr;
     unsigned long long *stats = nullptr;
     void *plan = nullptr;
-    cudaError_t e = cudaMalloc(&blk, fx_copy_bytes(h->g));
+    cudaError_t e = cudaMalloc(&blk, fx_copy_bytes(h->g, form));
     if (e == cudaSuccess) e = cudaMalloc(&stats, (2 * NF + 1) * sizeof(unsigned long long));
-    if (e == cudaSuccess) e = fx_encode_map(blk, h->g, &h->fx_map);
+    if (e == cudaSuccess && form != FX_COLUMNS) e = fx_encode_map(blk, h->g, &h->fx_map);
     if (e == cudaSuccess) e = cudaMalloc(&plan, fx_plan_bytes());
     if (e == cudaSuccess) e = cudaMemsetAsync(plan, 0, fx_plan_bytes(), h->stream);
     // extremes: largest keys start at 0, smallest at all ones, then the count of
@@ -673,13 +669,13 @@ static bool capturing(const ac_handle *h) {
 // areas are not there and cannot be had: no memory left for them (remembered), or a first
 // substep under capture.  *use is cleared then.
 static int ensure_fx_auto(ac_handle *h, int *use) {
-    if (h->stencil_mode == AC_STENCIL_FIXED || h->fx_block) return ensure_fx(h);
+    if (h->stencil_mode == AC_STENCIL_FIXED || h->fx_block) return ensure_fx(h, *use);
     if (!h->fx_refused && !capturing(h)) {
-        const int rc = ensure_fx(h);
+        const int rc = ensure_fx(h, *use);
         if (rc != AC_ERR_OOM) return rc;
         h->fx_refused = 1;
     }
-    *use = 0;
+    *use = FX_NONE;
     return AC_OK;
 }
 
@@ -811,9 +807,14 @@ extern "C" int ac_integrate_substep(ac_handle *h, double dt, int s) {
     L.dt = dt;
     L.s = s;
     // (integer sums need 32-bit neighbour offsets: fewer than 2^31 cells per array)
-    L.use_fx = 0;
-    if (h->stencil_mode != AC_STENCIL_FP64 && h->g.elems < (1ll << 31))
-        L.use_fx = fx_applicable(h) ? 1 : (fx_unequal(h) ? 2 : 0);
+    L.use_fx = FX_NONE;
+    if (h->stencil_mode != AC_STENCIL_FP64 && h->g.elems < (1ll << 31)) {
+        const int equal = fx_applicable(h);
+        if (equal || fx_unequal(h)) {
+            if (h->fx_shape < 0) h->fx_shape = fx_form(h->g, equal);
+            L.use_fx = h->fx_shape;
+        }
+    }
     L.dx[0] = h->grid.lx / h->grid.nx;
     L.dx[1] = h->grid.ly / h->grid.ny;
     L.dx[2] = h->grid.lz / h->grid.nz;

@@ -102,12 +102,12 @@ struct SubstepLaunch {
     double alpha, beta, dt;
     int s;
     unsigned long long *cfl_max;  // substep 0: device word for the max CFL speed (or NULL)
-    // binary64 with integer stencil sums (periodic grids): use_fx = 1 for equal spacing,
-    // 2 for unequal; int64 copies of the fields, padded by their periodic halo, with their
-    // tensor map, 17 words of per-field extremes and the device plan of the substep
-    // (fx_plan_bytes()); use_fx = 0 selects plain binary64 sums.
+    // binary64 with integer stencil sums (periodic grids): use_fx = one of the forms below,
+    // FX_NONE for plain binary64 sums; int64 copies of the fields, but for FX_COLUMNS padded
+    // by their periodic halo and with a tensor map, 17 words of per-field extremes and the
+    // device plan of the substep (fx_plan_bytes()).
     int use_fx;
-    void *fx_copies;           // fx_copy_bytes()
+    void *fx_copies;           // fx_copy_bytes(), of use_fx
     const CUtensorMap *fx_map;
     unsigned long long *fx_stats;
     void *fx_plan;
@@ -118,9 +118,13 @@ struct SubstepLaunch {
     // extremes, plan, quantisation), before the substep kernel itself
     cudaEvent_t ev_mid;
 };
+// Forms of the integer-sum path: 16 x 16 tiles with equal or unequal spacing, columns with
+// equal spacing; fx_form chooses by the box's shape.
+enum { FX_NONE = 0, FX_EQUAL = 1, FX_UNEQUAL = 2, FX_COLUMNS = 3 };
+int fx_form(const Geom &g, bool equal);
 constexpr unsigned FX_WAIT_LIMIT = 1u << 18;  // polls (3.8 us each): a second
 size_t fx_plan_bytes();
-size_t fx_copy_bytes(const Geom &g);
+size_t fx_copy_bytes(const Geom &g, int form);
 cudaError_t fx_encode_map(void *base, const Geom &g, CUtensorMap *map);
 // Substeps run in each mode (group scales, per-field scales, plain binary64)
 // since the plan was zeroed; synchronises `st`.

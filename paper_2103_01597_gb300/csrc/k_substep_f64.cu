@@ -1,6 +1,7 @@
 // FP64 substep: exact integer stencil sums on cubic periodic grids (the fast
 // path), plain binary64 stencil arithmetic otherwise.
 #include <cmath>
+#include <type_traits>
 
 #include <cudaTypedefs.h>
 
@@ -31,12 +32,59 @@ static int fx_zchunk(long long tiles, int nz) {
     return best;
 }
 
-// Padded row length (even: the strides of the tensor map are multiples of 16 bytes),
-// bytes of the eight padded int64 arrays, and the tensor map over them: dims (px,
-// py, pz, field), box one plane of a tile with its halo, all fields.
+// Launch shape of the kernels that go column by column: threads of (32, 4) cells, enough
+// z-slices for several waves of CTAs, up to 16 cells per thread.
+static int fx_column_zchunk(const Geom &g) {
+    const long long xy = (long long)((g.nx + 31) / 32) * ((g.ny + 3) / 4);
+    const long long z = xy * g.nz / (8 * 152);
+    return (int)(z < 1 ? 1 : (z > 16 ? 16 : z));
+}
+
+// Which form the box's shape asks for.  Tiles of 16 x 16 cells and copies padded by three
+// cells on each side suit boxes with extent in every direction; a thin box pads them away.
+// The times of either, in us, from what one plane takes (GB300, 54 boxes from one cell to
+// 2048^2 x 8, equal spacing and ratios of 1.25, within a fifth or so): a CTA of the tiles
+// takes 8.6 a plane (unequal 10.8) and one more to start; a pair of column CTAs on an SM
+// 8.5 to 16.4 a plane by its rows and 4.6 to start (plain stencils 16.5 to 41 and 7.5);
+// the copies 23 us a million cells, the columns' 17.
+int fx_form(const Geom &g, bool equal) {
+    const long long tiles = (long long)((g.nx + FXT - 1) / FXT) * ((g.ny + FXT - 1) / FXT);
+    const int zc = fx_zchunk(tiles, g.nz), rows = g.ny < 4 ? g.ny : 4;
+    const double waves = (double)((tiles * ((g.nz + zc - 1) / zc) + 151) / 152);
+    const double mcells = 1e-6 * g.elems;
+    const double mpadded = 1e-6 * (g.nx + 2 * R) * (double)(g.ny + 2 * R) * (g.nz + 2 * R);
+    const double tile = 4.0 + 23.0 * mpadded + waves * (zc + 1) * (equal ? 8.6 : 10.8);
+    static const double group[4] = {8.5, 13.2, 15.0, 16.4}, plain[4] = {16.5, 22.0, 32.0, 41.0};
+    const int cz = fx_column_zchunk(g);
+    const long long blocks = (long long)((g.nx + 31) / 32) * ((g.ny + 3) / 4) * ((g.nz + cz - 1) / cz);
+    const double pairs = blocks < 304 ? 1.0 : blocks / 304.0;
+    if (equal)
+        return tile <= 6.0 + 17.0 * mcells + pairs * (4.6 + cz * group[rows - 1]) ? FX_EQUAL : FX_COLUMNS;
+    // Unequal spacing: below 16384 cells, or with no more than one CTA of plain stencils to an
+    // SM, preparation is what counts (24^3 93 us a step plain, some 118 with tiles, 60x20x14
+    // 94 against 125); from there on the model decides, small boxes with a full row of a tile
+    // aside (26^3 118 against 158, 17x31x33 119 against 158, but 16x1x1100 332 against 293).
+    if (g.elems < 16384 || blocks <= 152) return FX_NONE;
+    return (g.elems < 32768 && g.nx >= FXT) || 17.0 + tile <= pairs * (7.5 + cz * plain[rows - 1])
+               ? FX_UNEQUAL
+               : FX_NONE;
+}
+
+// Padded row length (even: the strides of the tensor map are multiples of 16 bytes), the
+// geometry of the int64 copies, their bytes, and the tensor map over the padded ones: dims
+// (px, py, pz, field), box one plane of a tile with its halo, all fields.
 static int fx_px(const Geom &g) { return (g.nx + 2 * R + 1) & ~1; }
-size_t fx_copy_bytes(const Geom &g) {
-    return (size_t)NF * fx_px(g) * (g.ny + 2 * R) * (g.nz + 2 * R) * sizeof(long long);
+static Geom fx_geom(const Geom &g, int form) {
+    Geom c = g;
+    if (form == FX_COLUMNS) return c;
+    c.px = fx_px(g);
+    c.pxy = (long long)c.px * (g.ny + 2 * R);
+    c.origin = R * c.pxy + (long long)R * c.px + R;
+    c.elems = c.pxy * (g.nz + 2 * R);
+    return c;
+}
+size_t fx_copy_bytes(const Geom &g, int form) {
+    return (size_t)NF * fx_geom(g, form).elems * sizeof(long long);
 }
 cudaError_t fx_encode_map(void *base, const Geom &g, CUtensorMap *map) {
     void *fn = nullptr;
@@ -88,12 +136,10 @@ cudaError_t launch_substep_f64(const SubstepLaunch &L, cudaStream_t st, int *lau
         a.w[q] = static_cast<double *>(L.w[q]);
         fx.f[q] = a.fin[q];
     }
-    fx.px = fx_px(L.g);
-    fx.py = L.g.ny + 2 * R;
-    fx.pz = L.g.nz + 2 * R;
-    fx.pxy = (long long)fx.px * fx.py;
-    for (int q = 0; q < NF; ++q)
-        fx.F[q] = static_cast<long long *>(L.fx_copies) + q * fx.pxy * fx.pz;
+    fx.halo = L.use_fx == FX_COLUMNS ? 0 : R;
+    fx.py = L.g.ny + 2 * fx.halo;
+    fx.g = fx_geom(L.g, L.use_fx);
+    for (int q = 0; q < NF; ++q) fx.F[q] = static_cast<long long *>(L.fx_copies) + q * fx.g.elems;
     a.k = to_dev<double>(L.c, L.ph);
     a.alpha = L.alpha;
     a.beta = L.beta;
@@ -105,7 +151,7 @@ cudaError_t launch_substep_f64(const SubstepLaunch &L, cudaStream_t st, int *lau
     a.cfl_max = L.cfl_max;
     // the step folded into the RHS coefficients; with unequal spacing they hold the
     // smallest one and the numerators carry the ratios
-    const bool aniso = L.use_fx == 2;
+    const bool aniso = L.use_fx == FX_UNEQUAL;
     const double h = fmin(L.dx[0], fmin(L.dx[1], L.dx[2]));
     FxCoefs fc = {};
     if (aniso) {
@@ -146,34 +192,41 @@ cudaError_t launch_substep_f64(const SubstepLaunch &L, cudaStream_t st, int *lau
     FxPlan *plan = static_cast<FxPlan *>(L.fx_plan);
     cudaError_t e;
     fx_stats_kernel<<<fx_grid(n / 2), 256, 0, st>>>(fx, n, L.fx_stats, plan, L.ph.gamma_cp, L.ph.gm1,
-                                                   aniso);
-    fx_quantize_kernel<<<fx_grid(32ll * fx.py * fx.pz), 256, 0, st>>>(fx, L.g, plan);
+                                                   L.use_fx);
+    if (fx.g.elems > 256ll * 152 * 8)
+        fx_quantize_kernel<2><<<fx_grid((fx.g.elems + 1) / 2), 256, 0, st>>>(fx, L.g, plan);
+    else
+        fx_quantize_kernel<1><<<fx_grid(fx.g.elems), 256, 0, st>>>(fx, L.g, plan);
     if (L.ev_mid) {
         e = cudaEventRecord(L.ev_mid, st);
         if (e != cudaSuccess) return e;
     }
 
     const dim3 block(32, 4, 1);
-    const unsigned gx = (L.g.nx + block.x - 1) / block.x;
-    const unsigned gy = (L.g.ny + block.y - 1) / block.y;
-    const long long xy_blocks = (long long)gx * gy;
-    int zchunk = (int)((xy_blocks * L.g.nz) / (8 * 152));
-    zchunk = zchunk < 1 ? 1 : (zchunk > 16 ? 16 : zchunk);
-    a.zchunk = zchunk;
-    const dim3 grid(gx, gy, (L.g.nz + zchunk - 1) / zchunk);
+    a.zchunk = fx_column_zchunk(L.g);
+    const dim3 grid((L.g.nx + 31) / 32, (L.g.ny + 3) / 4, (L.g.nz + a.zchunk - 1) / a.zchunk);
     const bool ext = L.ph.ext(), cfl = a.cfl_max != nullptr;
     // one kernel per plan; those the plan did not choose return at once
-#define AC_FX(C, X)                                                                \
-    do {                                                                           \
-        e = aniso ? launch_fx_group<C, X, true>(a, *L.fx_map, fc, plan, L.fx_polls, L.fx_err, st)   \
-                  : launch_fx_group<C, X, false>(a, *L.fx_map, fc, plan, L.fx_polls, L.fx_err, st); \
-        if (e != cudaSuccess) return e;                                            \
-        if (aniso) substep_fx_fallback_kernel<C, X, false><<<grid, block, 0, st>>>(a, fx, fc, plan); \
-        else substep_fx_fallback_kernel<C, X, true><<<grid, block, 0, st>>>(a, fx, fc, plan); \
-    } while (0)
-    if (ext) { if (cfl) AC_FX(true, true); else AC_FX(false, true); }
-    else { if (cfl) AC_FX(true, false); else AC_FX(false, false); }
-#undef AC_FX
+    auto launch = [&](auto c, auto x) -> cudaError_t {
+        constexpr bool C = decltype(c)::value, X = decltype(x)::value;
+        if (L.use_fx == FX_COLUMNS) {
+            substep_fx_column_kernel<C, X><<<grid, block, 0, st>>>(a, fx, fc, plan);
+            substep_fx_fallback_kernel<C, X, FX_COLUMNS><<<grid, block, 0, st>>>(a, fx, fc, plan);
+            return cudaSuccess;
+        }
+        const cudaError_t r =
+            aniso ? launch_fx_group<C, X, true>(a, *L.fx_map, fc, plan, L.fx_polls, L.fx_err, st)
+                  : launch_fx_group<C, X, false>(a, *L.fx_map, fc, plan, L.fx_polls, L.fx_err, st);
+        if (r != cudaSuccess) return r;
+        if (aniso) substep_fx_fallback_kernel<C, X, FX_UNEQUAL><<<grid, block, 0, st>>>(a, fx, fc, plan);
+        else substep_fx_fallback_kernel<C, X, FX_EQUAL><<<grid, block, 0, st>>>(a, fx, fc, plan);
+        return cudaSuccess;
+    };
+    using yes = std::true_type;
+    using no = std::false_type;
+    e = ext ? (cfl ? launch(yes(), yes()) : launch(no(), yes()))
+            : (cfl ? launch(yes(), no()) : launch(no(), no()));
+    if (e != cudaSuccess) return e;
     *launches += 4;
     return cudaGetLastError();
 }

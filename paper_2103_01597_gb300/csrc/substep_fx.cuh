@@ -34,6 +34,8 @@
 
 #include <cuda.h>
 
+#include <type_traits>
+
 #include "fx_arith.cuh"
 #include "substep.cuh"
 
@@ -85,12 +87,14 @@ __device__ __forceinline__ unsigned long long fx_round_grid(unsigned long long b
 
 // The int64 copies: eight arrays back to back, each padded by the radius-3 periodic
 // halo (which the quantisation writes), so that the tensor memory accelerator can
-// fetch any tile with its halo as one box.
+// fetch any tile with its halo as one box; without the halo (halo = 0) for the boxes
+// that go column by column.
 struct FxPtrs {
     const double *f[NF];
     long long *F[NF];
-    int px, py, pz;     // padded extents: n + 6, px made even (16-byte strides)
-    long long pxy;      // px py
+    int halo;
+    int py;  // rows of a plane
+    Geom g;  // of the copies: with the halo px = nx + 6 made even (16-byte strides)
 };
 
 // The quantisation plan of one substep (device memory, written by
@@ -107,7 +111,7 @@ struct FxPlan {
 // on the kernel.  Thread 0 also counts the substep under its mode: plain,
 // per-field (a component more than one binade below its group's largest) or group.
 __device__ __forceinline__ void fx_plan(unsigned long long *stats, FxPlan *plan, double gamma_cp,
-                                        double gm1, int aniso) {
+                                        double gm1, int form) {
     const int q = threadIdx.x;
     int bad = 0, zero = 1, e = -100000, ec = -100000;
     double c = 0.0, big = 0.0;
@@ -156,11 +160,14 @@ __device__ __forceinline__ void fx_plan(unsigned long long *stats, FxPlan *plan,
     if (g == 1) out |= ec > eg + 4 || (zero && c != 0.0 && ec < eg - FX_GROUP_SLACK);
     if (q == 0) out |= !(big < 64.0) || !(xb < 64.0);
     const int any_out = __any_sync(0xffffffffu, out);
-    // (FX_FIELD wants equal spacing: without it the plain stencils take its place)
-    const int kern = any_bad || (aniso && any_out) ? FX_PLAIN : (any_out ? FX_FIELD : FX_GROUP);
+    // (FX_FIELD wants equal spacing: without it the plain stencils take its place; the
+    // columns' FX_GROUP has binary64 products and only asks for the narrower slack)
     const int mode = any_bad ? FX_PLAIN : (far ? FX_FIELD : FX_GROUP);
+    const int kern = form == FX_COLUMNS ? mode
+                     : any_bad || (form == FX_UNEQUAL && any_out) ? FX_PLAIN
+                     : any_out ? FX_FIELD : FX_GROUP;
     int s = FX_FIELD_BITS - (e > -100000 ? e : 0);
-    if (kern == FX_GROUP) s = FX_BITS - eg;
+    if (kern == FX_GROUP) s = form == FX_COLUMNS ? FX_FIELD_BITS - eg : FX_BITS - eg;
     if (q < NF) {
         plan->zero[q] = zero;
         plan->s[q] = s;
@@ -168,7 +175,7 @@ __device__ __forceinline__ void fx_plan(unsigned long long *stats, FxPlan *plan,
     }
     if (q == 0) {
         plan->kern = kern;
-        if (!aniso) plan->taken[mode] += 1ull;
+        if (form != FX_UNEQUAL) plan->taken[mode] += 1ull;
     }
 }
 
@@ -180,7 +187,7 @@ __device__ __forceinline__ void fx_plan(unsigned long long *stats, FxPlan *plan,
 // 32^3 substep's 42.
 __global__ void __launch_bounds__(256) fx_stats_kernel(FxPtrs p, long long n, unsigned long long *stats,
                                                        FxPlan *plan, double gamma_cp, double gm1,
-                                                       int aniso) {
+                                                       int form) {
     unsigned long long hi[NF], lo[NF];
 #pragma unroll
     for (int q = 0; q < NF; ++q) {
@@ -241,13 +248,18 @@ __global__ void __launch_bounds__(256) fx_stats_kernel(FxPtrs p, long long n, un
     __syncthreads();
     if (!last || threadIdx.x >= 32) return;
     __threadfence();
-    fx_plan(stats, plan, gamma_cp, gm1, aniso);
+    fx_plan(stats, plan, gamma_cp, gm1, form);
     if (threadIdx.x == 0) stats[2 * NF] = 0ull;
 }
 
 // F = round(f 2^s) - round(c 2^s) by integer operations on the binary64 bits, with
-// the periodic halo; nothing to do in FX_PLAIN.  A warp takes one padded row at a
-// time, two cells per lane, all sixteen loads ahead of the stores.
+// the periodic halo if the copies have one; nothing to do in FX_PLAIN.  The copies are
+// written in order, PER cells a thread (256 apart, so that a warp's stores and loads are
+// contiguous; two where that still fills the chip), all loads ahead of the stores; the
+// place in the box of a CTA's first cell is divided out once.  (A warp to each padded row
+// instead left long rows to few warps, 2.7 ms for 65536 x 1 x 1, and narrow rows to few
+// lanes.)
+template <int PER>
 __global__ void __launch_bounds__(256) fx_quantize_kernel(FxPtrs p, Geom g, const FxPlan *plan) {
     if (plan->kern == FX_PLAIN) return;
     int s[NF], zero[NF];
@@ -263,39 +275,33 @@ __global__ void __launch_bounds__(256) fx_quantize_kernel(FxPtrs p, Geom g, cons
                        : (long long)(fx_round_grid((unsigned long long)__double_as_longlong(v), s[q]) -
                                      C[q]);
     };
-    const int lane = threadIdx.x & 31;
-    const long long rows = (long long)p.py * p.pz;
-    const bool small = g.nx < R;  // the halo wraps around more than once
-    for (long long r = blockIdx.x * 8ll + (threadIdx.x >> 5); r < rows; r += gridDim.x * 8ll) {
-        const int k = (int)(r / p.py), j = (int)(r - (long long)k * p.py);
-        const long long src = wrap_near(k - R, g.nz) * g.pxy + (long long)wrap_near(j - R, g.ny) * g.px;
-        const long long dst = r * p.px + R;
-        // a cell and its images in the row's halo
-        auto put = [&](int q, int x, long long v) {
-            long long *row = p.F[q] + dst;
-            row[x] = v;
-            if (small) {
-                for (int h = x - g.nx; h >= -R; h -= g.nx) row[h] = v;
-                for (int h = x + g.nx; h < g.nx + R; h += g.nx) row[h] = v;
-            } else {
-                if (x < R) row[x + g.nx] = v;
-                if (x >= g.nx - R) row[x - g.nx] = v;
-            }
-        };
-        for (int x = lane; x < g.nx; x += 64) {
-            const int x1 = x + 32 < g.nx ? x + 32 : x;
-            double v[NF], w[NF];
+    const unsigned px = p.g.px, py = p.py;
+    for (long long t0 = blockIdx.x * (256ll * PER); t0 < p.g.elems; t0 += gridDim.x * (256ll * PER)) {
+        const unsigned row0 = (unsigned)(t0 >> 32 ? t0 / px : (unsigned)t0 / px);
+        const unsigned x0 = (unsigned)t0 - row0 * px;
+        const unsigned k0 = row0 / py, j0 = row0 - k0 * py;
+        long long src[PER];
+        double v[PER][NF];
 #pragma unroll
-            for (int q = 0; q < NF; ++q) {
-                v[q] = __ldg(p.f[q] + src + x);
-                w[q] = __ldg(p.f[q] + src + x1);
-            }
-#pragma unroll
-            for (int q = 0; q < NF; ++q) {
-                put(q, x, fix(v[q], q));
-                if (x1 != x) put(q, x1, fix(w[q], q));
-            }
+        for (int u = 0; u < PER; ++u) {
+            // the cell of the state that this cell of the copies holds
+            const bool in = t0 + threadIdx.x + 256 * u < p.g.elems;
+            const unsigned x = x0 + (in ? threadIdx.x + 256 * u : 0u), rows = x / px;
+            const unsigned j = j0 + rows, planes = j / py;
+            src[u] = wrap_near((int)(k0 + planes) - p.halo, g.nz) * g.pxy +
+                     (long long)wrap_near((int)(j - planes * py) - p.halo, g.ny) * g.px +
+                     wrap_near((int)(x - rows * px) - p.halo, g.nx);
         }
+#pragma unroll
+        for (int q = 0; q < NF; ++q)
+#pragma unroll
+            for (int u = 0; u < PER; ++u) v[u][q] = __ldg(p.f[q] + src[u]);
+#pragma unroll
+        for (int q = 0; q < NF; ++q)
+#pragma unroll
+            for (int u = 0; u < PER; ++u)
+                if (t0 + threadIdx.x + 256 * u < p.g.elems)
+                    p.F[q][t0 + threadIdx.x + 256 * u] = fix(v[u][q], q);
     }
 }
 
@@ -451,38 +457,32 @@ __device__ __forceinline__ void cell_physics_fx(const double (&u)[3], const doub
     }
 }
 
-// One field around the cell at padded index c.
-struct FxFieldView {
-    const long long *f;
-    const long long &c;
-    long long pxy;
-    int px;
-    AC_BC_ONLY(long long bc_lim;)
-    __device__ __forceinline__ long long operator()(int dx, int dy, int dz) const {
-        return __ldg(f + AC_BC(c + dz * pxy + (long long)dy * px + dx, bc_lim, AC_BC_STENCIL));
-    }
-};
-
-// One (x, y) column of the substep with per-field scales (FX_FIELD): sums across
-// the components of u or A are formed in binary64 from per-field integer numerators.
-template <bool CFL, bool EXT>
-__device__ __forceinline__ void fx_field_column(const SubstepArgs<double, double> &a, const FxPtrs &fx,
+// One (x, y) column of the substep with integer stencils and binary64 products.  PF:
+// per-field scales (FX_FIELD), so sums across the components of u or A are formed in
+// binary64 from per-field integer numerators; otherwise one scale per group (the columns'
+// FX_GROUP).
+// IX addresses the int64 copies, with the halo or without.
+template <bool PF, class IX, bool CFL, bool EXT>
+__device__ __forceinline__ void fx_column(const SubstepArgs<double, double> &a, const FxPtrs &fx,
                                           const FxCoefs &fc, const FxPlan *plan,
                                           const double *etab, int i, int j, double &cfl) {
-    // Each field's scale 2^(E - FX_BITS) is applied to its converted numerators
+    // Each field's scale 2^-s is applied to its converted numerators
     // by an exponent add on the integer pipe (fx_scaled), so only the grid
     // coefficients -- kernel parameters, read from the constant bank -- multiply
     // on the FP64 pipe, and no scaled coefficient occupies registers (the
-    // kernels sit at 255 registers).
+    // kernels sit at 255 registers).  In FX_GROUP the components of u and of A
+    // share their exponent.
     int kh[NF];
 #pragma unroll
     for (int q = 0; q < NF; ++q) kh[q] = -plan->s[q] * (1 << 20);
-    // first derivative of field q from its numerator, without the factor c1
-    // (cell_physics_fx applies it)
+    // first derivative of field q from its numerator; the gradients of ln rho, s
+    // and u stay without the factor c1 (cell_physics_fx applies it)
+    auto d1 = [&](long long N, int q) -> double { return fx_scaled(N, kh[q]) * fc.c1dt; };
     auto d1r = [&](long long N, int q) -> double { return fx_scaled(N, kh[q]); };
     const int k0 = blockIdx.z * a.zchunk;
     const int k1 = min(k0 + a.zchunk, a.g.nz);
-    const long long col = ((long long)(j + R)) * fx.px + i + R;
+    IX ix;
+    ix.set_xy(i, j, fx.g);
     double2 exy = make_double2(0.0, 0.0);
     if (a.force_on) {
         const double2 ex = a.ftab[i], ey = a.ftab[a.g.nx + j];
@@ -490,8 +490,11 @@ __device__ __forceinline__ void fx_field_column(const SubstepArgs<double, double
         exy.y = ex.x * ey.y + ex.y * ey.x;
     }
     for (int kk = k0; kk < k1; ++kk) {
-        const long long c = (kk + R) * fx.pxy + col;
-        const long long o = kk * a.g.pxy + (long long)j * a.g.px + i;
+        ix.set_z(kk, fx.g);
+        // (copies without a halo are addressed like the state)
+        const long long o = std::is_same<IX, IdxPeriodic32>::value
+                                ? ix(0, 0, 0)
+                                : kk * a.g.pxy + (long long)j * a.g.px + i;
         // Centre values (the binary64 state) and the thermodynamic factors: at the
         // top of the cell in the CFL variant (substep 0), after the stencil sums in
         // the other; each placement measured fastest for its variant at 256^3
@@ -512,12 +515,10 @@ __device__ __forceinline__ void fx_field_column(const SubstepArgs<double, double
             frc[1] = fc.amp_dt[1] * cph;
             frc[2] = fc.amp_dt[2] * cph;
         }
-        auto view = [&](int q) {
-            return FxFieldView{fx.F[q], c, fx.pxy, fx.px AC_BC_ONLY(, fx.pxy * fx.pz)};
-        };
-        const FxFieldView Fl = view(0), Fs = view(4);
-        const FxFieldView Fu[3] = {view(1), view(2), view(3)};
-        const FxFieldView Fa[3] = {view(5), view(6), view(7)};
+        using View = GlobalView<long long, IX>;
+        const View Fl{fx.F[0], ix}, Fs{fx.F[4], ix};
+        const View Fu[3] = {{fx.F[1], ix}, {fx.F[2], ix}, {fx.F[3], ix}};
+        const View Fa[3] = {{fx.F[5], ix}, {fx.F[6], ix}, {fx.F[7], ix}};
         // first derivatives
         double gl[3], gs[3], gu[3][3], B[3];
         gl[0] = d1r(nd1<0>(Fl), 0);
@@ -528,19 +529,26 @@ __device__ __forceinline__ void fx_field_column(const SubstepArgs<double, double
         gs[2] = d1r(nd1<2>(Fs), 4);
 #pragma unroll
         for (int m = 0; m < 3; ++m) {
-            gu[m][0] = d1r(nd1<0>(Fu[m]), 1 + m);
-            gu[m][1] = d1r(nd1<1>(Fu[m]), 1 + m);
-            gu[m][2] = d1r(nd1<2>(Fu[m]), 1 + m);
+            const int qu = PF ? 1 + m : 1;  // one live exponent in FX_GROUP
+            gu[m][0] = d1r(nd1<0>(Fu[m]), qu);
+            gu[m][1] = d1r(nd1<1>(Fu[m]), qu);
+            gu[m][2] = d1r(nd1<2>(Fu[m]), qu);
         }
-        B[0] = (fx_scaled(nd1<1>(Fa[2]), kh[7]) - fx_scaled(nd1<2>(Fa[1]), kh[6])) * fc.c1dt;
-        B[1] = (fx_scaled(nd1<2>(Fa[0]), kh[5]) - fx_scaled(nd1<0>(Fa[2]), kh[7])) * fc.c1dt;
-        B[2] = (fx_scaled(nd1<0>(Fa[1]), kh[6]) - fx_scaled(nd1<1>(Fa[0]), kh[5])) * fc.c1dt;
+        if constexpr (PF) {
+            B[0] = (fx_scaled(nd1<1>(Fa[2]), kh[7]) - fx_scaled(nd1<2>(Fa[1]), kh[6])) * fc.c1dt;
+            B[1] = (fx_scaled(nd1<2>(Fa[0]), kh[5]) - fx_scaled(nd1<0>(Fa[2]), kh[7])) * fc.c1dt;
+            B[2] = (fx_scaled(nd1<0>(Fa[1]), kh[6]) - fx_scaled(nd1<1>(Fa[0]), kh[5])) * fc.c1dt;
+        } else {
+            B[0] = d1(nd1<1>(Fa[2]) - nd1<2>(Fa[1]), 5);
+            B[1] = d1(nd1<2>(Fa[0]) - nd1<0>(Fa[2]), 5);
+            B[2] = d1(nd1<0>(Fa[1]) - nd1<1>(Fa[0]), 5);
+        }
         // lap V_i = sum_a N2_aa(V_i) / (180 dx^2);
         // grad(div V)_i = [4 N2_ii(V_i) + NX_ij(V_j) + NX_ik(V_k)] / (720 dx^2);
         // component C of V contributes 4 N2_CC to entry C and its two mixed
         // numerators to the other two entries.
         double viscl[3], lapa[3], J[3];
-        {
+        if constexpr (PF) {
             // per-field scaled numerators, summed across components in binary64
             double LU[3], GU[3], LA[3], GA[3];
 #pragma unroll
@@ -591,6 +599,64 @@ __device__ __forceinline__ void fx_field_column(const SubstepArgs<double, double
                 lapa[m] = LA[m] * fc.inv180dx2;
                 J[m] = fma(GA[m], fc.inv720dx2, -lapa[m]);
             }
+        } else {
+            long long LU[3], GU[3];
+            {
+                const long long c0 = Fu[0](0, 0, 0);
+                const long long xx = nd2<0>(Fu[0], c0), yy = nd2<1>(Fu[0], c0), zz = nd2<2>(Fu[0], c0);
+                LU[0] = xx + yy + zz;
+                GU[0] = 4 * xx;
+                GU[1] = ndab<0, 1>(Fu[0]);
+                GU[2] = ndab<0, 2>(Fu[0]);
+            }
+            {
+                const long long c0 = Fu[1](0, 0, 0);
+                const long long xx = nd2<0>(Fu[1], c0), yy = nd2<1>(Fu[1], c0), zz = nd2<2>(Fu[1], c0);
+                LU[1] = xx + yy + zz;
+                GU[1] += 4 * yy;
+                GU[0] += ndab<0, 1>(Fu[1]);
+                GU[2] += ndab<1, 2>(Fu[1]);
+            }
+            {
+                const long long c0 = Fu[2](0, 0, 0);
+                const long long xx = nd2<0>(Fu[2], c0), yy = nd2<1>(Fu[2], c0), zz = nd2<2>(Fu[2], c0);
+                LU[2] = xx + yy + zz;
+                GU[2] += 4 * zz;
+                GU[0] += ndab<0, 2>(Fu[2]);
+                GU[1] += ndab<1, 2>(Fu[2]);
+            }
+            // the same two sums for A; j = grad(div A) - lap A
+            long long LA[3], GA[3];
+            {
+                const long long c0 = Fa[0](0, 0, 0);
+                const long long xx = nd2<0>(Fa[0], c0), yy = nd2<1>(Fa[0], c0), zz = nd2<2>(Fa[0], c0);
+                LA[0] = xx + yy + zz;
+                GA[0] = 4 * xx;
+                GA[1] = ndab<0, 1>(Fa[0]);
+                GA[2] = ndab<0, 2>(Fa[0]);
+            }
+            {
+                const long long c0 = Fa[1](0, 0, 0);
+                const long long xx = nd2<0>(Fa[1], c0), yy = nd2<1>(Fa[1], c0), zz = nd2<2>(Fa[1], c0);
+                LA[1] = xx + yy + zz;
+                GA[1] += 4 * yy;
+                GA[0] += ndab<0, 1>(Fa[1]);
+                GA[2] += ndab<1, 2>(Fa[1]);
+            }
+            {
+                const long long c0 = Fa[2](0, 0, 0);
+                const long long xx = nd2<0>(Fa[2], c0), yy = nd2<1>(Fa[2], c0), zz = nd2<2>(Fa[2], c0);
+                LA[2] = xx + yy + zz;
+                GA[2] += 4 * zz;
+                GA[0] += ndab<0, 2>(Fa[2]);
+                GA[1] += ndab<1, 2>(Fa[2]);
+            }
+#pragma unroll
+            for (int m = 0; m < 3; ++m) {
+                viscl[m] = fma(fx_scaled(LU[m], kh[1]), fc.nu180, fx_scaled(GU[m], kh[1]) * fc.nu2160);
+                lapa[m] = fx_scaled(LA[m], kh[5]) * fc.inv180dx2;
+                J[m] = fma(fx_scaled(GA[m], kh[5]), fc.inv720dx2, -lapa[m]);
+            }
         }
         // EXT: lap xi = gamma / c_p lap s + (gamma - 1) lap ln rho (conduction)
         double lapxi = 0.0;
@@ -626,6 +692,10 @@ __device__ __forceinline__ void fx_field_column(const SubstepArgs<double, double
         }
     }
 }
+
+// How a form's int64 copies are addressed.
+template <int FORM> struct FxIndex { using type = IdxPadded; };
+template <> struct FxIndex<FX_COLUMNS> { using type = IdxPeriodic32; };
 
 // ---- FX_GROUP: integer stencils, integer products --------------------------------
 //
@@ -1318,19 +1388,20 @@ __global__ void __launch_bounds__(2 * FXT * FXT, 1)
     if (CFL) block_max_to_global(cfl, a.cfl_max);
 }
 
-// What FX_GROUP does not take: FX_FIELD (equal spacing only: FIELD), and FX_PLAIN, plain
+// What substep_fx_kernel does not take: FX_FIELD (FORM FX_EQUAL) and FX_PLAIN, plain
 // binary64 stencils, the arithmetic of AC_STENCIL_FP64.  Launched every substep beside
 // substep_fx_kernel (its own register allocation: with the group body in one kernel
 // ptxas spilled); whichever the plan did not choose returns at once, which costs a
 // small grid 3.7 us a launch, so these two share one.  Two CTAs of 128 threads per SM
 // (8 warps, as many as 255 registers allow).
-template <bool CFL, bool EXT, bool FIELD>
+template <bool CFL, bool EXT, int FORM>
 __global__ void __launch_bounds__(128, 2) substep_fx_fallback_kernel(const SubstepArgs<double, double> a,
                                                                      const FxPtrs fx, FxCoefs fc,
                                                                      const FxPlan *plan) {
+    using IX = typename FxIndex<FORM>::type;
     const int kern = plan->kern;
     if (kern == FX_GROUP) return;
-    if (!FIELD || kern == FX_PLAIN) {
+    if (FORM == FX_UNEQUAL || kern == FX_PLAIN) {
         substep_body<double, double, IdxPeriodic32, CFL, 3, EXT>(a);
         return;
     }
@@ -1340,7 +1411,23 @@ __global__ void __launch_bounds__(128, 2) substep_fx_fallback_kernel(const Subst
     __shared__ double etab[512];
     exp_tab_stage(etab);
     double cfl = 0.0;
-    if (active) fx_field_column<CFL, EXT>(a, fx, fc, plan, etab, i, j, cfl);
+    if (active) fx_column<true, IX, CFL, EXT>(a, fx, fc, plan, etab, i, j, cfl);
+    if (CFL) block_max_to_global(cfl, a.cfl_max);
+}
+
+// The columns' FX_GROUP, for boxes too thin for the 16 x 16 tiles (fx_form).
+template <bool CFL, bool EXT>
+__global__ void __launch_bounds__(128, 2) substep_fx_column_kernel(const SubstepArgs<double, double> a,
+                                                                   const FxPtrs fx, FxCoefs fc,
+                                                                   const FxPlan *plan) {
+    if (plan->kern != FX_GROUP) return;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int j = blockIdx.y * blockDim.y + threadIdx.y;
+    const bool active = i < a.g.nx && j < a.g.ny;
+    __shared__ double etab[512];
+    exp_tab_stage(etab);
+    double cfl = 0.0;
+    if (active) fx_column<false, IdxPeriodic32, CFL, EXT>(a, fx, fc, plan, etab, i, j, cfl);
     if (CFL) block_max_to_global(cfl, a.cfl_max);
 }
 
