@@ -61,6 +61,13 @@ FX_TRAFFIC_PER_CELL = {"group": (452677120 + 229116288) / 2097152,
 # sm__inst_executed_pipe_fp64 x 32 / cells, 128^3 forced; the instruction stream
 # does not depend on the grid), per form: substep-0 (CFL) and substep-1/2 variants.
 FX_FP64_PIPE_INST_PER_CELL = {"group": (59.6774, 58.3281), "field": (236.3125, 209.3125)}
+def products_share(forms):
+    """Share of the substeps, counted as by ac_get_stencil_forms, that ran integer products,
+    the others per-field scales; None if none ran or any ran another form."""
+    products, group, field, plain = forms
+    return products / (products + field) if products + field and not group + plain else None
+
+
 # DRAM bytes per cell of one launch of the binary32 tiled substep, the mean over
 # substeps 0, 1, 2 (ncu, 256^3 forced, one step: 1970.1 MB read + written per
 # launch on average over 16,777,216 cells; algorithmic 96, 128, 128 B/cell)
@@ -502,7 +509,7 @@ def run_ours(args, wl):
     evs = [[[torch.cuda.Event(enable_timing=True) for _ in range(2)] for _ in range(3)]
            for _ in range(args.steps)]
     launches0 = ac.ac_launch_count(sim.h)
-    modes0 = ac.ac_get_stencil_modes(sim.h)
+    modes0, forms0 = ac.ac_get_stencil_modes(sim.h), ac.ac_get_stencil_forms(sim.h)
     # CUDA events around the substep kernel itself (and its preparation kernels),
     # recorded by the library on its stream over the timed region
     ac.ac_set_kernel_timing(sim.h, True)
@@ -535,6 +542,7 @@ def run_ours(args, wl):
     kern = {s: kern_ms[s] / 1e3 for s in range(3)}
     avg_all = statistics.mean(kern.values())
     modes = [m1 - m0 for m0, m1 in zip(modes0, ac.ac_get_stencil_modes(sim.h))]
+    forms = [m1 - m0 for m0, m1 in zip(forms0, ac.ac_get_stencil_forms(sim.h))]
     if wl["precision"] == "fp64":
         flops = {s: flops_per_cell(order, s) * ncell for s in range(3)}
         equiv = statistics.mean(flops[s] / kern[s] for s in range(3)) / 1e12
@@ -543,15 +551,12 @@ def run_ours(args, wl):
         # measured denominator: the library's DFMA-chain probe (2 flops per FMA)
         dfma = ac.ac_diag_fma_rate(ac.AC_FP64, stream.cuda_stream)
         peak = 2 * dfma / 1e12
-        # the count per cell of the form the timed substeps ran (none for plain
-        # binary64 stencils, which this table does not cover).  A substep counted
-        # under field scales (components more than one binade apart) still runs the
-        # group form up to six binades, so the per-field counts, the larger ones, are
-        # taken only where every substep was counted so.
+        # the count per cell weighted by the forms that the timed substeps ran (none for
+        # a thin box's or plain stencils, which this table does not cover)
         inst = None
         traffic = None
-        if fixed and order == 6 and sum(modes) and not modes[2] and not wl.get("entropy"):
-            fg = 1.0 if modes[0] else 0.0
+        fg = products_share(forms)
+        if fixed and order == 6 and fg is not None and not wl.get("entropy"):
             G, F = FX_FP64_PIPE_INST_PER_CELL["group"], FX_FP64_PIPE_INST_PER_CELL["field"]
             inst = [fg * G[v] + (1 - fg) * F[v] for v in range(2)]
             traffic = (fg * FX_TRAFFIC_PER_CELL["group"] +
@@ -733,6 +738,9 @@ def run_ours(args, wl):
                 "gpu_launches": launches, "clocks": clocks,
                 "stencil_modes": ({"group_scales": modes[0], "field_scales": modes[1],
                                    "plain_binary64": modes[2]} if sum(modes) else None),
+                "stencil_forms": ({"integer_products": forms[0], "thin_box_scales": forms[1],
+                                   "field_scales": forms[2], "plain_binary64": forms[3]}
+                                  if sum(forms) else None),
                 "parity_sampled": parity, "fp32_vs_fp64": fp32_err,
                 "last_cfl_speed": cfl,
                 "substep_ms": {str(s): 1e3 * avg[s] for s in range(3)}}

@@ -217,7 +217,7 @@ int ac_get_stencil_order(const ac_handle *h, int *order);
  * on but for thin boxes, where the plain stencils are the faster, use them too, each
  * axis's numerators scaled to the smallest spacing, while the state lies in the ranges
  * of the form b = 56 below; ac_get_stencil_path and ac_get_stencil_modes do not count
- * that form.)  With
+ * that form, ac_get_stencil_forms does.)  With
  * integer sums every field is first written, on the device before each
  * substep, as int64 fixed point about its own offset: F = round((f - c)
  * 2^(b - E)), c the midpoint of the field's range and 2^E above its half-range
@@ -249,7 +249,7 @@ int ac_get_stencil_order(const ac_handle *h, int *order);
  * AC_STENCIL_FIXED returns the error.  The
  * kernel's waits for that copy are bounded: if one runs out, the state is undefined and
  * the next of ac_store, ac_store_w, ac_store_f32, ac_last_cfl, ac_reduce,
- * ac_get_stencil_modes and (where it has happened by then) substep 0 of a step returns
+ * ac_get_stencil_modes, ac_get_stencil_forms and (where it has happened by then) substep 0 of a step returns
  * AC_ERR_TIMEOUT, once.
  */
 #define AC_STENCIL_AUTO 0
@@ -267,6 +267,20 @@ int ac_get_stencil_path(const ac_handle *h, int *fixed);
 #define AC_STENCIL_MODE_FIELD 1
 #define AC_STENCIL_MODE_PLAIN 2
 int ac_get_stencil_modes(ac_handle *h, unsigned long long counts[3]);
+/*
+ * counts[m] = substeps of the integer-sum path, with any spacing, that ran in form m: which
+ * arithmetic the state and the box's shape led to (the modes above count by the state
+ * alone).  PRODUCTS: integer stencils and products on tiles (b = 56); GROUP: the thin
+ * boxes' common scales; FIELD: scales of their own, binary64 products; PLAIN: binary64
+ * stencils because of the state.  Substeps that ran plain stencils for another reason (the
+ * mode, the order, the layout, dt, the box) are in none.  Synchronises the handle's
+ * stream.
+ */
+#define AC_STENCIL_FORM_PRODUCTS 0
+#define AC_STENCIL_FORM_GROUP 1
+#define AC_STENCIL_FORM_FIELD 2
+#define AC_STENCIL_FORM_PLAIN 3
+int ac_get_stencil_forms(ac_handle *h, unsigned long long counts[4]);
 
 /* Substeps 0, 1, 2 with the same dt (one full Runge-Kutta step). */
 int ac_integrate_step(ac_handle *h, double dt);

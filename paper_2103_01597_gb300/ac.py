@@ -32,6 +32,7 @@ AC_LAYOUT_PERIODIC, AC_LAYOUT_PADDED = 0, 1
 AC_MAX, AC_MIN, AC_SUM, AC_RMS = 0, 1, 2, 3
 AC_STENCIL_AUTO, AC_STENCIL_FP64, AC_STENCIL_FIXED = 0, 1, 2
 AC_STENCIL_MODE_GROUP, AC_STENCIL_MODE_FIELD, AC_STENCIL_MODE_PLAIN = 0, 1, 2
+AC_STENCIL_FORM_PRODUCTS, AC_STENCIL_FORM_GROUP, AC_STENCIL_FORM_FIELD, AC_STENCIL_FORM_PLAIN = 0, 1, 2, 3
 AC_CONV_TCGEN05, AC_CONV_MMA_SYNC, AC_CONV_TCGEN05_PAIR = 0, 1, 2
 AC_TILE_32X8, AC_TILE_16X16 = 0, 1
 AC_Q_UMAG, AC_Q_EKIN, AC_Q_EMAG, AC_Q_CFL = 8, 9, 10, 11
@@ -105,6 +106,7 @@ def load_library(path=None):
         "ac_set_stencil_mode": ([_vp, _c.c_int], _c.c_int),
         "ac_get_stencil_path": ([_vp, ctypes.POINTER(_c.c_int)], _c.c_int),
         "ac_get_stencil_modes": ([_vp, ctypes.POINTER(_c.c_ulonglong)], _c.c_int),
+        "ac_get_stencil_forms": ([_vp, ctypes.POINTER(_c.c_ulonglong)], _c.c_int),
         "ac_diag_fma_rate": ([_c.c_int, _pd, _vp], _c.c_int),
         "ac_set_kernel_timing": ([_vp, _c.c_int], _c.c_int),
         "ac_kernel_timings": ([_vp, _pd, _pd, ctypes.POINTER(_c.c_int)], _c.c_int),
@@ -305,6 +307,15 @@ def ac_get_stencil_modes(h):
     plain binary64 stencils (AC_STENCIL_MODE_GROUP/FIELD/PLAIN), as a 3-tuple."""
     out = (ctypes.c_ulonglong * 3)()
     _check(_lib.ac_get_stencil_modes(h, out), "ac_get_stencil_modes")
+    return tuple(int(v) for v in out)
+
+
+def ac_get_stencil_forms(h):
+    """Substeps of the integer-sum path that ran as integer products on tiles, with a thin
+    box's common scales, with per-field scales and as plain binary64 stencils
+    (AC_STENCIL_FORM_PRODUCTS/GROUP/FIELD/PLAIN), as a 4-tuple."""
+    out = (ctypes.c_ulonglong * 4)()
+    _check(_lib.ac_get_stencil_forms(h, out), "ac_get_stencil_forms")
     return tuple(int(v) for v in out)
 
 

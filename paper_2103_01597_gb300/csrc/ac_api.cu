@@ -683,7 +683,15 @@ extern "C" int ac_get_stencil_modes(ac_handle *h, unsigned long long counts[3]) 
     if (!h || !counts) return AC_ERR_ARG;
     counts[0] = counts[1] = counts[2] = 0;
     if (!h->fx_plan) return AC_OK;
-    CK(fx_plan_taken(h->fx_plan, counts, h->stream));
+    CK(fx_plan_counts(h->fx_plan, false, counts, h->stream));
+    return timed_out(h);
+}
+
+extern "C" int ac_get_stencil_forms(ac_handle *h, unsigned long long counts[4]) {
+    if (!h || !counts) return AC_ERR_ARG;
+    for (int i = 0; i < 4; ++i) counts[i] = 0;
+    if (!h->fx_plan) return AC_OK;
+    CK(fx_plan_counts(h->fx_plan, true, counts, h->stream));
     return timed_out(h);
 }
 

@@ -128,7 +128,7 @@ size_t fx_copy_bytes(const Geom &g, int form);
 cudaError_t fx_encode_map(void *base, const Geom &g, CUtensorMap *map);
 // Substeps run in each mode (group scales, per-field scales, plain binary64)
 // since the plan was zeroed; synchronises `st`.
-cudaError_t fx_plan_taken(const void *plan, unsigned long long taken[3], cudaStream_t st);
+cudaError_t fx_plan_counts(const void *plan, bool ran, unsigned long long *counts, cudaStream_t st);
 
 cudaError_t launch_substep(const SubstepLaunch &L, cudaStream_t st, int *launches);
 cudaError_t launch_halo(int precision, const Geom &g, void *const f[NF], cudaStream_t st);

@@ -234,10 +234,11 @@ cudaError_t launch_substep_f64(const SubstepLaunch &L, cudaStream_t st, int *lau
 // Size of the device plan of the integer-sum path (allocated by the handle).
 size_t fx_plan_bytes() { return sizeof(FxPlan); }
 
-// Substeps run in each mode of the integer-sum path, read from a plan.
-cudaError_t fx_plan_taken(const void *plan, unsigned long long taken[3], cudaStream_t st) {
+// Substeps counted in each mode, or (ran) that each form ran, read from a plan.
+cudaError_t fx_plan_counts(const void *plan, bool ran, unsigned long long *counts, cudaStream_t st) {
     const FxPlan *p = static_cast<const FxPlan *>(plan);
-    cudaError_t e = cudaMemcpyAsync(taken, p->taken, 3 * sizeof(unsigned long long),
+    cudaError_t e = cudaMemcpyAsync(counts, ran ? p->ran : p->taken,
+                                    (ran ? 4 : 3) * sizeof(unsigned long long),
                                     cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     return e;

@@ -105,6 +105,7 @@ struct FxPlan {
     int s[NF];                 // F = round((f - c) 2^s), s = b - E
     unsigned long long C[NF];  // round(c 2^s) modulo 2^64
     unsigned long long taken[3];  // substeps counted in each mode (cumulative)
+    unsigned long long ran[4];    // substeps that each form ran (AC_STENCIL_FORM_*, cumulative)
 };
 
 // One warp: lane q < NF plans field q (offset, exponent), then the lanes agree
@@ -175,6 +176,9 @@ __device__ __forceinline__ void fx_plan(unsigned long long *stats, FxPlan *plan,
     }
     if (q == 0) {
         plan->kern = kern;
+        plan->ran[kern == FX_PLAIN   ? AC_STENCIL_FORM_PLAIN
+                  : kern == FX_FIELD ? AC_STENCIL_FORM_FIELD
+                  : form == FX_COLUMNS ? AC_STENCIL_FORM_GROUP : AC_STENCIL_FORM_PRODUCTS] += 1ull;
         if (form != FX_UNEQUAL) plan->taken[mode] += 1ull;
     }
 }
