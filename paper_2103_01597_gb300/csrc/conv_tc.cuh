@@ -697,9 +697,11 @@ __global__ void __launch_bounds__(CTHREADS, 1)
         // EPI_MASK_BF16: the bias gradient, the sums over cells of what is written.  A
         // thread adds its cell's COUT channels in binary32 for BTILES tiles, then the
         // warp adds its lanes in a tree, after which lane c holds channel c and goes on
-        // in binary64.  (As a kernel of its own that read the 134 MB of a 128^3 layer
+        // in binary64: eight binary32 additions one upon the other, as few as any sum of
+        // the output layer's kernel has (three tiles or sixteen: 948 us a training step
+        // at 128^3 either way).  (As a kernel of its own that read the 134 MB of a 128^3 layer
         // back: 41 us; here the layer takes as long as without.)
-        constexpr int BTILES = 16;
+        constexpr int BTILES = 3;
         constexpr int BS = EPI == EPI_MASK_BF16 ? COUT : 1;
         static_assert(EPI != EPI_MASK_BF16 || COUT == 32, "a channel per lane");
         float bs[BS];
