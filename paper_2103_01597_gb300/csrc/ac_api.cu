@@ -124,12 +124,8 @@ int ac::valid_params(const ac_params *p) {
 }
 
 cudaError_t ac::zero_now(void *p, size_t bytes) {
-    cudaStream_t st = nullptr;
-    cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(p, 0, bytes, st);
-    const cudaError_t s = cudaStreamSynchronize(st), d = cudaStreamDestroy(st);
-    return e != cudaSuccess ? e : (s != cudaSuccess ? s : d);
+    const cudaError_t e = cudaMemsetAsync(p, 0, bytes, cudaStreamPerThread);
+    return e != cudaSuccess ? e : cudaStreamSynchronize(cudaStreamPerThread);
 }
 
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }

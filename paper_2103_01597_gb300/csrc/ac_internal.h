@@ -161,9 +161,9 @@ struct ReduceLaunch {
     int blocks;
 };
 int reduce_max_blocks();
-// Zeroes new device memory before it returns, behind no other stream's work: what a
-// kernel on any stream relies on later (a memset on the default stream would be ordered
-// with neither a non-blocking stream nor the host).
+// Zeroes new device memory before it returns: what a kernel on any stream relies on later
+// (a memset on the default stream alone would be ordered with neither a non-blocking
+// stream nor the host).  On the thread's own stream: one made for it took 50 us.
 cudaError_t zero_now(void *p, size_t bytes);
 cudaError_t launch_reduce(const ReduceLaunch &L, cudaStream_t st, int *launches);
 
