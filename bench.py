@@ -52,15 +52,15 @@ def bytes_per_cell(elem_f, elem_w, s):
 # Nominal dense FP64 rate of one GB300 (no measured FP64 peak is provided).
 FP64_NOMINAL_TFLOPS = 1.25
 # DRAM bytes per cell of one launch of the integer FP64 substep kernel (ncu, 128^3,
-# substep-1/2 variant, over 2,097,152 cells): group scales (forced state) 452.7 MB
-# read + 229.1 MB written; the per-field form of the fallback kernel (u_z scaled by
+# substep-1/2 variant, over 2,097,152 cells): integer products (forced state) 452.5 MB
+# read + 225.1 MB written; the per-field form of the fallback kernel (u_z scaled by
 # 1e-3) 429.3 + 236.7 MB.
-FX_TRAFFIC_PER_CELL = {"group": (452677120 + 229116288) / 2097152,
+FX_TRAFFIC_PER_CELL = {"group": (452491904 + 225127680) / 2097152,
                        "field": (429260800 + 236704256) / 2097152}
 # FP64-pipe thread instructions per cell of that kernel (ncu
 # sm__inst_executed_pipe_fp64 x 32 / cells, 128^3 forced; the instruction stream
 # does not depend on the grid), per form: substep-0 (CFL) and substep-1/2 variants.
-FX_FP64_PIPE_INST_PER_CELL = {"group": (59.6774, 58.3281), "field": (236.3125, 209.3125)}
+FX_FP64_PIPE_INST_PER_CELL = {"group": (63.4942, 62.2734), "field": (236.3125, 209.3125)}
 def products_share(forms):
     """Share of the substeps, counted as by ac_get_stencil_forms, that ran integer products,
     the others per-field scales; None if none ran or any ran another form."""

@@ -273,12 +273,13 @@ cudaError_t launch_gather_f32(const void *src, int elem_size, const Geom &g, int
 // reduce_cells_kernel, bound by memory.  E_M sums and, in binary32, the CFL speed go
 // through reduce_curl_kernel, whose threads march along z (the periodic offsets of x and
 // y are set once).  In binary64 an FP64-pipe instruction costs a warp about 78 cycles, so
-// the six derivatives of the curl are taken in integers there (fx_arith.cuh).  The largest CFL speed (reduce_cfl_max_kernel) is searched with a
-// binary32 upper bound, exact binary64 speeds only where it exceeds the largest known.
+// the six derivatives of the curl are taken in integers there (fx_arith.cuh).  The
+// largest CFL speed (reduce_cfl_max_kernel) is searched with a binary32 upper bound, exact
+// binary64 speeds only where it exceeds the largest known.
 // The rest (max and min of E_K and E_M, other orders, CFL sums) takes the general kernel.
-// Measured at 256^3 in binary64, host time of one call each: E_K 245 us, E_M 883, rms |u|
-// 147, the CFL speed 1187, min ln rho 58, together 2530 (6470 all through the general
-// kernel).
+// Measured at 256^3 in binary64, host time of one call each: E_K 245 us, E_M 930 (883 with
+// one scale for all 36 values, which lost bits to uniform parts of A), rms |u| 145, the
+// CFL speed 1196, min ln rho 58, together 2580 (6470 all through the general kernel).
 // ---------------------------------------------------------------------------
 constexpr int RED_THREADS = 256;
 constexpr int RED_MAX_BLOCKS = 8 * 152;  // eight 256-thread CTAs per SM

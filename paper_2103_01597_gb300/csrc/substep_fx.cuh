@@ -17,15 +17,17 @@
 //    numerators are exact integers, the products of the right-hand side (u . grad,
 //    S . grad ln rho, S : S, j x B, j^2, u x B) exact integer dot products
 //    (fx_arith.cuh), the exponentials fixed point; what remains on the FP64 pipe
-//    is one multiply-add per term of Eqs. B.1-B.4 and the Runge-Kutta update (58
-//    instructions per cell).
+//    is a multiply-add or two per term of Eqs. B.1-B.4 and the Runge-Kutta update (62
+//    instructions per cell).  Thin boxes (fx_form) go column by column over copies
+//    without a halo instead, with b = 50, one binade of slack and binary64 products.
 //  * FX_FIELD (b = 50): some component lies further below its group's largest, so
 //    every field keeps its own scale; integer numerators are converted one by one
 //    and the sums across components (curl A, grad(div u), grad(div A)) and the
 //    products run in binary64 -- a component far smaller than the others (a
 //    near-2-D flow, a weak field component) is resolved to 2^-50 of its own range.
 //    States beyond the ranges FX_GROUP is sized for take it too: exponents
-//    outside +-200, a mean flow 2^4 times its range, |ln rho| or |xi| over 64.
+//    outside +-200, a mean flow 2^4 times its range, a uniform component of u far below
+//    the others, |ln rho| or |xi| over 64 (with unequal spacing FX_PLAIN takes them).
 //  * FX_PLAIN: a NaN or infinity in the state, or a range outside
 //    [2^-960, 2^960): the substep runs plain binary64 stencils, exactly what
 //    AC_STENCIL_FP64 computes (so a non-finite value propagates as in the
@@ -715,8 +717,9 @@ template <> struct FxIndex<FX_COLUMNS> { using type = IdxPeriodic32; };
 // the FP64 pipe, 179 instructions a cell); these integer products with stencil points
 // loaded through L1 5.95 (load latency at 2 warps per scheduler); one thread per cell
 // on the ring 3.72; two threads in lockstep between CTA barriers 4.11; without CTA
-// barriers (FxMarch) 3.40; with the halves balanced 3.18, 3.22 since conversions take every size.  Bound now by the issue of
-// its 3900 instructions a cell (about half the issue slots; ALU 48%, FP64 pipe 55%).
+// barriers (FxMarch) 3.40; with the halves balanced 3.18, and 3.29 since conversions take
+// every size and the pressure's gradients a scale each.  Bound now by the issue of its
+// 4270 instructions a cell (about half the issue slots; ALU 48%, FP64 pipe 55%).
 constexpr int FXT = 16;                            // tile edge
 constexpr int FXR = FXT + 2 * R;                   // staged row
 constexpr int FX_FIELD_TILE = FXR * FXR;           // cells of one staged field plane
